@@ -21,24 +21,37 @@ ROOT = os.path.dirname(HERE)
 SRC = os.path.join(HERE, "gv_cpu.cpp")
 SO = os.path.join(HERE, "_gv_cpu.so")
 CSRC = os.path.join(ROOT, "paper_1512_06637_gb300", "csrc")
+RANK_SRC = os.path.join(HERE, "gv_rank_cpu.cpp")
+RANK_SO = os.path.join(HERE, "_gv_rank_cpu.so")
 DEPS = [SRC, os.path.join(HERE, "shim", "cuda_runtime.h"), os.path.join(HERE, "shim", "math_constants.h"),
         os.path.join(CSRC, "solid_fp64.cuh"), os.path.join(CSRC, "desc_build.h"), os.path.join(CSRC, "gv_desc.h"),
         os.path.join(ROOT, "include", "gv.h")]
+RANK_DEPS = [RANK_SRC, os.path.join(CSRC, "rank_fp64.cuh"), os.path.join(CSRC, "solid_fp32.cuh")] + DEPS
 KINDS = {"box": 0, "trd": 1, "trap": 2, "tube": 3, "cone": 4, "polycone": 5}
 _lock = threading.Lock()
 _lib = None
 
 
+def _compile(src: str, so: str, deps: list, force: bool = False) -> str:
+    if not force and os.path.exists(so) and os.path.getmtime(so) >= max(os.path.getmtime(d) for d in deps):
+        return so
+    tmp = so + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O3", "-std=c++17", "-fopenmp", "-ffp-contract=off", "-fno-fast-math", "-fPIC", "-shared",
+           "-I", os.path.join(HERE, "shim"), "-I", os.path.join(ROOT, "include"), "-I", CSRC, src, "-o", tmp]
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, so)
+    return so
+
+
 def build(force: bool = False) -> str:
     """Compile ``_gv_cpu.so`` with g++ (no GPU needed)."""
-    if not force and os.path.exists(SO) and os.path.getmtime(SO) >= max(os.path.getmtime(d) for d in DEPS):
-        return SO
-    tmp = SO + f".tmp{os.getpid()}"
-    cmd = ["g++", "-O3", "-std=c++17", "-fopenmp", "-ffp-contract=off", "-fno-fast-math", "-fPIC", "-shared",
-           "-I", os.path.join(HERE, "shim"), "-I", os.path.join(ROOT, "include"), "-I", CSRC, SRC, "-o", tmp]
-    subprocess.run(cmd, check=True)
-    os.replace(tmp, SO)
-    return SO
+    return _compile(SRC, SO, DEPS, force)
+
+
+def load_ranked():
+    """The library's ranked binary64 evaluation compiled for the host (for tests)."""
+    with _lock:
+        return ctypes.CDLL(_compile(RANK_SRC, RANK_SO, RANK_DEPS))
 
 
 def _load():

@@ -1,0 +1,49 @@
+// gv_rank_cpu.cpp -- the library's ranked binary64 evaluation (rank_fp64.cuh) compiled for the
+// host, for tests that compare it with the whole binary64 evaluation (gv_cpu.cpp) without a GPU.
+#include <cuda_runtime.h>  // the host stand-ins (shim/)
+#include "rank_fp64.cuh"
+
+using namespace gv;
+
+template <int FAMILY>
+static bool one(const Desc& S, const uint2* const p[6], int64_t i, bool dirs, const f64::Track& T, unsigned want,
+                f64::Result& R) {
+  const f32::TrackF F = f32::load_track<(FAMILY >= 2)>(p[0], p[1], p[2], p[3], p[4], p[5], i, dirs);
+  f32::R32 r;
+  f64::rank32<FAMILY>(S, F, want, r);
+  if (r.flag) return false;
+  f64::query_ranked<FAMILY>(S, T, f64::Verdict{r.rank}, R);
+  return true;
+}
+
+// The requested results of n tracks against a descriptor of gvcpu_build; ranked[i] tells whether
+// track i had a certain verdict (its results are left alone if not).
+extern "C" void gvcpu_query_ranked(const void* desc, int64_t n, const double* const* t, unsigned want, int8_t* ranked,
+                                   int8_t* inside, double* din, double* dout, double* sin, double* sout) {
+  Desc S;
+  std::memcpy(&S, desc, sizeof(Desc));
+  const uint2* p[6];
+  for (int c = 0; c < 6; c++) p[c] = reinterpret_cast<const uint2*>(t[c]);
+  const bool dirs = want & (f64::kWantDin | f64::kWantDout);
+#pragma omp parallel for schedule(static, 4096)
+  for (int64_t i = 0; i < n; i++) {
+    f64::Track T{t[0][i], t[1][i], t[2][i], 0, 0, 0};
+    if (dirs) { T.u = t[3][i]; T.v = t[4][i]; T.w = t[5][i]; }
+    f64::Result R;
+    bool ok = false;
+    if (!(S.flags & kFp64Only)) switch (S.type) {
+      case kBox: ok = one<0>(S, p, i, dirs, T, want, R); break;
+      case kTrd:
+      case kTrap: ok = one<1>(S, p, i, dirs, T, want, R); break;
+      case kTube: ok = one<2>(S, p, i, dirs, T, want, R); break;
+      default: ok = one<3>(S, p, i, dirs, T, want, R); break;
+    }
+    ranked[i] = ok;
+    if (!ok) continue;
+    inside[i] = (int8_t)R.code;
+    din[i] = R.din;
+    dout[i] = R.dout;
+    sin[i] = R.sin;
+    sout[i] = R.sout;
+  }
+}

@@ -20,3 +20,26 @@ using std::copysign;
 using std::fabs;
 using std::nan;
 using std::sqrt;
+
+// Stand-ins for what the binary32 passes (solid_fp32.cuh) use.  Reciprocal, division and
+// reciprocal square root are correctly rounded here; the device's approximate ones lie within
+// the passes' error bounds.
+#include <cstring>
+using std::fmaf;
+using std::isfinite;
+using std::isinf;
+struct uint2 { uint32_t x, y; };
+static inline uint2 make_uint2(uint32_t x, uint32_t y) { return {x, y}; }
+template <class T> static inline T __ldg(const T* p) { return *p; }
+template <class To, class From> static inline To shim_bits(From v) {
+  To r;
+  std::memcpy(&r, &v, sizeof(r));
+  return r;
+}
+static inline float __uint_as_float(uint32_t v) { return shim_bits<float>(v); }
+static inline uint32_t __float_as_uint(float v) { return shim_bits<uint32_t>(v); }
+static inline long long __double_as_longlong(double v) { return shim_bits<long long>(v); }
+static inline float __frcp_rn(float v) { return 1.0f / v; }
+static inline float __fdividef(float a, float b) { return a / b; }
+static inline float rsqrtf(float v) { return 1.0f / std::sqrt(v); }
+static inline int __ffs(uint32_t v) { return __builtin_ffs((int)v); }

@@ -1,13 +1,14 @@
-// query_fp64.cu -- the plain binary64 query pass: one thread per track, the solid
-// descriptor staged in shared memory.  A basket of a primitive solid large enough to give every
-// SM a 2048-track tile is evaluated in tiles ordered by work class (k_query_fp64_tiles): the pass is bound
-// by the FP64 pipe, which spends the same on a warp instruction whatever its active lanes, so
-// warps of one class (inside, outside and entering, outside and missing, near a surface) run
-// fewer instructions for the same tracks.  Smaller baskets and booleans go in index order,
-// grid-stride over the basket (k_query_fp64).  Per track the arithmetic is the same either way.
+// query_fp64.cu -- the plain binary64 query pass.  Primitive solids take the ranked pass
+// (k_query_rank64): binary32 decides which constraint and which crossing give the results, binary64
+// evaluates those.  What has no binary32 form is evaluated whole, one thread per track: booleans in
+// index order (k_query_fp64); solids with features finer than binary32 resolves in tiles ordered by
+// work class when the basket gives every SM a 2048-track tile (k_query_fp64_tiles: the FP64 pipe
+// spends the same on a warp instruction whatever its active lanes, so warps of one class run fewer
+// instructions), else in index order.  Per track the bits are the same in every one of them.
 #include "gv_debug.cuh"
 #include "gv_internal.h"
 #include "solid_fp64.cuh"
+#include "rank_fp64.cuh"
 #include "work_class.cuh"
 
 namespace gv {
@@ -120,6 +121,137 @@ __global__ void __launch_bounds__(256) k_query_fp64_tiles(const Desc* __restrict
   }
 }
 
+template <int FAMILY>
+static __device__ __noinline__ void query_whole(const Desc& S, const QueryArgs& a, int64_t i, unsigned want) {
+  f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
+  if (want & (f64::kWantDin | f64::kWantDout)) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+  f64::Result R;
+  if (FAMILY == 0) f64::box_query(S, T, want, R);
+  else if (FAMILY == 1) f64::planar_query(S, T, want, R);
+  else f64::pcon_query(S, T, want, R);
+  if (a.inside) a.inside[i] = (int8_t)R.code;
+  if (a.din) a.din[i] = R.din;
+  if (a.dout) a.dout[i] = R.dout;
+  if (a.sin) a.sin[i] = R.sin;
+  if (a.sout) a.sout[i] = R.sout;
+}
+
+// The ranked binary64 pass (rank_fp64.cuh) in tiles of 256 * ITEMS consecutive tracks: a block
+// ranks its tile's tracks in binary32 (one verdict word per track in shared memory), orders them by
+// the binary64 work their verdict asks for, and evaluates that work in this order, so that the FP64
+// pipe sees full warps.  While one resident block evaluates, others rank: the two halves use
+// different pipes.  A track without a certain verdict goes on the block's list, which is evaluated
+// whole when 256 have gathered and at the end.
+// Measured (GB300, all five queries): cone, 2^20 tracks, 500 -> 180 us; 8-plane polycone, 4 M tracks,
+// 6876 -> 1274 us; tube DistanceToOut, 50021 tracks, 44.6 -> 24.3 us (before: every candidate in
+// binary64, tiles ordered by class).  FP64 warp instructions per 32 tracks: cone 226 -> 42, polycone
+// 859 -> 45; issue 41-45% and FP64 23-46% busy: bound by latency at 24 warps per SM.  Three blocks of
+// 256 threads (80 registers) against two (128): 1274 against 1389 us (polycone).
+constexpr int kWholeFlush = 256;
+template <int FAMILY, int ITEMS>
+__global__ void __launch_bounds__(256, 3) k_query_rank64(const Desc* __restrict__ desc, QueryArgs a) {
+  constexpr int NT = 256, TILE = NT * ITEMS;
+  constexpr uint32_t NC = f64::kRankClasses;
+  __shared__ Desc S;
+  __shared__ uint32_t ver[TILE];
+  __shared__ uint16_t ord[TILE];
+  __shared__ int64_t whole[TILE + kWholeFlush];
+  __shared__ unsigned cnt[NC], nwhole;
+  stage_desc(S, desc);
+  const int tid = threadIdx.x;
+  const unsigned lane = tid & 31u;
+  if (tid == 0) nwhole = 0u;
+  const unsigned want = (a.inside ? f64::kWantCode : 0u) | (a.din ? f64::kWantDin : 0u) |
+                        (a.dout ? f64::kWantDout : 0u) | (a.sin ? f64::kWantSin : 0u) |
+                        (a.sout ? f64::kWantSout : 0u);
+  const bool dirs = want & (f64::kWantDin | f64::kWantDout);
+  const uint2 *X = reinterpret_cast<const uint2*>(a.x), *Y = reinterpret_cast<const uint2*>(a.y),
+              *Z = reinterpret_cast<const uint2*>(a.z), *Ux = reinterpret_cast<const uint2*>(a.u),
+              *Uy = reinterpret_cast<const uint2*>(a.v), *Uz = reinterpret_cast<const uint2*>(a.w);
+  for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {
+    const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
+    if (tid < (int)NC) cnt[tid] = 0u;
+    __syncthreads();
+    for (int j = tid; j < len; j += NT) {
+      const int64_t i = t0 + j;
+      const f32::TrackF T = f32::load_track<(FAMILY >= 2)>(X, Y, Z, Ux, Uy, Uz, i, dirs);
+      GV_DCHECK(!dirs || dbg_unit(a.u[i], a.v[i], a.w[i]), kDbgDirection, i);
+      f32::R32 R;
+      f64::rank32<FAMILY>(S, T, want, R);
+      if (R.flag) {
+        ver[j] = 0xFFFFFFFFu;
+        whole[atomicAdd(&nwhole, 1u)] = i;
+      } else {
+        ver[j] = R.rank;
+        atomicAdd(&cnt[f64::rank_class<FAMILY>(f64::Verdict{R.rank})], 1u);
+      }
+    }
+    __syncthreads();
+    const unsigned gathered = nwhole;
+    unsigned ranked = 0;
+    if (tid < 32) {  // exclusive sums of the class counts
+      const unsigned c = lane < NC ? cnt[lane] : 0u;
+      unsigned run = c;
+      for (int o = 1; o < 8; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, run, o);
+        if ((int)lane >= o) run += v;
+      }
+      __syncwarp();
+      if (lane < NC) cnt[lane] = run - c;
+    }
+    __syncthreads();
+    for (int j = tid; j < len; j += NT)
+      if (ver[j] != 0xFFFFFFFFu) ord[atomicAdd(&cnt[f64::rank_class<FAMILY>(f64::Verdict{ver[j]})], 1u)] = (uint16_t)j;
+    __syncthreads();
+    ranked = cnt[NC - 1];
+    for (unsigned p = tid; p < ranked; p += NT) {
+      const int j = ord[p];
+      const int64_t i = t0 + j;
+      f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
+      if (dirs) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+      f64::Result R;
+      f64::query_ranked<FAMILY>(S, T, f64::Verdict{ver[j]}, R);
+      if (a.inside) a.inside[i] = (int8_t)R.code;
+      if (a.din) a.din[i] = R.din;
+      if (a.dout) a.dout[i] = R.dout;
+      if (a.sin) a.sin[i] = R.sin;
+      if (a.sout) a.sout[i] = R.sout;
+    }
+    if (gathered >= (unsigned)kWholeFlush) {
+      for (unsigned q = tid; q < gathered; q += NT) query_whole<FAMILY>(S, a, whole[q], want);
+      __syncthreads();
+      if (tid == 0) nwhole = 0u;
+    }
+    __syncthreads();  // the tile's shared arrays are reused by the next tile
+  }
+  __syncthreads();
+  for (unsigned q = tid; q < nwhole; q += NT) query_whole<FAMILY>(S, a, whole[q], want);
+}
+
+template <int FAMILY, int ITEMS>
+static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaStream_t stream) {
+  static const int occ = [] {
+    int o = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_query_rank64<FAMILY, ITEMS>, 256, 0) != cudaSuccess || o < 1) {
+      cudaGetLastError();
+      o = 1;
+    }
+    return o;
+  }();
+  const int64_t tiles = (a.n + 256 * ITEMS - 1) / (256 * ITEMS);
+  const int64_t cap = (int64_t)sms * occ;
+  k_query_rank64<FAMILY, ITEMS><<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, stream>>>(s->d, a);
+}
+
+// Tiles of 2048 tracks when every resident block gets four of them, of 1024 when it gets one, else of
+// 256: a short basket is spread over every SM.
+template <int FAMILY>
+static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaStream_t stream) {
+  if (a.n >= (int64_t)sms * 3 * 4 * 2048) launch_rank64<FAMILY, 8>(s, a, sms, stream);
+  else if (a.n >= (int64_t)sms * 3 * 1024) launch_rank64<FAMILY, 4>(s, a, sms, stream);
+  else launch_rank64<FAMILY, 1>(s, a, sms, stream);
+}
+
 template <int FAMILY, int ITEMS>
 static int64_t tiles_grid(int64_t tiles, int sms) {
   // resident blocks per SM of the kernel (queried once: it depends only on the kernel and the GPU)
@@ -138,6 +270,16 @@ cudaError_t launch_query_fp64(const gv_solid* s, const QueryArgs& a, cudaStream_
   if (a.n == 0) return cudaSuccess;
   const int threads = 256;
   const int sms = sm_count();
+  if (s->h.type != kBool && !(s->h.flags & kFp64Only)) {
+    switch (s->h.type) {
+      case kBox: launch_rank64<0>(s, a, sms, stream); break;
+      case kTrd:
+      case kTrap: launch_rank64<1>(s, a, sms, stream); break;
+      case kTube: launch_rank64<2>(s, a, sms, stream); break;
+      default: launch_rank64<3>(s, a, sms, stream); break;
+    }
+    return cudaGetLastError();
+  }
   // tiles of 2048 tracks when the basket gives four of them to every resident block (two per SM),
   // else of 1024 (more tiles, fewer SMs idle in the last round); none below one 2048 tile per SM
   if (s->h.type != kBool && a.n >= (int64_t)sms * 2048) {

@@ -56,7 +56,24 @@ struct R32 {
   int code;
   float din, dout, sin, sout;
   bool flag;
+  uint32_t rank;  // RANK passes: the verdict for the binary64 evaluation (Verdict)
 };
+
+// The RANK instances of the passes decide, with the same certified arithmetic, which constraint
+// gives the safety and which crossing gives the distance; the binary64 value of that one quantity
+// is then the value of the whole binary64 evaluation (rank_fp64.cuh).  A verdict packs
+//   bits 0-1   code
+//   bits 3-5   constraint that gives the safety (kWhole: the largest of the piece's constraints)
+//   bits 6-10  its section (polycone family)
+//   bits 11-13 crossing that gives the distance (kNone: DistanceToIn +inf, DistanceToOut 0)
+//   bits 14-18 its section, or z-plane index
+//   bit 19     the distance sought is DistanceToOut (else DistanceToIn)
+// Box: constraint and crossing 1-3, the axis; trd/trap: 1-4 the side plane, 5 the z slab;
+// polycone family: the names below.  A track whose verdict is not certain has R32::flag set.
+enum : uint32_t { kNone = 0, kOuter = 1, kInner = 2, kZLow = 3, kZHigh = 4, kPhiS = 5, kPhiE = 6, kWhole = 7 };
+constexpr uint32_t kVerGoalOut = 1u << 19;
+__device__ __forceinline__ uint32_t ver_safety(uint32_t kind, int k) { return kind << 3 | (uint32_t)k << 6; }
+__device__ __forceinline__ uint32_t ver_dist(uint32_t kind, int k) { return kind << 11 | (uint32_t)k << 14; }
 
 struct Val {  // value with an absolute error bound
   float v, e;
@@ -188,6 +205,23 @@ struct SInt {
   __device__ __forceinline__ float err() const { return fmaxf(s - lo, hi - s); }
 };
 __device__ __forceinline__ SInt sint() { return {-F_INF, -F_INF, -F_INF}; }
+
+// Which of several values is the largest (smallest, with sign = -1), when that is certain: `id`
+// of the best and the nearest bound of the others.
+struct Arg {
+  float v, e, other;
+  uint32_t id;
+  __device__ __forceinline__ void add(float g, float E, uint32_t k) {
+    if (g > v) {
+      other = fmaxf(other, v + e);
+      v = g; e = E; id = k;
+    } else {
+      other = fmaxf(other, g + E);
+    }
+  }
+  __device__ __forceinline__ bool sure() const { return other < v - e; }
+};
+__device__ __forceinline__ Arg arg_none() { return {-F_INF, 0.f, -F_INF, kNone}; }
 __device__ __forceinline__ int decide(const SInt& S, bool& flag) {
   if (S.lo > HF) return 2;
   if (S.hi < -HF) return 0;
@@ -227,7 +261,7 @@ __device__ __forceinline__ Gv plane_g(const float* nh, const float* nl, float ch
 // the near face the slab is entered at -b and left at -a, otherwise entered at a
 // and left at b.  DistanceToOut = min exit, DistanceToIn = max entry when it comes
 // before the min exit.
-template <bool FRAME = false>
+template <bool FRAME = false, bool RANK = false>
 __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   const float ph[3] = {T.xh, T.yh, T.zh}, pl[3] = {T.xl, T.yl, T.zl}, d[3] = {T.u, T.v, T.w};
   Gv g[3];
@@ -240,10 +274,16 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
   R.code = decide(si, R.flag);
   R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
   R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
-  if (R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
+  if (!RANK && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
+  if (RANK) {
+    Arg m = arg_none();
+    for (int i = 0; i < 3; i++) m.add(g[i].g, g[i].E, i + 1);
+    R.rank = (uint32_t)R.code | ver_safety(R.code == 1 ? (uint32_t)kNone : m.sure() ? m.id : (uint32_t)kWhole, 0);
+  }
   if (!(want & (kWantDin | kWantDout))) return;
   Val tn{-BIG, 0.f}, tf{BIG, 0.f};
   bool miss = false, any_out = false, all_in = true;
+  Arg an = arg_none(), af = arg_none();  // RANK: the last entry, the first exit
   for (int i = 0; i < 3; i++) {
     const bool toward = (ph[i] < 0) == (d[i] < 0);  // toward the face on the point's side
     if (FRAME && fabsf(d[i]) <= 4.f * T.dfl) R.flag = true;  // sign of d not certain
@@ -258,8 +298,13 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
         A.e = fmaf(1.01f * fabsf(a) * T.dfl, inv, A.e);
         B.e = fmaf(fmaf(1.01f * b, T.dfl, T.fl), inv, B.e);
       }
-      tn = vmax(tn, toward ? Val{-B.v, B.e} : A);
-      tf = vmin(tf, toward ? Val{-A.v, A.e} : B);
+      const Val en = toward ? Val{-B.v, B.e} : A, ex = toward ? Val{-A.v, A.e} : B;
+      tn = vmax(tn, en);
+      tf = vmin(tf, ex);
+      if (RANK) {
+        an.add(en.v, en.e, i + 1);
+        af.add(-ex.v, ex.e, i + 1);
+      }
     }
     // surface start: constraints within the band
     if (g[i].g >= -HF) {
@@ -275,7 +320,7 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
     if (R.code == 2) R.dout = -1.f;
     else if (R.code == 1 && !all_in) R.dout = 0.f;
     else {
-      if (!certified(tf)) R.flag = true;
+      if (!RANK && !certified(tf)) R.flag = true;
       R.dout = unbig(tf.v);
       if (R.code == 1) {  // an entering surface point: inside (no tolerance) halfway to the exit?
         const float h = 0.5f * tf.v;
@@ -298,9 +343,22 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
     else {
       if (!apart(tn, tf) || fabsf(tf.v) <= tf.e) R.flag = true;
       if (tn.v < tf.v && tf.v > 0) {
-        if (!certified(tn)) R.flag = true;
+        if (!RANK && !certified(tn)) R.flag = true;
         R.din = tn.v;
       } else R.din = F_INF;
+    }
+  }
+  if (RANK) {
+    const bool out = R.code == 0 || (R.code == 1 && all_in);
+    if (out) {
+      R.rank |= kVerGoalOut;
+      if ((want & kWantDout) && !(R.code == 1 && R.dout == 0.f)) {
+        R.rank |= ver_dist(af.id, 0);
+        R.flag |= !af.sure() || af.id == kNone;
+      }
+    } else if ((want & kWantDin) && R.din < F_INF) {
+      R.rank |= ver_dist(an.id, 0);
+      R.flag |= !an.sure() || an.id == kNone;
     }
   }
 }
@@ -310,7 +368,7 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
 // One uniform path as for the box: every side plane gives one crossing
 // t = -g / (n.d), an entry when n.d < 0 and an exit when n.d > 0; the z slab
 // gives its two crossings like a box axis.
-template <bool FRAME = false>
+template <bool FRAME = false, bool RANK = false>
 __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   Gv g[5];
   float gd[5], egd[5];
@@ -329,10 +387,16 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
   R.code = decide(si, R.flag);
   R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
   R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
-  if (R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
+  if (!RANK && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
+  if (RANK) {
+    Arg m = arg_none();
+    for (int i = 0; i < 5; i++) m.add(g[i].g, g[i].E, i + 1);
+    R.rank = (uint32_t)R.code | ver_safety(R.code == 1 ? (uint32_t)kNone : m.sure() ? m.id : (uint32_t)kWhole, 0);
+  }
   if (!(want & (kWantDin | kWantDout))) return;
   Val tn{-BIG, 0.f}, tf{BIG, 0.f};
   bool miss = false, any_out = false, all_in = true;
+  Arg an = arg_none(), af = arg_none();  // RANK: the last entry, the first exit
   for (int i = 0; i < 4; i++) {
     // along or nearly along the face plane: sliding is decided in binary64
     if (fabsf(gd[i]) <= egd[i] + TAUF && fabsf(g[i].g) <= HF + g[i].E) R.flag = true;
@@ -347,6 +411,10 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
     const bool entry = gd[i] < 0;
     tn = vmax(tn, entry ? tv : Val{-BIG, 0.f});
     tf = vmin(tf, entry ? Val{BIG, 0.f} : tv);
+    if (RANK) {
+      if (entry) an.add(tv.v, tv.e, i + 1);
+      else af.add(-tv.v, tv.e, i + 1);
+    }
   }
   {  // z slab
     const bool toward = (T.zh < 0) == (T.w < 0);
@@ -363,8 +431,13 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
         A.e = fmaf(1.01f * fabsf(a) * T.dfl, iw, A.e);
         B.e = fmaf(fmaf(1.01f * b, T.dfl, T.fl), iw, B.e);
       }
-      tn = vmax(tn, toward ? Val{-B.v, B.e} : A);
-      tf = vmin(tf, toward ? Val{-A.v, A.e} : B);
+      const Val en = toward ? Val{-B.v, B.e} : A, ex = toward ? Val{-A.v, A.e} : B;
+      tn = vmax(tn, en);
+      tf = vmin(tf, ex);
+      if (RANK) {
+        an.add(en.v, en.e, 5);
+        af.add(-ex.v, ex.e, 5);
+      }
     }
   }
   for (int i = 0; i < 5; i++) {
@@ -379,7 +452,7 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
     if (R.code == 2) R.dout = -1.f;
     else if (R.code == 1 && !all_in) R.dout = 0.f;
     else {
-      if (!certified(tf)) R.flag = true;
+      if (!RANK && !certified(tf)) R.flag = true;
       R.dout = unbig(tf.v);
       if (R.code == 1) {  // an entering surface point: inside (no tolerance) halfway to the exit?
         const float h = 0.5f * tf.v;
@@ -404,9 +477,22 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
     else {
       if (!apart(tn, tf) || fabsf(tf.v) <= tf.e) R.flag = true;
       if (tn.v < tf.v && tf.v > 0) {
-        if (!certified(tn)) R.flag = true;
+        if (!RANK && !certified(tn)) R.flag = true;
         R.din = tn.v;
       } else R.din = F_INF;
+    }
+  }
+  if (RANK) {
+    const bool out = R.code == 0 || (R.code == 1 && all_in);
+    if (out) {
+      R.rank |= kVerGoalOut;
+      if ((want & kWantDout) && !(R.code == 1 && R.dout == 0.f)) {
+        R.rank |= ver_dist(af.id, 0);
+        R.flag |= !af.sure() || af.id == kNone;
+      }
+    } else if ((want & kWantDin) && R.din < F_INF) {
+      R.rank |= ver_dist(an.id, 0);
+      R.flag |= !an.sure() || an.id == kNone;
     }
   }
 }
@@ -485,7 +571,7 @@ __device__ __forceinline__ F2 df_norm(float h, float l) {
   return {s, l - (s - h)};
 }
 
-template <bool TUBE, bool FRAME>
+template <bool TUBE, bool FRAME, bool RANK = false>
 __device__ inline Quad quad32(float a, float al, const Lat& L, const TrackF& T, F2 rad, float erad, F2 A0,
                               float rh, float rl) {
   Quad q;
@@ -533,7 +619,8 @@ __device__ inline Quad quad32(float a, float al, const Lat& L, const TrackF& T, 
   const float eD = fmaf(2.f * fabsf(B), eB, fmaf(fabsf(A), eC, fmaf(fabsf(C), eA, fmaf(eB, eB,
                    fmaf(4.f * U * U, b2.h + fabsf(ac.h), fmaf(2.f * U, fabsf(disc), 1e-30f))))));
   if (disc < -eD) return q;
-  if (disc <= eD) { q.unsure = true; return q; }
+  // RANK: a crossing farther from a touch than the binary64 touch bound (far below eD)
+  if (disc <= (RANK ? 2.f * eD : eD)) { q.unsure = true; return q; }
   const float eB1 = fmaf(U, fabsf(B), eB), eA1 = fmaf(U, fabsf(A), eA), eC1 = fmaf(U, fabsf(C), eC);
   const float rs = rsqrtf(disc);
   const float sq = disc * rs;
@@ -643,10 +730,23 @@ struct Walk {
   Val tcur, ans;     // search/stretch position, answer
   float rh, rl, r2h, erad, iw;
   int k, step, st, guard;
+  uint32_t pid, did;  // RANK: phi planes behind PH and X2 (kPid*), the answer's crossing (ver_dist)
   bool zc, answered, u, goal_out, surf, need_in, need_out, in_range, live;
 };
 
-template <bool TUBE, bool FRAME = false>
+// RANK: which phi plane (E, else S) bounds the phi interval below and above, and whether the two
+// planes are too close to tell.
+enum : uint32_t { kPidLoE = 1, kPidLoTie = 2, kPidHiE = 4, kPidHiTie = 8 };
+__device__ __forceinline__ uint32_t phi_ids(const Iv& a, const Iv& b) {
+  uint32_t id = 0;
+  if (b.lo.v > a.lo.v) id |= kPidLoE;
+  if (a.lo.v > -BIG && b.lo.v > -BIG && !apart(a.lo, b.lo)) id |= kPidLoTie;
+  if (b.hi.v < a.hi.v) id |= kPidHiE;
+  if (a.hi.v < BIG && b.hi.v < BIG && !apart(a.hi, b.hi)) id |= kPidHiTie;
+  return id;
+}
+
+template <bool TUBE, bool FRAME = false, bool RANK = false>
 __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want, R32& R, Walk& W) {
   W.live = false;
   W.need_in = W.need_out = false;
@@ -709,32 +809,61 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   const float s = si.s;
   R.code = decide(si, R.flag);
   if (FRAME && near_plane) R.flag = true;
+  if (RANK) R.rank = (uint32_t)R.code;
 
   if (want & (kWantSin | kWantSout)) {
     R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
     R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
-    if (nz == 2 && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
+    if (!RANK && nz == 2 && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
+    // RANK: the constraint that gives a piece's value (the phi value's plane is certain or kWhole)
+    Gv ph{gphi, fmaxf(gphi - phlo, phhi - gphi)};
+    uint32_t phk = kWhole;
+    if (RANK && has_phi) {
+      if (fabsf(pa.g - pb.g) > pa.E + pb.E) phk = ((pa.g < pb.g) == wide) ? (uint32_t)kPhiS : (uint32_t)kPhiE;
+    }
+    if (RANK && nz == 2 && R.code != 1) {
+      Arg m = arg_none();
+      m.add(lo_.g, lo_.E, kOuter);
+      if (has_in) m.add(li_.g, li_.E, kInner);
+      m.add(gz0, Ez0, kZLow);
+      m.add(gz1, Ez1, kZHigh);
+      if (has_phi) m.add(ph.g, ph.E, phk);
+      R.rank |= ver_safety(m.sure() ? m.id : (uint32_t)kWhole, 0);
+    }
     if (nz > 2 && R.code != 1) {
       // sections as closed pieces (own z-planes included), each a max of constraints
-      auto closed_df = [&](int k) -> Val {
+      auto closed_df = [&](int k, uint32_t& kind) -> Val {
         SInt c = sint();
+        Arg m = arg_none();
         const Lat lo2 = k == k0 ? lo_ : lateral<TUBE>(S.oah[k], S.oal[k], S.obh[k], S.obl[k], S.ok_[k], rh, rl, T, true);
         c.add(lo2.g, lo2.E);
+        if (RANK) m.add(lo2.g, lo2.E, kOuter);
         if ((S.inner >> k) & 1u) {
           const Lat li2 = k == k0 ? li_ : lateral<TUBE>(S.iah[k], S.ial[k], S.ibh[k], S.ibl[k], S.ik_[k], rh, rl, T, false);
           c.add(li2.g, li2.E);
+          if (RANK) m.add(li2.g, li2.E, kInner);
         }
         const float gk0 = (S.zh[k] - T.zh) + (S.zl[k] - T.zl);
         const float gk1 = (T.zh - S.zh[k + 1]) + (T.zl - S.zl[k + 1]);
-        c.add(gk0, 4.f * U * fabsf(gk0) + G42 * (fabsf(T.zh) + fabsf(S.zh[k])) + T.fl);
-        c.add(gk1, 4.f * U * fabsf(gk1) + G42 * (fabsf(T.zh) + fabsf(S.zh[k + 1])) + T.fl);
+        const float Ek0 = 4.f * U * fabsf(gk0) + G42 * (fabsf(T.zh) + fabsf(S.zh[k])) + T.fl;
+        const float Ek1 = 4.f * U * fabsf(gk1) + G42 * (fabsf(T.zh) + fabsf(S.zh[k + 1])) + T.fl;
+        c.add(gk0, Ek0);
+        c.add(gk1, Ek1);
         if (has_phi) c.add_int(gphi, phlo, phhi);
+        if (RANK) {
+          m.add(gk0, Ek0, kZLow);
+          m.add(gk1, Ek1, kZHigh);
+          if (has_phi) m.add(ph.g, ph.E, phk);
+          kind = m.sure() ? m.id : (uint32_t)kWhole;
+        }
         return {c.s, c.err()};
       };
       if (R.code == 0) {  // SafetyToOut: the containing piece
-        const Val c = closed_df(k0);
+        uint32_t kind = kWhole;
+        const Val c = closed_df(k0, kind);
         R.sout = -c.v;
-        if (!certified({fabsf(c.v), c.e})) R.flag = true;
+        if (!RANK && !certified({fabsf(c.v), c.e})) R.flag = true;
+        if (RANK) R.rank |= ver_safety(kind, k0);
       } else {
         // SafetyToIn = min over pieces.  Plain binary32 values with their bounds give an
         // upper bound umin on the minimum; only pieces whose lower bound is below it can
@@ -785,13 +914,25 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
           if (!(v - e > umin)) cand |= 1u << k;
         }
         Val best{BIG, 0.f};
+        Arg m = arg_none();  // RANK: the smallest piece (two pieces bounded by the phi planes are equal)
+        uint32_t mkind = kNone;
         while (cand) {
           const int k = __ffs(cand) - 1;
           cand &= cand - 1u;
-          best = vmin(best, closed_df(k));
+          uint32_t kind = kWhole;
+          const Val c = closed_df(k, kind);
+          best = vmin(best, c);
+          if (RANK && !(mkind == kind && (kind == kPhiS || kind == kPhiE))) {
+            m.add(-c.v, c.e, (uint32_t)k);
+            if (m.id == (uint32_t)k) mkind = kind;
+          }
         }
         R.sin = best.v;
-        if (!certified(best)) R.flag = true;
+        if (!RANK && !certified(best)) R.flag = true;
+        if (RANK) {
+          R.flag |= !m.sure();
+          R.rank |= ver_safety(mkind, (int)m.id);
+        }
       }
     }
   }
@@ -878,6 +1019,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   if (R.code == 2 && (want & kWantDout)) R.dout = -1.f;
   W.need_out = (R.code == 0 || entering) && (want & kWantDout);
   W.need_in = (R.code == 2 || leaving) && (want & kWantDin);
+  if (RANK && (R.code == 0 || entering)) R.rank |= kVerGoalOut;
   if (!W.need_out && !W.need_in) return false;
 
   // Distances in interval form, over the sections the ray meets for t >= 0 in t order.
@@ -896,9 +1038,12 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   // one) counts as passed.  Inside and outside tracks run the same loop body.
   bool u = false;
   Iv PH = iv_all(), X2 = iv_none();
+  W.pid = 0u;
   if (has_phi) {
-    if (!wide) PH = iv_and(iv_half(pa.g, pa.E, nds, ends, true, u), iv_half(pb.g, pb.E, nde, ende, true, u));
-    else X2 = iv_and(iv_half(pa.g, pa.E, nds, ends, false, u), iv_half(pb.g, pb.E, nde, ende, false, u));
+    const Iv ha = iv_half(pa.g, pa.E, nds, ends, !wide, u), hb = iv_half(pb.g, pb.E, nde, ende, !wide, u);
+    if (RANK) W.pid = phi_ids(ha, hb);
+    if (!wide) PH = iv_and(ha, hb);
+    else X2 = iv_and(ha, hb);
     if (!X2.empty && !(X2.lo.v < X2.hi.v)) {  // no wedge along the ray, unless too close to tell
       if (!apart(X2.lo, X2.hi)) u = true;
       X2 = iv_none();
@@ -936,6 +1081,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   W.zc = surf;  // tcur is 0+
   W.ans = Val{BIG, 0.f};
   W.answered = false;
+  W.did = 0u;
   W.u = u;
   W.guard = 0;
   W.live = true;
@@ -954,7 +1100,7 @@ __device__ __forceinline__ Val plane_time(const Desc& S, const TrackF& T, float 
 
 // One section of the walk: the section W.k and its intervals, SEARCH and STRETCH in it,
 // then the next section.  W.live turns false when the walk is over.
-template <bool TUBE, bool FRAME = false>
+template <bool TUBE, bool FRAME = false, bool RANK = false>
 __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
   const int last = S.nz - 1;
   bool u = W.u;
@@ -994,14 +1140,15 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
   if (!beyond) {
     const float ao = TUBE ? 0.f : S.oah[k];
     const Lat Lo = lateral<TUBE>(S.oah[k], S.oal[k], S.obh[k], S.obl[k], S.ok_[k], W.rh, W.rl, T, true);
-    const Quad qo = quad32<TUBE, FRAME>(ao, TUBE ? 0.f : S.oal[k], Lo, T, W.rad, W.erad, W.A0, W.rh, W.rl);
+    const Quad qo = quad32<TUBE, FRAME, RANK>(ao, TUBE ? 0.f : S.oal[k], Lo, T, W.rad, W.erad, W.A0, W.rh, W.rl);
     u |= qo.unsure;
-    const Iv lat = iv_and(iv_region(qo, Lo.g, Lo.E, u), W.PH);  // lateral and phi part of C
+    const Iv reg = iv_region(qo, Lo.g, Lo.E, u);
+    const Iv lat = iv_and(reg, W.PH);  // lateral and phi part of C
     Iv X1 = iv_none();
     if ((S.inner >> k) & 1u) {
       const float ai = TUBE ? 0.f : S.iah[k];
       const Lat Li = lateral<TUBE>(S.iah[k], S.ial[k], S.ibh[k], S.ibl[k], S.ik_[k], W.rh, W.rl, T, false);
-      const Quad qi = quad32<TUBE, FRAME>(ai, TUBE ? 0.f : S.ial[k], Li, T, W.rad, W.erad, W.A0, W.rh, W.rl);
+      const Quad qi = quad32<TUBE, FRAME, RANK>(ai, TUBE ? 0.f : S.ial[k], Li, T, W.rad, W.erad, W.A0, W.rh, W.rl);
       u |= qi.unsure;
       X1 = iv_region(qi, -Li.g, Li.E, u);
       if (!X1.empty && !(X1.lo.v < X1.hi.v)) {  // no hole along the ray, unless too close to tell
@@ -1011,6 +1158,20 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
     }
     const Iv& X2 = W.X2;
     const Iv C = iv_and(lat, slab);
+    // RANK: the crossing an answer t is, from the values it was taken from; unsure when another
+    // of them lies within reach of it.
+    auto among = [&](Val t, Val a, uint32_t ia, Val b, uint32_t ib, Val c, uint32_t ic, Val d, uint32_t id) {
+      uint32_t near = 0, at = kNone;
+      if (fabsf(a.v - t.v) <= a.e + t.e) { near++; at = ia; }
+      if (fabsf(b.v - t.v) <= b.e + t.e) { near++; at = ib; }
+      if (fabsf(c.v - t.v) <= c.e + t.e) { near++; at = ic; }
+      if (fabsf(d.v - t.v) <= d.e + t.e) { near++; at = id; }
+      if (near != 1 || at == kNone) u = true;
+      W.did = at;
+    };
+    const Val none{BIG, 0.f};
+    const uint32_t plo = (W.pid & kPidLoTie) ? (uint32_t)kNone : ver_dist((W.pid & kPidLoE) ? kPhiE : kPhiS, 0);
+    const uint32_t phi = (W.pid & kPidHiTie) ? (uint32_t)kNone : ver_dist((W.pid & kPidHiE) ? kPhiE : kPhiS, 0);
     // v at or before tcur (passed): the same crossing, certainly earlier, or within 0+
     auto passed = [&](Val v) -> bool {
       if (W.zc) return !after0(v);
@@ -1038,6 +1199,13 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
         W.ans = t;
         W.answered = true;
         W.st = kDone;
+        if (RANK) {
+          // an entry by the section's slab is one by the solid's first plane along the ray
+          const bool first = (step > 0 && k == 0) || (step < 0 && k + 1 == last);
+          const uint32_t zid = !first ? (uint32_t)kNone : ver_dist(kZLow, step > 0 ? 0 : last);
+          if (t.v == C.lo.v) among(t, reg.lo, ver_dist(kOuter, k), W.PH.lo, plo, slab.lo, zid, none, kNone);
+          else among(t, X1.empty ? none : X1.hi, ver_dist(kInner, k), X2.empty ? none : X2.hi, phi, none, kNone, none, kNone);
+        }
         return;
       }
       W.st = kStretch;  // DistanceToOut from the piece's start, or a leaving point inside at 0+
@@ -1048,8 +1216,10 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
     if (W.st == kStretch) {
       const int at = in_piece(lat, X1, X2, W.tcur, W.zc);
       Val e = lat.hi;  // end of the inside stretch holding tcur
-      if (!X1.empty && (W.zc ? after0(X1.lo) : X1.lo.v > W.tcur.v)) e = vmin(e, X1.lo);
-      if (!X2.empty && (W.zc ? after0(X2.lo) : X2.lo.v > W.tcur.v)) e = vmin(e, X2.lo);
+      const bool x1 = !X1.empty && (W.zc ? after0(X1.lo) : X1.lo.v > W.tcur.v);
+      const bool x2 = !X2.empty && (W.zc ? after0(X2.lo) : X2.lo.v > W.tcur.v);
+      if (x1) e = vmin(e, X1.lo);
+      if (x2) e = vmin(e, X2.lo);
       if (at <= 0) {  // the section must hold tcur (the profile is continuous)
         u = true;
         W.st = kDone;
@@ -1062,6 +1232,7 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
           W.ans = slab.hi;
           W.answered = true;
           W.st = kDone;
+          if (RANK) W.did = ver_dist(kZLow, step > 0 ? last : 0);
         } else {
           W.st = kDone;  // leaves through an end plane: no entry after it
         }
@@ -1069,6 +1240,7 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
         W.ans = e;
         W.answered = true;
         W.st = kDone;
+        if (RANK) among(e, reg.hi, ver_dist(kOuter, k), W.PH.hi, phi, x1 ? X1.lo : none, ver_dist(kInner, k), x2 ? X2.lo : none, plo);
       } else {  // a leaving point's stretch ends: look for the next entry
         W.tcur = e;
         W.zc = false;
@@ -1084,9 +1256,15 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
 }
 
 // The distances from a finished walk (nothing when none was needed).
+template <bool RANK = false>
 __device__ inline void pcon_end(const Walk& W, R32& R) {
   bool u = W.u;
   if (W.st == kStretch) u = true;  // a stretch must end at a surface
+  if (RANK) {
+    if ((W.need_out || W.need_in) && (u || (W.need_out && !W.answered && R.code == 0))) R.flag = true;
+    if (W.answered) R.rank |= W.did;
+    return;
+  }
   if (W.need_out) {
     // entering surface point whose ray never gets inside: 0
     const Val d = W.answered ? W.ans : Val{0.f, 0.f};
@@ -1099,12 +1277,13 @@ __device__ inline void pcon_end(const Walk& W, R32& R) {
   }
 }
 
-template <bool TUBE, bool FRAME = false>
+template <bool TUBE, bool FRAME = false, bool RANK = false>
 __device__ inline void pcon32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   Walk W;
-  if (pcon_begin<TUBE, FRAME>(S, T, want, R, W))
-    while (W.live) pcon_step<TUBE, FRAME>(S, T, W);
-  pcon_end(W, R);
+  W.answered = false;
+  if (pcon_begin<TUBE, FRAME, RANK>(S, T, want, R, W))
+    while (W.live) pcon_step<TUBE, FRAME, RANK>(S, T, W);
+  pcon_end<RANK>(W, R);
 }
 
 }  // namespace f32
