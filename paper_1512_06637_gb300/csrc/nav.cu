@@ -26,6 +26,7 @@
 #include <vector>
 #include <array>
 #include "gv_internal.h"
+#include "nav_cull.cuh"
 #include "solid_fp32.cuh"
 #include "solid_fp64.cuh"
 
@@ -75,12 +76,14 @@ struct gv_geom {
   gv::NodeD* d_nodes = nullptr;
   int32_t* d_children = nullptr;
   gv::Desc* d_solids = nullptr;
+  gv::Cull* d_cull = nullptr;  // per node
   gv::GridD* d_grids = nullptr;
   int32_t* d_cells = nullptr;
   int32_t* d_list = nullptr;
   bool use_vox = true;
   bool walk32 = false;  // some node with a grid has at least kWalk32Min daughters
   std::vector<gv::NodeD> nodes;
+  std::vector<gv::Cull> cull;
   std::vector<int32_t> children;
   std::vector<gv::Desc> solids;
   std::vector<gv::GridD> grids;
@@ -314,6 +317,29 @@ __device__ __forceinline__ void order_by_kind(int kind, int m, int* scount, int*
   __syncthreads();
 }
 
+// The same for a tile of len tracks (more than one per thread): perm[r] is the offset of rank r.
+__device__ __forceinline__ void order_tile(const NodeD* __restrict__ nodes, const Desc* __restrict__ solids, int nnodes,
+                                           const int32_t* __restrict__ node, int len, const Vox& vox, int* scount,
+                                           uint8_t* skind, uint16_t* perm) {
+  const int t = threadIdx.x;
+  if (t < kKinds) scount[t] = 0;
+  __syncthreads();
+  for (int j = t; j < len; j += blockDim.x) {
+    const int32_t v = node[j];
+    const int kind = (v >= 0 && v < nnodes) ? volume_kind(nodes, solids, v, vox) : kKinds - 2;
+    skind[j] = (uint8_t)kind;
+    atomicAdd(&scount[kind], 1);
+  }
+  __syncthreads();
+  if (t == 0) {
+    int acc = 0;
+    for (int k = 0; k < kKinds; k++) { const int c = scount[k]; scount[k] = acc; acc += c; }
+  }
+  __syncthreads();
+  for (int j = t; j < len; j += blockDim.x) perm[atomicAdd(&scount[skind[j]], 1)] = (uint16_t)j;
+  __syncthreads();
+}
+
 // One thread per track; the block's 256 tracks are taken in order of the kind of volume
 // they are in, so that a warp runs one path through the geometry.
 __global__ void __launch_bounds__(256) k_nav_fp64(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
@@ -350,22 +376,7 @@ __global__ void __launch_bounds__(256) k_nav_fp64_tiles(const NodeD* __restrict_
   const int t = threadIdx.x;
   for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {  // block-uniform
     const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
-    if (t < kKinds) scount[t] = 0;
-    __syncthreads();
-    for (int j = t; j < len; j += 256) {
-      const int32_t v = a.node[t0 + j];
-      const int kind = (v >= 0 && v < nnodes) ? volume_kind(nodes, solids, v, vox) : kKinds - 2;
-      skind[j] = (uint8_t)kind;
-      atomicAdd(&scount[kind], 1);
-    }
-    __syncthreads();
-    if (t == 0) {
-      int acc = 0;
-      for (int k = 0; k < kKinds; k++) { const int c = scount[k]; scount[k] = acc; acc += c; }
-    }
-    __syncthreads();
-    for (int j = t; j < len; j += 256) sperm[atomicAdd(&scount[skind[j]], 1)] = (uint16_t)j;
-    __syncthreads();
+    order_tile(nodes, solids, nnodes, a.node + t0, len, vox, scount, skind, sperm);
     for (int r = t; r < len; r += 256) nav_step64(nodes, children, solids, nnodes, a, t0 + sperm[r], vox);
     __syncthreads();  // the tile's shared arrays are reused by the next tile
   }
@@ -503,6 +514,195 @@ __device__ __forceinline__ void group_merge(unsigned mask, Top2<DEDUP>& top) {
     const int ow2 = DEDUP ? __shfl_xor_sync(mask, top.w2, off) : kNone;
     top.add(ob1, oe1, ow1);
     top.add(ob2, oe2, ow2);
+  }
+}
+
+// One thread per track, for geometries whose nodes are scanned (no grid walk): the block takes its
+// tracks in order of volume kind in tiles of 1024; every daughter gets the plain look of
+// nav_cull.cuh, and only those it leaves (a ray that may meet the daughter, a safety that may be
+// the least) are evaluated with certified bounds.  A lane leaves from none to a dozen daughters, so
+// the warp gathers its 32 tracks' (track, daughter) pairs in shared memory and evaluates them 32 at
+// a time, one per lane; each lane then reads its own pairs' results.
+// Measured (GB300, nested detector, 2^22 tracks with safety): 12.0 -> 2.75 ms (before: 8 lanes per
+// track, every daughter evaluated: 1214 warp instructions per track at 18 of 32 lanes; now 263 at 26).
+// Without the pairs, each lane evaluating its own daughters: 5.8 ms (12 lanes).  Three blocks per SM
+// (80 registers) 2.73, tiles of 2048 2.72 ms.
+constexpr int kScanTile = 1024;
+constexpr int kScanPairs = 256;  // pairs a warp evaluates per round
+struct ScanWarp {
+  float w[12][32];           // the warp's tracks, split (world frame)
+  int32_t node[32];
+  uint32_t pair[kScanPairs]; // track's lane << 27 | daughter order
+  float din[kScanPairs], sin[kScanPairs];  // results (din NaN: flagged)
+};
+__global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
+                                                       const Desc* __restrict__ solids, const Cull* __restrict__ cull,
+                                                       int nnodes, NavArgs a, uint32_t* __restrict__ wl,
+                                                       unsigned long long* __restrict__ cnt, Vox vox) {
+  constexpr int kMother = 0x7ffffffe, kNone = 0x7fffffff;
+  const unsigned lane = threadIdx.x & 31u;
+  const bool want_saf = a.safety != nullptr;
+  const unsigned want = f32::kWantDin | (want_saf ? f32::kWantSin : 0u);
+  const uint2 *X = reinterpret_cast<const uint2*>(a.x), *Y = reinterpret_cast<const uint2*>(a.y),
+              *Z = reinterpret_cast<const uint2*>(a.z), *Ux = reinterpret_cast<const uint2*>(a.u),
+              *Uy = reinterpret_cast<const uint2*>(a.v), *Uz = reinterpret_cast<const uint2*>(a.w);
+  __shared__ int scount[kKinds];
+  __shared__ uint16_t sperm[kScanTile];
+  __shared__ uint8_t skind[kScanTile];
+  __shared__ ScanWarp swarp[8];
+  ScanWarp& Q = swarp[threadIdx.x >> 5];
+  const int tile = a.n >= (int64_t)gridDim.x * kScanTile ? kScanTile : 256;  // short baskets: more blocks
+  for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < a.n; t0 += (int64_t)gridDim.x * tile) {  // block-uniform
+    const int len = a.n - t0 < tile ? (int)(a.n - t0) : tile;
+    order_tile(nodes, solids, nnodes, a.node + t0, len, vox, scount, skind, sperm);
+    for (int r0 = 0; r0 < len; r0 += 256) {
+      const int r = r0 + (int)threadIdx.x;
+      const bool valid = r < len;
+      const int64_t i = t0 + (valid ? sperm[r] : 0);
+      bool flag = false;
+      Top2<false> top{F_INF, 0.f, F_INF, 0.f, kNone, kNone};
+      float saf = F_INF, mdout = 0.f, mssf = 0.f;
+      int32_t v = -1;
+      PlainTrack P;
+      int count = 0;
+      const int32_t* ids = nullptr;
+      if (valid) {
+        v = a.node[i];
+        flag = v < 0 || v >= nnodes;
+      }
+      if (valid && !flag) {
+        const f32::TrackF W = f32::load_track(X, Y, Z, Ux, Uy, Uz, i, true);
+        const float c[12] = {W.xh, W.yh, W.zh, W.xl, W.yl, W.zl, W.u, W.v, W.w, W.ul, W.vl, W.wl};
+#pragma unroll
+        for (int k = 0; k < 12; k++) Q.w[k][lane] = c[k];
+        const NodeD& N = nodes[v];
+        f32::R32 R;
+        query32(solids[N.desc], to_local32(N, W), f32::kWantDout | (want_saf ? f32::kWantSout : 0u), R);
+        flag = W.bad || R.flag || R.dout < 0;  // a point outside its own volume: binary64 decides
+        top.add(R.dout, half_tol(R.dout), kMother);
+        if (want_saf) saf = R.sout;
+        mdout = R.dout;
+        mssf = saf;
+        P = plain_track(W);
+        ids = children + N.first;
+        count = flag ? 0 : N.count;
+      }
+      // The plain look.  s1, s2: the two daughters of least plain safety among those not evaluated
+      // anyway; s3 the third's; ub the upper bound of the least safety.
+      float s1 = F_INF, s2 = F_INF, s3 = F_INF, ub = saf;
+      int j1 = -1, j2 = -1, j0 = 0;
+      bool all = false;  // evaluate every daughter (several of nearly the same safety)
+      while (__any_sync(0xffffffffu, j0 < count)) {
+        unsigned mask = 0u;
+        const int m = min(32, count - j0);
+        for (int b = 0; b < m; b++) {
+          const Cull& C = cull[ids[j0 + b]];
+          const int tag = C.tag;
+          bool take = all || tag == kCullNever || (want_saf && tag == kCullOther);
+          if (!take) {
+            const PlainLocal L = plain_local(C, P);
+            take = !plain_miss(C, P, L);
+            if (want_saf) {
+              const float s = plain_safety(C, L), lb = s - L.margin;
+              ub = fminf(ub, s < L.margin ? F_INF : s + L.margin);  // a point not outside gives none
+              if (take) {  // evaluated anyway
+              } else if (lb < s1) {
+                s3 = s2; s2 = s1; j2 = j1; s1 = lb; j1 = j0 + b;
+              } else if (lb < s2) {
+                s3 = s2; s2 = lb; j2 = j0 + b;
+              } else {
+                s3 = fminf(s3, lb);
+              }
+            }
+          }
+          if (take) mask |= 1u << b;
+        }
+        const int first = j0;
+        j0 += 32;
+        if (want_saf && !all && m > 0 && j0 >= count) {  // the last daughters: those of least safety too
+          if (s3 <= ub) {  // start over, without the look
+            all = true;
+            j0 = 0;
+            mask = 0u;
+            top = Top2<false>{mdout, half_tol(mdout), F_INF, 0.f, kMother, kNone};
+            saf = mssf;
+          } else {
+            if (!(s1 <= ub)) j1 = -1;
+            if (!(s2 <= ub)) j2 = -1;
+          }
+        }
+        const bool ends = want_saf && !all && m > 0 && j0 >= count;
+        // evaluate the pairs in rounds
+        unsigned extra = ends ? (j1 >= 0 ? 1u : 0u) | (j2 >= 0 ? 2u : 0u) : 0u;
+        while (__any_sync(0xffffffffu, mask | extra)) {
+          const int mine = __popc(mask) + __popc(extra);
+          int at = mine;
+          for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, at, o);
+            if ((int)lane >= o) at += up;
+          }
+          const int total = min(__shfl_sync(0xffffffffu, at, 31), kScanPairs);
+          at -= mine;
+          int end = at;
+          while ((mask | extra) && end < kScanPairs) {
+            int j;
+            if (mask) {
+              j = first + __ffs(mask) - 1;
+              mask &= mask - 1u;
+            } else {
+              j = (extra & 1u) ? j1 : j2;
+              extra &= extra - 1u;
+            }
+            Q.pair[end++] = lane << 27 | (uint32_t)j;
+          }
+          Q.node[lane] = v;
+          __syncwarp();
+          for (int q = (int)lane; q < total; q += 32) {
+            const uint32_t e = Q.pair[q];
+            const unsigned l = e >> 27;
+            f32::TrackF W;
+            W.xh = Q.w[0][l]; W.yh = Q.w[1][l]; W.zh = Q.w[2][l];
+            W.xl = Q.w[3][l]; W.yl = Q.w[4][l]; W.zl = Q.w[5][l];
+            W.u = Q.w[6][l]; W.v = Q.w[7][l]; W.w = Q.w[8][l];
+            W.ul = Q.w[9][l]; W.vl = Q.w[10][l]; W.wl = Q.w[11][l];
+            W.bad = false;
+            const NodeD& C = nodes[children[nodes[Q.node[l]].first + (int)(e & 0x7ffffffu)]];
+            f32::R32 R;
+            query32(solids[C.desc], to_local32(C, W), want, R);
+            Q.din[q] = R.flag ? CUDART_NAN_F : R.din;
+            Q.sin[q] = R.sin;
+          }
+          __syncwarp();
+          for (int q = at; q < end; q++) {
+            const float t = Q.din[q];
+            flag |= isnan(t);
+            if (t >= 0) top.add(t, half_tol(t), (int)(Q.pair[q] & 0x7ffffffu));
+            if (want_saf && Q.sin[q] >= 0) saf = fminf(saf, Q.sin[q]);
+          }
+          __syncwarp();
+        }
+      }
+      if (valid && !flag) {
+        // the winner must be certain: the runner-up's interval may not meet it; no finite step:
+        // binary64 decides
+        flag = !isfinite(top.b1) || top.b2 - top.e2 <= top.b1 + top.e1;
+        if (!flag) {
+          a.step[i] = (double)top.b1;
+          if (want_saf) a.safety[i] = isfinite(saf) ? (double)saf : -1.0;
+          a.next[i] = top.w1 == kMother ? -1 : ids[top.w1];
+        }
+      }
+      const bool push = valid && flag;
+      const unsigned m = __ballot_sync(0xffffffffu, push);
+      if (m) {
+        unsigned long long at = 0;
+        const int leader = __ffs(m) - 1;
+        if ((int)lane == leader) at = atomicAdd(cnt, (unsigned long long)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, leader);
+        if (push) wl[at + __popc(m & ((1u << lane) - 1u))] = (uint32_t)i;
+      }
+    }
+    __syncthreads();  // the tile's shared arrays are reused by the next tile
   }
 }
 
@@ -1116,6 +1316,31 @@ static void build_grids(gv_geom* g) {
   }
 }
 
+// The plain records of nav_cull.cuh.
+static void build_cull(gv_geom* g) {
+  g->cull.resize(g->nnodes);
+  for (int v = 0; v < g->nnodes; v++) {
+    const NodeD& N = g->nodes[v];
+    const Desc& h = g->solids[N.desc];
+    Cull& C = g->cull[v];
+    std::memset(&C, 0, sizeof(C));
+    for (int i = 0; i < 9; i++) C.R[i] = (float)N.R[i];
+    double mag = 0;
+    for (int i = 0; i < 3; i++) {
+      C.t[i] = (float)N.t[i];
+      C.e[i] = (float)h.ext[i];
+      mag += std::fabs(N.t[i]) + h.ext[i];
+    }
+    C.margin = (float)(4e-6 * mag);
+    C.solid = N.desc;
+    if (h.type == kBool || (h.flags & kFp64Only)) C.tag = kCullNever;
+    else if (h.type == kBox) C.tag = kCullBox;
+    else if (h.type == kTube && !(h.flags & kHasPhi)) C.tag = kCullTube;
+    else C.tag = kCullOther;
+    if (C.tag == kCullTube && (h.inner & 1u)) C.rmin = (float)h.in[0].b;  // a = 0: the radius
+  }
+}
+
 }  // namespace gv
 
 extern "C" {
@@ -1176,9 +1401,12 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
   const int nrec = table_size(uniq.data(), g->nsolids);  // booleans carry their components along
   for (const gv_solid* u : uniq) g->solids.push_back(u->h);  // host copies for the grid builder
   build_grids(g);
+  build_cull(g);
   cudaError_t e = cudaGetDevice(&g->device);
   if (e == cudaSuccess) e = cudaMalloc(&g->d_nodes, sizeof(NodeD) * nnodes);
   if (e == cudaSuccess) e = cudaMalloc(&g->d_children, sizeof(int32_t) * g->children.size());
+  if (e == cudaSuccess) e = cudaMalloc(&g->d_cull, sizeof(Cull) * nnodes);
+  if (e == cudaSuccess) e = cudaMemcpy(g->d_cull, g->cull.data(), sizeof(Cull) * nnodes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&g->d_solids, sizeof(Desc) * nrec);
   if (e == cudaSuccess) g->solids = table_records(uniq.data(), g->nsolids, g->d_solids);
   if (e == cudaSuccess) e = cudaMemcpy(g->d_nodes, g->nodes.data(), sizeof(NodeD) * nnodes, cudaMemcpyHostToDevice);
@@ -1207,6 +1435,7 @@ void gv_geom_destroy(gv_geom* g) {
   if (g->d_nodes) cudaFree(g->d_nodes);
   if (g->d_children) cudaFree(g->d_children);
   if (g->d_solids) cudaFree(g->d_solids);
+  if (g->d_cull) cudaFree(g->d_cull);
   if (g->d_grids) cudaFree(g->d_grids);
   if (g->d_cells) cudaFree(g->d_cells);
   if (g->d_list) cudaFree(g->d_list);
@@ -1272,15 +1501,17 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
     ws->fused_blocks = 0;  // this pass counts its refinements in the counter
     cudaError_t e = cudaMemsetAsync(ws->counter, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return cuda_error(e, "nav: counter reset");
-    const int64_t per_block = 256 / kLanes;
-    int64_t blocks = std::min<int64_t>((t->n + per_block - 1) / per_block, (int64_t)sms * 8);
     const Vox vox = vox_of(g);
-    if (vox.grids && g->walk32)
+    if (vox.grids && g->walk32) {
+      const int64_t per_block = 256 / kLanes;
+      const int64_t blocks = std::min<int64_t>((t->n + per_block - 1) / per_block, (int64_t)sms * 8);
       k_nav_fp32<true><<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a,
                                                          ws->idx, ws->counter, vox);
-    else
-      k_nav_fp32<false><<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a,
-                                                          ws->idx, ws->counter, vox);
+    } else {
+      const int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sms * 2);
+      k_nav_scan32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
+                                                     ws->idx, ws->counter, vox);
+    }
     k_nav_refine<<<(unsigned)(sms * 2), 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a, ws->idx,
                                                        ws->counter, vox_of(g));
   }
