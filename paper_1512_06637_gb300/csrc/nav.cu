@@ -13,10 +13,11 @@
 // Locate descends from the world into the first daughter (in index order) that
 // does not classify the point as outside.
 //
-// Kernels: binary64, one thread per track; binary32 with kLanes lanes per track
-// (daughters dealt round-robin to the lanes, results combined with warp
-// shuffles), whose tracks with an ambiguous minimum, an uncertain daughter or a
-// polycone are recomputed by the binary64 kernel from a worklist.  World-to-node
+// Kernels: binary64, one thread per track, with the candidates ranked in certified binary32 and
+// only the deciding one evaluated in binary64 (the same bits); binary32, one thread per track
+// over scanned daughters (k_nav_scan32) or kLanes lanes per track along a grid (k_nav_fp32), whose
+// tracks with an ambiguous minimum or an uncertain daughter are recomputed by the binary64 step from
+// a worklist.  World-to-node
 // transforms are composed on the host (binary64, no fused multiply-add) and
 // applied on the device with round-to-nearest operations in a fixed order, so the
 // binary64 results and codes agree with any evaluation that uses the same order.
@@ -27,6 +28,7 @@
 #include <array>
 #include "gv_internal.h"
 #include "nav_cull.cuh"
+#include "rank_fp64.cuh"
 #include "solid_fp32.cuh"
 #include "solid_fp64.cuh"
 
@@ -50,13 +52,27 @@ struct GridD {
   double lo[3], cell[3], inv[3];  // origin, cell edges, their inverses
   int32_t n[3];                   // cells per axis
   int32_t start;                  // first cell's entry in the geometry's cell table
+  int32_t safe;                   // first cell's safety list (-1: none)
+  float flo[3], fcell[3], finv[3];
 };
+
+// An entry of a cell's safety list: a daughter and a lower bound of its SafetyToIn at the cell's
+// centre.  A list holds the kSafeList daughters of least bound, in increasing order.
+struct SafeEnt {
+  float s;
+  int32_t node;
+};
+constexpr int kSafeList = 64;
+// Lists are built for grids of at most these many daughters and cells.
+constexpr int kSafeDaughters = 8192, kSafeCells = 32768;
 
 // Device pointers of a geometry's grids (grids == nullptr: no grid is used).
 struct Vox {
   const GridD* grids;
   const int32_t* cells;  // per cell: [begin, end) into list
   const int32_t* list;
+  const SafeEnt* safe;   // kSafeList entries per cell (node -1: fewer daughters)
+  const float* safe_cut;  // per cell: a lower bound for the daughters not listed
 };
 
 // Nodes with at least this many daughters get a grid.
@@ -66,6 +82,7 @@ constexpr int kVoxelMin = 16;
 // dozen daughters.
 constexpr int kWalk32Min = 128;
 
+constexpr float kInf32 = __builtin_huge_valf();
 constexpr int kLanes = 8;  // lanes per track in the binary32 kernel
 
 }  // namespace gv
@@ -80,6 +97,8 @@ struct gv_geom {
   gv::GridD* d_grids = nullptr;
   int32_t* d_cells = nullptr;
   int32_t* d_list = nullptr;
+  gv::SafeEnt* d_safe = nullptr;
+  float* d_safe_cut = nullptr;
   bool use_vox = true;
   bool walk32 = false;  // some node with a grid has at least kWalk32Min daughters
   std::vector<gv::NodeD> nodes;
@@ -146,6 +165,32 @@ __device__ __forceinline__ void candidates64(const NodeD& N, const int32_t* __re
   count = vox.cells[2 * cell + 1] - vox.cells[2 * cell];
 }
 
+// The same for a point in plain binary32 in N's frame (Cull of N), when it is certain which cell the
+// point is in (false: not certain).
+__device__ __forceinline__ bool candidates32(const NodeD& N, const Cull& C, const int32_t* __restrict__ children,
+                                             const Vox& vox, const PlainTrack& P, const int32_t*& ids, int& count) {
+  ids = children + N.first;
+  count = N.count;
+  if (!vox.grids || N.grid < 0) return true;
+  const GridD& G = vox.grids[N.grid];
+  const PlainLocal L = plain_local(C, P);
+  int c[3];
+  bool sure = true, out = false;
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const float f = (L.q[a] - G.flo[a]) * G.finv[a], tol = 2.f * L.margin * G.finv[a] + 1e-6f * fabsf(f);
+    const float k = floorf(f);
+    sure &= f - k > tol && k + 1.f - f > tol && isfinite(f);
+    out |= f < -tol || f > (float)G.n[a] + tol;
+    c[a] = min(max((int)k, 0), G.n[a] - 1);
+  }
+  if (out) { count = 0; return true; }
+  const int cell = G.start + (c[2] * G.n[1] + c[1]) * G.n[0] + c[0];
+  ids = vox.list + vox.cells[2 * cell];
+  count = vox.cells[2 * cell + 1] - vox.cells[2 * cell];
+  return sure;
+}
+
 struct NavArgs {
   const double *x, *y, *z, *u, *v, *w;
   const int32_t* node;
@@ -210,83 +255,193 @@ struct Dda {
 // the tie margin of `best`.
 __device__ __forceinline__ bool walk_done(double tenter, double best) { return tenter > best + 4e-9 * (1.0 + best); }
 
-__device__ inline void grid_entries(const NodeD* __restrict__ nodes, const Desc* __restrict__ solids, const NodeD& N,
-                                    const Vox& vox, const double p[3], const double d[3], double& best, int32_t& who,
-                                    bool& have, double& runner) {
-  const GridD& G = vox.grids[N.grid];
-  double q[3], e[3];
-  to_local64(N, p[0], p[1], p[2], q[0], q[1], q[2]);
-  rot_local64(N, d[0], d[1], d[2], e[0], e[1], e[2]);
+// The world track in plain binary32 (hi parts).
+__device__ __forceinline__ PlainTrack plain_world(const double p[3], const double d[3]) {
+  const float x = (float)p[0], y = (float)p[1], z = (float)p[2];
+  return {x, y, z, (float)d[0], (float)d[1], (float)d[2], 4e-6f * (fabsf(x) + fabsf(y) + fabsf(z))};
+}
+// No daughter first met at `from` or later can give a distance within a tie margin of `best`.
+__device__ __forceinline__ bool beyond(float from, double best) { return (double)from > best + 1e-6 * (1.0 + best); }
+
+// What is the same for every track of a launch.
+struct Geo {
+  const NodeD* nodes;
+  const int32_t* children;
+  const Desc* solids;
+  const Cull* cull;
+  int nnodes;
+  Vox vox;
+};
+
+// The daughters of a node that a ray may enter, one after the other: all of them in index order, or,
+// in a node with a grid, those listed in the cells along the ray; certain misses and daughters
+// first met beyond the best distance so far are passed over.
+struct Finder {
+  const Geo& g;
+  const NodeD& N;
+  PlainTrack P;
+  const GridD* G;  // nullptr: scan
   Dda D;
-  if (!D.begin(G, q, e)) return;
-  int32_t recent[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
-  int slot = 0;
-  f64::Track T;
-  f64::Result R;
-  do {
-    if (have && walk_done(D.tenter, best)) break;
-    const int cell = D.cell(G);
-    for (int j = vox.cells[2 * cell]; j < vox.cells[2 * cell + 1]; j++) {
-      const int32_t id = vox.list[j];
-      bool seen = false;
-      for (int r = 0; r < 8; r++) seen |= recent[r] == id;
-      if (seen) continue;
-      recent[slot] = id;
-      slot = (slot + 1) & 7;
-      const NodeD& C = nodes[id];
-      to_local64(C, p[0], p[1], p[2], T.x, T.y, T.z);
-      rot_local64(C, d[0], d[1], d[2], T.u, T.v, T.w);
-      query64(solids[C.desc], T, f64::kWantDin, R);
-      const double t = R.din;
-      if (t >= 0 && (!have || t < best || (t == best && (who == -1 || id < who)))) {
-        if (have && best < runner) runner = best;
-        best = t; who = id; have = true;
-      } else if (t >= 0 && id != who && t < runner) {  // a daughter seen again is not its own runner-up
-        runner = t;
-      }
+  int at, end;
+  bool over;
+  __device__ __forceinline__ Finder(const Geo& geo, const NodeD& node, const PlainTrack& plain, const double p[3],
+                                    const double d[3])
+      : g(geo), N(node), P(plain), G(nullptr), at(0), end(node.count), over(false) {
+    if (g.vox.grids && N.grid >= 0) {
+      G = g.vox.grids + N.grid;
+      double q[3], e[3];
+      to_local64(N, p[0], p[1], p[2], q[0], q[1], q[2]);
+      rot_local64(N, d[0], d[1], d[2], e[0], e[1], e[2]);
+      over = !D.begin(*G, q, e);
+      if (!over) cell();
     }
-  } while (D.advance(G));
+  }
+  __device__ __forceinline__ void cell() {
+    const int c = D.cell(*G);
+    at = g.vox.cells[2 * c];
+    end = g.vox.cells[2 * c + 1];
+  }
+  // the next daughter (-1: no more) given the best distance so far (`have`) and its node
+  __device__ __forceinline__ int32_t next(bool have, double best, int32_t who) {
+    while (!over) {
+      for (; at < end; at++) {
+        const int32_t id = G ? g.vox.list[at] : g.children[N.first + at];
+        if (id == who) continue;  // listed in several cells
+        const Cull& C = g.cull[id];
+        float from;
+        bool near;
+        if (plain_miss(C, P, plain_local(C, P), from, near)) continue;
+        if (have && beyond(from, best)) continue;
+        at++;
+        return id;
+      }
+      over = !G || !D.advance(*G) || (have && walk_done(D.tenter, best));
+      if (!over) cell();
+    }
+    return -1;
+  }
+};
+
+// The cell of a grid whose safety list serves a point: the nearest one; its distance from the
+// cell's centre (with margin).
+__device__ __forceinline__ int safe_cell(const GridD& G, const NodeD& N, const Cull& C, const PlainTrack& P, float& dist) {
+  const PlainLocal L = plain_local(C, P);
+  int c[3];
+  float d2 = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    c[a] = min(max((int)((L.q[a] - G.flo[a]) * G.finv[a]), 0), G.n[a] - 1);
+    const float m = L.q[a] - (G.flo[a] + ((float)c[a] + 0.5f) * G.fcell[a]);
+    d2 = fmaf(m, m, d2);
+  }
+  dist = 1.00001f * sqrtf(d2) + 4.f * L.margin;
+  return (c[2] * G.n[1] + c[1]) * G.n[0] + c[0];
 }
 
-__device__ inline void nav_step64(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                  const Desc* __restrict__ solids, int nnodes, const NavArgs& a, int64_t i,
-                                  const Vox& vox = Vox{nullptr, nullptr, nullptr}) {
-  const int32_t v = a.node[i];
-  if (v < 0 || v >= nnodes) {
-    a.step[i] = -1.0; a.next[i] = -1;
-    if (a.safety) a.safety[i] = -1.0;
-    return;
+// The daughters of a node that may have the least SafetyToIn, one after the other; a daughter whose
+// lower bound exceeds the least safety so far is passed over.  With a safety list the daughters come
+// in the order of their safety at the cell's centre s_c, and s_c less the point's distance from the
+// centre is a lower bound (a safety changes by at most the distance between two points).  `never`:
+// only the daughters without a binary32 form (else only the others).
+struct Nearest {
+  const Geo& g;
+  const NodeD& N;
+  const PlainTrack& P;
+  const SafeEnt* list;  // nullptr: scan
+  float dist, cut;
+  int at;
+  bool never;
+  __device__ __forceinline__ Nearest(const Geo& geo, const NodeD& node, const Cull& C, const PlainTrack& p, bool nv)
+      : g(geo), N(node), P(p), list(nullptr), dist(0.f), cut(kInf32), at(0), never(nv) {
+    if (g.vox.grids && N.grid >= 0 && g.vox.grids[N.grid].safe >= 0) {
+      const GridD& G = g.vox.grids[N.grid];
+      const int cell = G.safe + safe_cell(G, N, C, P, dist);
+      list = g.vox.safe + (int64_t)cell * kSafeList;
+      cut = g.vox.safe_cut[cell];
+    }
   }
-  const double x = a.x[i], y = a.y[i], z = a.z[i], u = a.u[i], vv = a.v[i], w = a.w[i];
-  const NodeD& N = nodes[v];
-  const bool want_saf = a.safety != nullptr;
+  __device__ __forceinline__ void restart(bool nv) { at = 0; never = nv; }
+  // are the daughters that no list holds certainly farther than `least`?
+  __device__ __forceinline__ bool complete(double least) const { return !list || (double)(cut - dist) > least; }
+  __device__ __forceinline__ int32_t next(double least) {
+    const int count = list ? kSafeList : N.count;
+    while (at < count) {
+      int32_t id;
+      if (list) {
+        const SafeEnt E = list[at];
+        if (E.node < 0 || (double)(E.s - dist) > least) break;
+        id = E.node;
+      } else {
+        id = g.children[N.first + at];
+      }
+      at++;
+      const Cull& C = g.cull[id];
+      if ((C.tag == kCullNever) != never) continue;
+      if (C.tag <= kCullTube) {
+        const PlainLocal L = plain_local(C, P);
+        if ((double)(plain_safety(C, L) - L.margin) > least) continue;
+      }
+      return id;
+    }
+    at = count;
+    return -1;
+  }
+};
+
+struct Step {
+  double step, safety, second;  // second: the next smaller candidate, or a lower bound above every tie margin
+  int32_t next;
+};
+
+__device__ __forceinline__ void local64(const NodeD& C, const double p[3], const double d[3], f64::Track& T) {
+  to_local64(C, p[0], p[1], p[2], T.x, T.y, T.z);
+  rot_local64(C, d[0], d[1], d[2], T.u, T.v, T.w);
+}
+
+// The step of a track in node v in binary64 throughout.
+static __device__ __noinline__ void nav_exact(const Geo& g, int32_t v, const double p[3], const double d[3], bool want_saf,
+                                              Step& out) {
+  const NodeD& N = g.nodes[v];
   f64::Track T;
   f64::Result R;
-  to_local64(N, x, y, z, T.x, T.y, T.z);
-  rot_local64(N, u, vv, w, T.u, T.v, T.w);
-  query64(solids[N.desc], T, f64::kWantDout | (want_saf ? f64::kWantSout : 0u), R);
-  double best = R.dout, saf = R.sout;
+  local64(N, p, d, T);
+  query64(g.solids[N.desc], T, f64::kWantDout | (want_saf ? f64::kWantSout : 0u), R);
+  double best = R.dout, runner = CUDART_INF, saf = R.sout;
   bool have = best >= 0, have_s = want_saf && saf >= 0;
   int32_t who = -1;
-  const bool grid = vox.grids && N.grid >= 0;
-  const unsigned want = (grid ? 0u : f64::kWantDin) | (want_saf ? f64::kWantSin : 0u);
-  for (int j = 0; want != 0u && j < N.count; j++) {  // with a grid: only the safeties
-    const int32_t c = children[N.first + j];
-    const NodeD& C = nodes[c];
-    to_local64(C, x, y, z, T.x, T.y, T.z);
-    rot_local64(C, u, vv, w, T.u, T.v, T.w);
-    query64(solids[C.desc], T, want, R);
-    if (!grid && R.din >= 0 && (!have || R.din < best || (R.din == best && who == -1))) { best = R.din; who = c; have = true; }
-    if (want_saf && R.sin >= 0 && (!have_s || R.sin < saf)) { saf = R.sin; have_s = true; }
+  Finder F(g, N, plain_world(p, d), p, d);
+  for (int32_t id; (id = F.next(have, best, who)) >= 0;) {
+    local64(g.nodes[id], p, d, T);
+    query64(g.solids[g.nodes[id].desc], T, f64::kWantDin, R);
+    const double t = R.din;
+    if (t >= 0 && (!have || t < best || (t == best && (who == -1 || id < who)))) {
+      if (have && best < runner) runner = best;
+      best = t; who = id; have = true;
+    } else if (t >= 0 && t < runner) {
+      runner = t;
+    }
   }
-  if (grid) {
-    const double p[3] = {x, y, z}, dd[3] = {u, vv, w};
-    double runner = CUDART_INF;
-    grid_entries(nodes, solids, N, vox, p, dd, best, who, have, runner);
+  if (want_saf) {
+    Nearest S(g, N, g.cull[v], F.P, false);
+    for (int pass = 0; pass < 2; pass++) {
+      if (pass) {  // a list that may leave out the nearest: every daughter
+        if (S.complete(have_s ? saf : CUDART_INF)) break;
+        S.list = nullptr;
+      }
+      for (int nv = 0; nv < 2; nv++) {
+        S.restart(nv != 0);
+        for (int32_t id; (id = S.next(have_s ? saf : CUDART_INF)) >= 0;) {
+          local64(g.nodes[id], p, d, T);
+          query64(g.solids[g.nodes[id].desc], T, f64::kWantSin, R);
+          if (R.sin >= 0 && (!have_s || R.sin < saf)) { saf = R.sin; have_s = true; }
+        }
+      }
+    }
   }
-  a.step[i] = have ? best : -1.0;
-  if (want_saf) a.safety[i] = have_s ? saf : -1.0;
-  a.next[i] = have ? who : -1;
+  out.step = have ? best : -1.0;
+  out.next = have ? who : -1;
+  out.safety = have_s ? saf : -1.0;
+  out.second = runner;
 }
 
 // Volume kinds for gathering tracks that run the same code (the paper's baskets of
@@ -338,60 +493,6 @@ __device__ __forceinline__ void order_tile(const NodeD* __restrict__ nodes, cons
   __syncthreads();
   for (int j = t; j < len; j += blockDim.x) perm[atomicAdd(&scount[skind[j]], 1)] = (uint16_t)j;
   __syncthreads();
-}
-
-// One thread per track; the block's 256 tracks are taken in order of the kind of volume
-// they are in, so that a warp runs one path through the geometry.
-__global__ void __launch_bounds__(256) k_nav_fp64(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                                  const Desc* __restrict__ solids, int nnodes, NavArgs a, Vox vox) {
-  __shared__ int scount[kKinds];
-  __shared__ int sperm[256];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {  // block-uniform
-    const int64_t i0 = base + threadIdx.x;
-    int kind = kKinds - 1;
-    if (i0 < a.n) {
-      const int32_t v = a.node[i0];
-      kind = (v >= 0 && v < nnodes) ? volume_kind(nodes, solids, v, vox) : kKinds - 2;
-    }
-    order_by_kind(kind, blockDim.x, scount, sperm);
-    const int64_t i = base + sperm[threadIdx.x];
-    if (i < a.n) nav_step64(nodes, children, solids, nnodes, a, i, vox);
-    __syncthreads();
-  }
-}
-
-// The same in tiles of 256 * kNavTileItems tracks per block iteration: longer runs of one kind, so
-// fewer warps straddle two kinds.  Taken for baskets of at least four tiles per resident block
-// (two per SM), so that the last round of tiles leaves few SMs idle.
-constexpr int kNavTileItems = 4;
-__global__ void __launch_bounds__(256) k_nav_fp64_tiles(const NodeD* __restrict__ nodes,
-                                                        const int32_t* __restrict__ children,
-                                                        const Desc* __restrict__ solids, int nnodes, NavArgs a,
-                                                        Vox vox) {
-  constexpr int TILE = 256 * kNavTileItems;
-  __shared__ int scount[kKinds];
-  __shared__ uint16_t sperm[TILE];
-  __shared__ uint8_t skind[TILE];
-  const int t = threadIdx.x;
-  for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {  // block-uniform
-    const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
-    order_tile(nodes, solids, nnodes, a.node + t0, len, vox, scount, skind, sperm);
-    for (int r = t; r < len; r += 256) nav_step64(nodes, children, solids, nnodes, a, t0 + sperm[r], vox);
-    __syncthreads();  // the tile's shared arrays are reused by the next tile
-  }
-}
-
-__global__ void __launch_bounds__(256) k_nav_refine(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                                    const Desc* __restrict__ solids, int nnodes, NavArgs a,
-                                                    const uint32_t* __restrict__ wl,
-                                                    const unsigned long long* __restrict__ cnt, Vox vox) {
-  const int64_t m = (int64_t)*cnt;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  // consecutive entries go to consecutive blocks: a short worklist is spread over every
-  // SM instead of filling the first few blocks (each entry is a long binary64 chain)
-  for (int64_t j = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; j < m; j += stride)
-    nav_step64(nodes, children, solids, nnodes, a, wl[j], vox);
 }
 
 // ------------------------------------------------------------ binary32
@@ -478,6 +579,41 @@ __device__ __forceinline__ void query32(const Desc& S, const f32::TrackF& T, uns
   else if (S.type == kTube) tube32_call(S, T, want, R);
   else if (S.type == kBool) R.flag = true;  // booleans: binary64 only
   else pcon32_call(S, T, want, R);
+}
+
+// The ranking instances of the passes in a placed volume's frame (rank_fp64.cuh).
+__device__ __noinline__ void planar_rank_call(const Desc& S, const f32::TrackF& T, unsigned want, f32::R32& R) {
+  f32::planar32<true, true>(S, T, want, R);
+}
+__device__ __noinline__ void tube_rank_call(const Desc& S, const f32::TrackF& T, unsigned want, f32::R32& R) {
+  f32::pcon32<true, true, true>(S, T, want, R);
+}
+__device__ __noinline__ void pcon_rank_call(const Desc& S, const f32::TrackF& T, unsigned want, f32::R32& R) {
+  f32::pcon32<false, true, true>(S, T, want, R);
+}
+__device__ __forceinline__ void rank_local32(const Desc& S, const f32::TrackF& T, unsigned want, f32::R32& R) {
+  R.flag = T.bad || S.type == kBool || (S.flags & kFp64Only);
+  R.code = 1;
+  R.din = R.dout = R.sin = R.sout = 0.f;
+  R.rank = 0u;
+  R.te = R.se = 0.f;
+  if (R.flag) return;
+  if (S.type == kBox) f32::box32<true, true>(S, T, want, R);
+  else if (S.type == kTrd || S.type == kTrap) planar_rank_call(S, T, want, R);
+  else if (S.type == kTube) tube_rank_call(S, T, want, R);
+  else pcon_rank_call(S, T, want, R);
+}
+__device__ __noinline__ void planar_ranked_call(const Desc& S, const f64::Track& T, f64::Verdict V, f64::Result& R) {
+  f64::planar_ranked(S, T, V, R);
+}
+__device__ __noinline__ void pcon_ranked_call(const Desc& S, const f64::Track& T, f64::Verdict V, f64::Result& R) {
+  f64::pcon_ranked(S, T, V, R);
+}
+__device__ __forceinline__ void ranked_local64(const Desc& S, const f64::Track& T, uint32_t rank, f64::Result& R) {
+  const f64::Verdict V{rank};
+  if (S.type == kBox) f64::box_ranked(S, T, V, R);
+  else if (S.type == kTrd || S.type == kTrap) planar_ranked_call(S, T, V, R);
+  else pcon_ranked_call(S, T, V, R);
 }
 
 // half of the output tolerance: the certified binary32 results are within it
@@ -601,7 +737,9 @@ __global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__
           bool take = all || tag == kCullNever || (want_saf && tag == kCullOther);
           if (!take) {
             const PlainLocal L = plain_local(C, P);
-            take = !plain_miss(C, P, L);
+            float from;
+            bool near;
+            take = !plain_miss(C, P, L, from, near) || near;
             if (want_saf) {
               const float s = plain_safety(C, L), lb = s - L.margin;
               ub = fminf(ub, s < L.margin ? F_INF : s + L.margin);  // a point not outside gives none
@@ -821,80 +959,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
   }
 }
 
-// ------------------------------------------------------------ transport loop
-
-// Locate one point in binary64 (gv_nav_locate's definition: from the world down, enter
-// the first daughter, in index order or in the point's grid cell, that does not classify
-// the point OUTSIDE; -1 outside the world) and report whether any classification on the
-// way was SURFACE (the point lies on a boundary within the tolerance).
-__device__ inline int32_t locate64_surf(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                        const Desc* __restrict__ solids, double x, double y, double z, bool& surf,
-                                        const Vox& vox) {
-  f64::Track T{0, 0, 0, 0, 0, 0};
-  f64::Result R;
-  to_local64(nodes[0], x, y, z, T.x, T.y, T.z);
-  query64(solids[nodes[0].desc], T, f64::kWantCode, R);
-  surf |= R.code == 1;
-  if (R.code == 2) return -1;
-  int32_t v = 0;
-  for (int depth = 0; depth < 64; depth++) {
-    const NodeD& N = nodes[v];
-    int32_t into = -1;
-    const int32_t* ids;
-    int count;
-    candidates64(N, children, vox, x, y, z, ids, count);  // a daughter whose band holds the point is listed
-    for (int j = 0; j < count; j++) {
-      const int32_t c = ids[j];
-      to_local64(nodes[c], x, y, z, T.x, T.y, T.z);
-      query64(solids[nodes[c].desc], T, f64::kWantCode, R);
-      surf |= R.code == 1;
-      if (R.code != 2) { into = c; break; }
-    }
-    if (into < 0) break;
-    v = into;
-  }
-  return v;
-}
-
-// The geometry half of a step for one point in node v (as nav_step64, without the
-// safety), and the next smaller candidate distance.
-__device__ inline void nav_one64(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                 const Desc* __restrict__ solids, int32_t v, const double p[3], const double d[3],
-                                 double& step, int32_t& next, double& second, const Vox& vox) {
-  const NodeD& N = nodes[v];
-  f64::Track T;
-  f64::Result R;
-  to_local64(N, p[0], p[1], p[2], T.x, T.y, T.z);
-  rot_local64(N, d[0], d[1], d[2], T.u, T.v, T.w);
-  query64(solids[N.desc], T, f64::kWantDout, R);
-  double best = R.dout, runner = CUDART_INF;
-  bool have = best >= 0;
-  int32_t who = -1;
-  if (vox.grids && N.grid >= 0) {
-    grid_entries(nodes, solids, N, vox, p, d, best, who, have, runner);
-    step = have ? best : -1.0;
-    next = have ? who : -1;
-    second = runner;
-    return;
-  }
-  for (int j = 0; j < N.count; j++) {
-    const int32_t c = children[N.first + j];
-    const NodeD& C = nodes[c];
-    to_local64(C, p[0], p[1], p[2], T.x, T.y, T.z);
-    rot_local64(C, d[0], d[1], d[2], T.u, T.v, T.w);
-    query64(solids[C.desc], T, f64::kWantDin, R);
-    const double t = R.din;
-    if (t >= 0 && (!have || t < best || (t == best && who == -1))) {
-      if (have && best < runner) runner = best;
-      best = t; who = c; have = true;
-    } else if (t >= 0 && t < runner) {
-      runner = t;
-    }
-  }
-  step = have ? best : -1.0;
-  next = have ? who : -1;
-  second = runner;
-}
+// ------------------------------------------------- binary64 steps, ranked in binary32
 
 // The binary32 track of a binary64 point and direction, split as the bulk pass splits its
 // inputs (world frame: no frame error yet).
@@ -923,61 +988,217 @@ __device__ __forceinline__ f32::TrackF track_from(const double p[3], const doubl
   return T;
 }
 
-// The geometry half of a step as nav_one64 gives it, with the candidates ranked in binary32
-// first: when the binary32 pass certifies the nearest boundary (its interval apart from every
-// other candidate's) and puts the runner-up beyond the near-tie margin, only that candidate
-// is evaluated in binary64.  Its binary64 distance is then the minimum nav_one64 finds (each
-// binary64 value lies in its candidate's interval), and the runner-up's lower bound gives the
-// same near-tie decision.  A node with a grid, a flagged query or a close runner-up goes to
-// nav_one64.
-__device__ __noinline__ void nav_one_rank32(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                      const Desc* __restrict__ solids, int32_t v, const double p[3], const double d[3],
-                                      double& step, int32_t& next, double& second, const Vox& vox) {
-  constexpr int kMother = 0x7ffffffe, kNone = 0x7fffffff;
-  const NodeD& N = nodes[v];
+// The least of several values known within bounds: the best one and the lowest bound of the others.
+struct Least {
+  float lo = kInf32, hi = kInf32, second = kInf32;
+  int32_t who = -2;
+  uint32_t rank = 0u;
+  __device__ __forceinline__ void add(float v, float e, int32_t id, uint32_t r) {
+    const float l = v - fmaf(2.f * f32::U, fabsf(v), e), h = v + fmaf(2.f * f32::U, fabsf(v), e);
+    if (who == -2 || h < hi) {
+      second = fminf(second, lo);
+      lo = l; hi = h; who = id; rank = r;
+    } else {
+      second = fminf(second, l);
+    }
+  }
+};
+
+// The step of nav_exact, bit for bit, with the candidates ranked by certified binary32 intervals:
+// the mother's exit and the entries of the daughters a plain look leaves (Finder).  When the nearest
+// interval is apart from all others by more than the tie margins, that one crossing is evaluated in
+// binary64 (rank_fp64.cuh), and likewise the least safety; anything uncertain goes to nav_exact.
+// Measured (GB300, same bits): step with safety among 1728 daughters, 2^18 tracks, 112 -> 9.9 ms (before:
+// every daughter's safety in binary64, FP64 pipe 81% busy); transport in the nested detector, 2^20 tracks,
+// 32 steps, 56.7 -> 21.3 ms (before: every daughter's entry in binary64).  Now bound by divergence (5 and
+// 12 of 32 lanes) and instruction fetch.
+static __device__ __forceinline__ void nav_ranked(const Geo& g, int32_t v, const double p[3], const double d[3], bool want_saf,
+                                                  Step& out) {
+  const NodeD& N = g.nodes[v];
   const f32::TrackF W = track_from(p, d);
-  bool ok = !W.bad && !(vox.grids && N.grid >= 0);
-  Top2<false> top{F_INF, 0.f, F_INF, 0.f, kNone, kNone};
+  Least near, safe;
+  f32::R32 R;
+  rank_local32(g.solids[N.desc], to_local32(N, W), f32::kWantDout | (want_saf ? f32::kWantSout : 0u), R);
+  bool ok = !R.flag && R.dout >= 0.f;
+  const uint32_t mrank = R.rank;
   if (ok) {
-    f32::R32 R;
-    query32(solids[N.desc], to_local32(N, W), f32::kWantDout, R);
-    ok = !R.flag && R.dout >= 0;
-    if (ok) top.add(R.dout, half_tol(R.dout), kMother);
-    for (int j = 0; ok && j < N.count; j++) {
-      const NodeD& C = nodes[children[N.first + j]];
-      query32(solids[C.desc], to_local32(C, W), f32::kWantDin, R);
-      if (R.flag) ok = false;
-      else if (R.din >= 0) top.add(R.din, half_tol(R.din), j);
+    near.add(R.dout, R.te, -1, mrank);
+    if (want_saf) safe.add(R.sout, R.se, -1, mrank);
+    Finder F(g, N, plain_track(W), p, d);
+    for (int32_t id; (id = F.next(true, (double)near.hi, near.who)) >= 0;) {
+      const NodeD& C = g.nodes[id];
+      rank_local32(g.solids[C.desc], to_local32(C, W), f32::kWantDin, R);
+      if (R.flag) {
+        const Desc& S = g.solids[C.desc];
+        if (!(S.type == kBool || (S.flags & kFp64Only))) { ok = false; break; }
+        f64::Track T;  // no binary32 form: the binary64 value itself
+        f64::Result R64;
+        local64(C, p, d, T);
+        query64(S, T, f64::kWantDin, R64);
+        R.din = (float)R64.din;
+        R.rank = ~0u;
+      }
+      if (R.din >= 0.f) near.add(R.din, R.te, id, R.rank);
     }
-    ok = ok && isfinite(top.b1) && top.b2 - top.e2 > top.b1 + top.e1;
-  }
-  if (ok) {
-    const bool mother = top.w1 == kMother;
-    const NodeD& M = mother ? N : nodes[children[N.first + top.w1]];
-    f64::Track T;
-    f64::Result R;
-    to_local64(M, p[0], p[1], p[2], T.x, T.y, T.z);
-    rot_local64(M, d[0], d[1], d[2], T.u, T.v, T.w);
-    query64(solids[M.desc], T, mother ? f64::kWantDout : f64::kWantDin, R);
-    const double t = mother ? R.dout : R.din;
-    const double lo2 = (double)top.b2 - (double)top.e2;  // the runner-up's lower bound
-    if (t >= 0 && lo2 - t > 2e-9 * (1.0 + t)) {
-      step = t;
-      next = mother ? -1 : children[N.first + top.w1];
-      second = lo2;
-      return;
+    ok = ok && near.second - near.hi > 4e-9f * (1.f + near.hi) && near.hi < f32::BIG;
+    if (ok && want_saf) {
+      Nearest S(g, N, g.cull[v], F.P, false);
+      for (int nv = 0; nv < 2; nv++) {
+        S.restart(nv != 0);
+        for (int32_t id; (id = S.next((double)safe.hi)) >= 0;) {
+          const NodeD& C = g.nodes[id];
+          if (nv == 0) {
+            rank_local32(g.solids[C.desc], to_local32(C, W), f32::kWantSin, R);
+            if (R.flag) { ok = false; break; }
+          } else {
+            f64::Track T;
+            f64::Result R64;
+            local64(C, p, d, T);
+            query64(g.solids[C.desc], T, f64::kWantSin, R64);
+            R.sin = (float)R64.sin;
+            R.se = 0.f;
+          }
+          if (R.sin >= 0.f) safe.add(R.sin, R.se, id, 0u);
+        }
+      }
+      ok = ok && safe.second > safe.hi && S.complete((double)safe.hi);
     }
   }
-  nav_one64(nodes, children, solids, v, p, d, step, next, second, vox);
+  if (!ok) {
+    nav_exact(g, v, p, d, want_saf, out);
+    return;
+  }
+  f64::Track T;
+  f64::Result R64;
+  const NodeD& M = near.who < 0 ? N : g.nodes[near.who];
+  local64(M, p, d, T);
+  if (near.rank == ~0u) query64(g.solids[M.desc], T, f64::kWantDin, R64);
+  else ranked_local64(g.solids[M.desc], T, near.rank, R64);
+  out.step = near.who < 0 ? R64.dout : R64.din;
+  out.next = near.who;
+  out.second = (double)near.second;
+  if (want_saf) {
+    if (safe.who < 0 && near.who < 0) {
+      out.safety = R64.sout;
+    } else {
+      const NodeD& C = safe.who < 0 ? N : g.nodes[safe.who];
+      local64(C, p, d, T);
+      query64(g.solids[C.desc], T, safe.who < 0 ? f64::kWantSout : f64::kWantSin, R64);
+      out.safety = safe.who < 0 ? R64.sout : R64.sin;
+    }
+  }
+}
+
+// One track of the binary64 step.
+__device__ __forceinline__ void nav_track(const Geo& g, const NavArgs& a, int64_t i) {
+  const int32_t v = a.node[i];
+  if (v < 0 || v >= g.nnodes) {
+    a.step[i] = -1.0; a.next[i] = -1;
+    if (a.safety) a.safety[i] = -1.0;
+    return;
+  }
+  const double p[3] = {a.x[i], a.y[i], a.z[i]}, d[3] = {a.u[i], a.v[i], a.w[i]};
+  Step o;
+  nav_ranked(g, v, p, d, a.safety != nullptr, o);
+  a.step[i] = o.step;
+  if (a.safety) a.safety[i] = o.safety;
+  a.next[i] = o.next;
+}
+
+// One thread per track; the block's 256 tracks are taken in order of the kind of volume
+// they are in, so that a warp runs one path through the geometry.
+__global__ void __launch_bounds__(256, 2) k_nav_fp64(Geo g, NavArgs a) {
+  __shared__ int scount[kKinds];
+  __shared__ int sperm[256];
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {  // block-uniform
+    const int64_t i0 = base + threadIdx.x;
+    int kind = kKinds - 1;
+    if (i0 < a.n) {
+      const int32_t v = a.node[i0];
+      kind = (v >= 0 && v < g.nnodes) ? volume_kind(g.nodes, g.solids, v, g.vox) : kKinds - 2;
+    }
+    order_by_kind(kind, blockDim.x, scount, sperm);
+    const int64_t i = base + sperm[threadIdx.x];
+    if (i < a.n) nav_track(g, a, i);
+    __syncthreads();
+  }
+}
+
+// The same in tiles of 256 * kNavTileItems tracks per block iteration: longer runs of one kind, so
+// fewer warps straddle two kinds.  Taken for baskets of at least four tiles per resident block
+// (two per SM), so that the last round of tiles leaves few SMs idle.
+constexpr int kNavTileItems = 4;
+__global__ void __launch_bounds__(256, 2) k_nav_fp64_tiles(Geo g, NavArgs a) {
+  constexpr int TILE = 256 * kNavTileItems;
+  __shared__ int scount[kKinds];
+  __shared__ uint16_t sperm[TILE];
+  __shared__ uint8_t skind[TILE];
+  const int t = threadIdx.x;
+  for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {  // block-uniform
+    const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
+    order_tile(g.nodes, g.solids, g.nnodes, a.node + t0, len, g.vox, scount, skind, sperm);
+    for (int r = t; r < len; r += 256) nav_track(g, a, t0 + sperm[r]);
+    __syncthreads();  // the tile's shared arrays are reused by the next tile
+  }
+}
+
+__global__ void __launch_bounds__(256, 2) k_nav_refine(Geo g, NavArgs a, const uint32_t* __restrict__ wl,
+                                                    const unsigned long long* __restrict__ cnt) {
+  const int64_t m = (int64_t)*cnt;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  // consecutive entries go to consecutive blocks: a short worklist is spread over every
+  // SM instead of filling the first few blocks (each entry is a long binary64 chain)
+  for (int64_t j = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; j < m; j += stride)
+    nav_track(g, a, wl[j]);
+}
+
+// ------------------------------------------------------------ transport loop
+
+// Locate one point in binary64 (gv_nav_locate's definition: from the world down, enter
+// the first daughter, in index order or in the point's grid cell, that does not classify
+// the point OUTSIDE; -1 outside the world) and report whether any classification on the
+// way was SURFACE (the point lies on a boundary within the tolerance).
+static __device__ __noinline__ int32_t locate64_surf(const Geo& g, double x, double y, double z, bool& surf) {
+  const NodeD* nodes = g.nodes;
+  const Desc* solids = g.solids;
+  const double p[3] = {x, y, z}, d0[3] = {0.0, 0.0, 0.0};
+  const PlainTrack P = plain_world(p, d0);
+  f64::Track T{0, 0, 0, 0, 0, 0};
+  f64::Result R;
+  to_local64(nodes[0], x, y, z, T.x, T.y, T.z);
+  query64(solids[nodes[0].desc], T, f64::kWantCode, R);
+  surf |= R.code == 1;
+  if (R.code == 2) return -1;
+  int32_t v = 0;
+  for (int depth = 0; depth < 64; depth++) {
+    const NodeD& N = nodes[v];
+    int32_t into = -1;
+    const int32_t* ids;
+    int count;
+    candidates64(N, g.children, g.vox, x, y, z, ids, count);  // a daughter whose band holds the point is listed
+    for (int j = 0; j < count; j++) {
+      const int32_t c = ids[j];
+      if (plain_outside(g.cull[c], plain_local(g.cull[c], P))) continue;
+      to_local64(nodes[c], x, y, z, T.x, T.y, T.z);
+      query64(solids[nodes[c].desc], T, f64::kWantCode, R);
+      surf |= R.code == 1;
+      if (R.code != 2) { into = c; break; }
+    }
+    if (into < 0) break;
+    v = into;
+  }
+  return v;
 }
 
 // Locate as locate64_surf, with the codes taken in binary32 when every one on the way is
 // certified (a certified code is the binary64 one); otherwise locate64_surf decides.
-__device__ __noinline__ int32_t locate_rank32(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                        const Desc* __restrict__ solids, double x, double y, double z, bool& surf,
-                                        const Vox& vox) {
+__device__ __forceinline__ int32_t locate_rank32(const Geo& g, double x, double y, double z, bool& surf) {
+  const NodeD* nodes = g.nodes;
+  const Desc* solids = g.solids;
   const double p[3] = {x, y, z}, d0[3] = {0.0, 0.0, 0.0};
   const f32::TrackF W = track_from(p, d0);
+  const PlainTrack P = plain_track(W);
   if (!W.bad) {
     bool sf = false;
     f32::R32 R;
@@ -993,9 +1214,11 @@ __device__ __noinline__ int32_t locate_rank32(const NodeD* __restrict__ nodes, c
           int32_t into = -1;
           const int32_t* ids;
           int count;
-          candidates64(N, children, vox, x, y, z, ids, count);
+          if (!candidates32(N, g.cull[v], g.children, g.vox, P, ids, count))
+            candidates64(N, g.children, g.vox, x, y, z, ids, count);
           for (int j = 0; j < count; j++) {
             const int32_t c = ids[j];
+            if (plain_outside(g.cull[c], plain_local(g.cull[c], P))) continue;
             query32(solids[nodes[c].desc], to_local32(nodes[c], W), f32::kWantCode, R);
             if (R.flag) { ok = false; break; }
             sf |= R.code == 1;
@@ -1011,19 +1234,16 @@ __device__ __noinline__ int32_t locate_rank32(const NodeD* __restrict__ nodes, c
       return v;
     }
   }
-  return locate64_surf(nodes, children, solids, x, y, z, surf, vox);
+  return locate64_surf(g, x, y, z, surf);
 }
 
 // Locate with the codes ranked in binary32 first (the same nodes as k_locate).
-__global__ void __launch_bounds__(256, 2) k_locate32(const NodeD* __restrict__ nodes,
-                                                  const int32_t* __restrict__ children,
-                                                  const Desc* __restrict__ solids, const double* __restrict__ x,
-                                                  const double* __restrict__ y, const double* __restrict__ z,
-                                                  int32_t* __restrict__ out, int64_t n, Vox vox) {
+__global__ void __launch_bounds__(256, 2) k_locate32(Geo g, const double* __restrict__ x, const double* __restrict__ y,
+                                                  const double* __restrict__ z, int32_t* __restrict__ out, int64_t n) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     bool surf = false;
-    out[i] = locate_rank32(nodes, children, solids, x[i], y[i], z[i], surf, vox);
+    out[i] = locate_rank32(g, x[i], y[i], z[i], surf);
   }
 }
 
@@ -1034,7 +1254,6 @@ struct TransportArgs {
   const double* sigma_n;                // n sigma of (scatter, absorb) per material, 1/mm
   const double* xi;                     // random numbers, [n][kmax][4], in (0, 1]
   int32_t kmax, nmat, nnodes;
-  int32_t rank32;                       // rank the step's candidates and the codes in binary32
   int8_t* reason;
   int32_t* steps;
   double *xo, *yo, *zo, *path;
@@ -1069,14 +1288,11 @@ __device__ __forceinline__ void flight_begin(const TransportArgs& a, int64_t i, 
 
 // The first half of one step of the loop of the Physics subsection (see gv.h) for track i:
 // the boundary distance, the physics step and, when the process acts first, the process.
-__device__ inline void flight_step(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                   const Desc* __restrict__ solids, const TransportArgs& a, int64_t i, Flight& F,
-                                   const Vox& vox) {
+__device__ inline void flight_step(const Geo& g, const TransportArgs& a, int64_t i, Flight& F) {
   const double* r = a.xi + ((size_t)i * (size_t)a.kmax + (size_t)F.k) * 4;
-  double dgeo, second;
-  int32_t next;
-  if (a.rank32) nav_one_rank32(nodes, children, solids, F.v, F.p, F.d, dgeo, next, second, vox);
-  else nav_one64(nodes, children, solids, F.v, F.p, F.d, dgeo, next, second, vox);
+  Step o;
+  nav_ranked(g, F.v, F.p, F.d, false, o);
+  const double dgeo = o.step, second = o.second;
   const int32_t m = a.material[F.v];
   if (dgeo < 0 || m < 0 || m >= a.nmat) { F.why = GV_LOST; F.live = false; return; }
   const double sig0 = a.sigma_n[2 * m], sig1 = a.sigma_n[2 * m + 1];
@@ -1106,15 +1322,12 @@ __device__ inline void flight_step(const NodeD* __restrict__ nodes, const int32_
 }
 
 // The second half of a step that ended at a boundary: locate the probe point past it.
-__device__ inline void flight_locate(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                     const Desc* __restrict__ solids, const TransportArgs& a, Flight& F,
-                                     const Vox& vox) {
+__device__ inline void flight_locate(const Geo& g, const TransportArgs& a, Flight& F) {
   bool surf = false;
   F.reloc = false;
   const double q0 = xadd(F.p[0], xmul(kPush, F.d[0])), q1 = xadd(F.p[1], xmul(kPush, F.d[1])),
                q2 = xadd(F.p[2], xmul(kPush, F.d[2]));
-  F.v = a.rank32 ? locate_rank32(nodes, children, solids, q0, q1, q2, surf, vox)
-                 : locate64_surf(nodes, children, solids, q0, q1, q2, surf, vox);
+  F.v = locate_rank32(g, q0, q1, q2, surf);
   F.near |= surf;
   if (F.v < 0) { F.why = GV_ESCAPED; F.live = false; return; }
   if (F.k >= a.kmax) F.live = false;  // truncated
@@ -1129,7 +1342,7 @@ __device__ __forceinline__ void flight_end(const TransportArgs& a, int64_t i, co
   a.tie[i] = F.near ? 1 : 0;
 }
 
-// Binary64, in baskets (the paper's scheduler gathers particles that sit in the same kind
+// The ranked binary64 step, in baskets (the paper's scheduler gathers particles that sit in the same kind
 // of volume, so that they run the same code): a block keeps a pool of one track per
 // thread in shared memory and loops: dead slots take the next tracks of the block's range;
 // the live tracks are ordered by the kind of volume they are in (solid type, whether the
@@ -1139,10 +1352,7 @@ __device__ __forceinline__ void flight_end(const TransportArgs& a, int64_t i, co
 // until its range is used up.
 constexpr int kTransportThreads = 512;
 
-__global__ void __launch_bounds__(kTransportThreads) k_transport(const NodeD* __restrict__ nodes,
-                                                                 const int32_t* __restrict__ children,
-                                                                 const Desc* __restrict__ solids, TransportArgs a,
-                                                                 Vox vox) {
+__global__ void __launch_bounds__(kTransportThreads) k_transport(Geo g, TransportArgs a) {
   constexpr int B = kTransportThreads;
   __shared__ double sp[3][B], sd[3][B], slen[B];
   __shared__ int64_t sidx[B];
@@ -1179,7 +1389,7 @@ __global__ void __launch_bounds__(kTransportThreads) k_transport(const NodeD* __
     const bool live = slive[t];
     if (!__syncthreads_or(live ? 1 : ((int64_t)snext < end ? 1 : 0))) break;
     // order the live tracks by volume kind (counting sort; empty slots last)
-    const int kind = live ? volume_kind(nodes, solids, sv[t], vox) : kKinds - 1;
+    const int kind = live ? volume_kind(g.nodes, g.solids, sv[t], g.vox) : kKinds - 1;
     atomicAdd(&scount[kind], 1);
     __syncthreads();
     if (t == 0) {
@@ -1198,7 +1408,7 @@ __global__ void __launch_bounds__(kTransportThreads) k_transport(const NodeD* __
       for (int c = 0; c < 3; c++) { F.p[c] = sp[c][s]; F.d[c] = sd[c][s]; }
       F.len = slen[s]; F.v = sv[s]; F.k = sk[s]; F.why = swhy[s]; F.near = snear[s]; F.live = true; F.reloc = false;
       const int64_t i = sidx[s];
-      flight_step(nodes, children, solids, a, i, F, vox);
+      flight_step(g, a, i, F);
       if (F.live) {
         for (int c = 0; c < 3; c++) { sp[c][s] = F.p[c]; sd[c][s] = F.d[c]; }
         slen[s] = F.len; sv[s] = F.v; sk[s] = F.k; swhy[s] = F.why; snear[s] = F.near; sreloc[s] = F.reloc;
@@ -1225,7 +1435,7 @@ __global__ void __launch_bounds__(kTransportThreads) k_transport(const NodeD* __
       for (int c = 0; c < 3; c++) { F.p[c] = sp[c][s]; F.d[c] = sd[c][s]; }
       F.len = slen[s]; F.v = sv[s]; F.k = sk[s]; F.why = swhy[s]; F.near = snear[s]; F.live = true; F.reloc = true;
       const int64_t i = sidx[s];
-      flight_locate(nodes, children, solids, a, F, vox);
+      flight_locate(g, a, F);
       if (F.live) {
         sv[s] = F.v; snear[s] = F.near;
       } else {
@@ -1233,6 +1443,56 @@ __global__ void __launch_bounds__(kTransportThreads) k_transport(const NodeD* __
         slive[s] = 0;
       }
       sreloc[s] = 0;
+    }
+    __syncthreads();
+  }
+}
+
+// The safety lists of one grid (one block per cell): the daughters' SafetyToIn at the cell's centre
+// in shared memory, then kSafeList times the least of them.
+__global__ void __launch_bounds__(256) k_safe_lists(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
+                                                    const Desc* __restrict__ solids, int node, const GridD* __restrict__ grids,
+                                                    SafeEnt* __restrict__ list, float* __restrict__ cut) {
+  extern __shared__ float val[];
+  __shared__ unsigned long long best[8];
+  const NodeD& N = nodes[node];
+  const GridD& G = grids[N.grid];
+  const int cell = blockIdx.x, i = cell % G.n[0], j = cell / G.n[0] % G.n[1], k = cell / G.n[0] / G.n[1];
+  const double q[3] = {G.lo[0] + (i + 0.5) * G.cell[0], G.lo[1] + (j + 0.5) * G.cell[1], G.lo[2] + (k + 0.5) * G.cell[2]};
+  double p[3];
+  for (int r = 0; r < 3; r++) p[r] = N.R[3 * r] * q[0] + N.R[3 * r + 1] * q[1] + N.R[3 * r + 2] * q[2] + N.t[r];
+  for (int c = threadIdx.x; c < N.count; c += blockDim.x) {
+    const NodeD& C = nodes[children[N.first + c]];
+    f64::Track T{0, 0, 0, 0, 0, 0};
+    f64::Result R;
+    to_local64(C, p[0], p[1], p[2], T.x, T.y, T.z);
+    query64(solids[C.desc], T, f64::kWantCode | f64::kWantSin, R);
+    // below the value by more than the rounding of any centre or frame change
+    val[c] = R.code == 2 ? fmaxf((float)R.sin * (1.f - 1e-5f) - 1e-5f, 0.f) : 0.f;
+  }
+  __syncthreads();
+  const int64_t at = (int64_t)(G.safe + cell) * kSafeList;
+  for (int e = 0; e <= kSafeList; e++) {
+    // values are not negative: their bit patterns order them
+    unsigned long long m = ~0ull;
+    for (int c = threadIdx.x; c < N.count; c += blockDim.x) {
+      const unsigned long long key = (unsigned long long)__float_as_uint(val[c]) << 32 | (unsigned)c;
+      m = key < m ? key : m;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long u = __shfl_xor_sync(0xffffffffu, m, o);
+      m = u < m ? u : m;
+    }
+    if ((threadIdx.x & 31) == 0) best[threadIdx.x >> 5] = m;
+    __syncthreads();
+    for (int w = 0; w < 8; w++) m = best[w] < m ? best[w] : m;
+    const bool none = (unsigned)(m >> 32) == 0x7f800000u || m == ~0ull;  // all taken
+    const int c = (int)(m & 0xffffffffu);
+    if (threadIdx.x == 0) {
+      const float s = none ? F_INF : __uint_as_float((unsigned)(m >> 32));
+      if (e < kSafeList) list[at + e] = none ? SafeEnt{F_INF, -1} : SafeEnt{s, children[N.first + c]};
+      else cut[G.safe + cell] = s;
+      if (!none) val[c] = F_INF;
     }
     __syncthreads();
   }
@@ -1291,7 +1551,11 @@ static void build_grids(gv_geom* g) {
       G.lo[r] = glo[r];
       G.cell[r] = (ghi[r] - glo[r]) / G.n[r];
       G.inv[r] = 1.0 / G.cell[r];
+      G.flo[r] = (float)G.lo[r];
+      G.fcell[r] = (float)G.cell[r];
+      G.finv[r] = (float)G.inv[r];
     }
+    G.safe = -1;
     G.start = (int)(g->cells.size() / 2);
     const int ncell = G.n[0] * G.n[1] * G.n[2];
     std::vector<std::vector<int32_t>> lists(ncell);
@@ -1331,7 +1595,7 @@ static void build_cull(gv_geom* g) {
       C.e[i] = (float)h.ext[i];
       mag += std::fabs(N.t[i]) + h.ext[i];
     }
-    C.margin = (float)(4e-6 * mag);
+    C.margin = (float)(1e-6 + 4e-6 * mag);
     C.solid = N.desc;
     if (h.type == kBool || (h.flags & kFp64Only)) C.tag = kCullNever;
     else if (h.type == kBox) C.tag = kCullBox;
@@ -1402,6 +1666,15 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
   for (const gv_solid* u : uniq) g->solids.push_back(u->h);  // host copies for the grid builder
   build_grids(g);
   build_cull(g);
+  int64_t safe_cells = 0;  // cells with a safety list
+  for (int v = 0; v < nnodes; v++) {
+    if (g->nodes[v].grid < 0) continue;
+    GridD& G = g->grids[g->nodes[v].grid];
+    const int64_t cells = (int64_t)G.n[0] * G.n[1] * G.n[2];
+    if (g->nodes[v].count > kSafeDaughters || cells > kSafeCells || safe_cells + cells > (1 << 24)) continue;
+    G.safe = (int32_t)safe_cells;
+    safe_cells += cells;
+  }
   cudaError_t e = cudaGetDevice(&g->device);
   if (e == cudaSuccess) e = cudaMalloc(&g->d_nodes, sizeof(NodeD) * nnodes);
   if (e == cudaSuccess) e = cudaMalloc(&g->d_children, sizeof(int32_t) * g->children.size());
@@ -1422,6 +1695,18 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
     if (e == cudaSuccess && !g->list.empty())
       e = cudaMemcpy(g->d_list, g->list.data(), sizeof(int32_t) * g->list.size(), cudaMemcpyHostToDevice);
   }
+  if (e == cudaSuccess && safe_cells > 0) {
+    e = cudaMalloc(&g->d_safe, sizeof(SafeEnt) * kSafeList * (size_t)safe_cells);
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_safe_cut, sizeof(float) * (size_t)safe_cells);
+    for (int v = 0; e == cudaSuccess && v < nnodes; v++) {
+      if (g->nodes[v].grid < 0 || g->grids[g->nodes[v].grid].safe < 0) continue;
+      const GridD& G = g->grids[g->nodes[v].grid];
+      k_safe_lists<<<G.n[0] * G.n[1] * G.n[2], 256, sizeof(float) * g->nodes[v].count>>>(
+          g->d_nodes, g->d_children, g->d_solids, v, g->d_grids, g->d_safe, g->d_safe_cut);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  }
   if (e != cudaSuccess) {
     gv_geom_destroy(g);
     return e == cudaErrorMemoryAllocation ? set_error(GV_ERR_OUT_OF_MEMORY, "geom: cudaMalloc failed") : cuda_error(e, "geom upload");
@@ -1439,6 +1724,8 @@ void gv_geom_destroy(gv_geom* g) {
   if (g->d_grids) cudaFree(g->d_grids);
   if (g->d_cells) cudaFree(g->d_cells);
   if (g->d_list) cudaFree(g->d_list);
+  if (g->d_safe) cudaFree(g->d_safe);
+  if (g->d_safe_cut) cudaFree(g->d_safe_cut);
   delete g;
 }
 
@@ -1453,8 +1740,12 @@ int32_t gv_geom_voxel_count(const gv_geom* g) { return g ? (int32_t)g->grids.siz
 int32_t gv_geom_node_count(const gv_geom* g) { return g ? g->nnodes : 0; }
 
 static gv::Vox vox_of(const gv_geom* g) {
-  if (!g->use_vox || !g->d_grids) return gv::Vox{nullptr, nullptr, nullptr};
-  return gv::Vox{g->d_grids, g->d_cells, g->d_list};
+  if (!g->use_vox || !g->d_grids) return gv::Vox{nullptr, nullptr, nullptr, nullptr, nullptr};
+  return gv::Vox{g->d_grids, g->d_cells, g->d_list, g->d_safe, g->d_safe_cut};
+}
+
+static gv::Geo geo_of(const gv_geom* g) {
+  return gv::Geo{g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, vox_of(g)};
 }
 
 gv_status gv_nav_locate(const gv_geom* g, const gv_tracks* t, int32_t* node, void* stream) {
@@ -1464,8 +1755,7 @@ gv_status gv_nav_locate(const gv_geom* g, const gv_tracks* t, int32_t* node, voi
   if (t->n == 0) return GV_OK;
   if (!t->x || !t->y || !t->z || !node) return set_error(GV_ERR_INVALID_ARG, "locate: NULL array");
   int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sm_count() * 8);
-  k_locate32<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(g->d_nodes, g->d_children, g->d_solids, t->x, t->y,
-                                                                   t->z, node, t->n, vox_of(g));
+  k_locate32<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(geo_of(g), t->x, t->y, t->z, node, t->n);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GV_OK : cuda_error(e, "locate launch");
 }
@@ -1489,11 +1779,10 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
     const int64_t tile = 256 * kNavTileItems;
     if (t->n >= (int64_t)sms * 2 * 4 * tile) {
       const int64_t blocks = std::min<int64_t>((t->n + tile - 1) / tile, (int64_t)sms * 2);
-      k_nav_fp64_tiles<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a,
-                                                         vox_of(g));
+      k_nav_fp64_tiles<<<(unsigned)blocks, 256, 0, st>>>(geo_of(g), a);
     } else {
       int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sms * 8);
-      k_nav_fp64<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a, vox_of(g));
+      k_nav_fp64<<<(unsigned)blocks, 256, 0, st>>>(geo_of(g), a);
     }
   } else {
     if (!ws) return set_error(GV_ERR_INVALID_ARG, "nav: GV_FP32_REFINE needs a workspace");
@@ -1512,8 +1801,7 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
       k_nav_scan32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
                                                      ws->idx, ws->counter, vox);
     }
-    k_nav_refine<<<(unsigned)(sms * 2), 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a, ws->idx,
-                                                       ws->counter, vox_of(g));
+    k_nav_refine<<<(unsigned)(sms * 2), 256, 0, st>>>(geo_of(g), a, ws->idx, ws->counter);
   }
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GV_OK : cuda_error(e, "nav launch");
@@ -1536,7 +1824,7 @@ gv_status gv_transport(const gv_geom* g, const gv_tracks* t, const int32_t* node
     if ((uintptr_t)ptrs[i] & 7u) return set_error(GV_ERR_INVALID_ARG, "transport: arrays must be 8-byte aligned");
   if ((uintptr_t)out->z & 7u) return set_error(GV_ERR_INVALID_ARG, "transport: arrays must be 8-byte aligned");
   TransportArgs a{t->x, t->y, t->z, t->dx, t->dy, t->dz, node0, node_material, sigma_n, xi, kmax, nmat, g->nnodes,
-                  prec == GV_FP32_REFINE ? 1 : 0, out->reason, out->steps, out->x, out->y, out->z, out->path, out->last, out->tie, t->n};
+                  out->reason, out->steps, out->x, out->y, out->z, out->path, out->last, out->tie, t->n};
   // Resident blocks only: each block owns a contiguous range of tracks and keeps its pool
   // full from it, so it drains (slots empty while its last tracks finish) once per range.
   static int resident = 0;
@@ -1547,8 +1835,7 @@ gv_status gv_transport(const gv_geom* g, const gv_tracks* t, const int32_t* node
   }
   const int sms = sm_count();
   const int64_t blocks = std::min<int64_t>((t->n + kTransportThreads - 1) / kTransportThreads, (int64_t)sms * resident);
-  k_transport<<<(unsigned)blocks, kTransportThreads, 0, (cudaStream_t)stream>>>(g->d_nodes, g->d_children, g->d_solids, a,
-                                                                                  vox_of(g));
+  k_transport<<<(unsigned)blocks, kTransportThreads, 0, (cudaStream_t)stream>>>(geo_of(g), a);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GV_OK : cuda_error(e, "transport launch");
 }

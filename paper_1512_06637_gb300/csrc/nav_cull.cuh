@@ -20,7 +20,7 @@ enum : int32_t { kCullBox = 0, kCullTube = 1, kCullOther = 2, kCullNever = 3 };
 struct alignas(16) Cull {
   float R[9], t[3];
   float e[3], rmin;  // rmin: inner radius of a full tube
-  float margin;      // 4e-6 (|t|_1 + |e|_1): the placement's share of the margin (mm)
+  float margin;      // 1e-6 + 4e-6 (|t|_1 + |e|_1): the placement's share of the margin (mm)
   int32_t tag, solid, pad;
 };
 
@@ -47,12 +47,14 @@ __device__ __forceinline__ PlainLocal plain_local(const Cull& C, const PlainTrac
 }
 
 // Does the ray certainly miss the bounding box?  The slabs are widened by the margin, so that a
-// ray that meets the box meets the widened one in binary32 too.  A ray nearly parallel to a face
-// or starting on the plane of one is never called a miss: the certified passes leave some of those
-// to binary64, and their answers shall not depend on this look.
-__device__ __forceinline__ bool plain_miss(const Cull& C, const PlainTrack& p, const PlainLocal& L) {
+// ray that meets the box meets the widened one in binary32 too, and not later: `from` is a lower
+// bound of its entry.  `near`: the ray is nearly parallel to a face or starts on the plane of one;
+// the certified binary32 results leave some of those to binary64, and whether they do shall not
+// depend on this look.
+__device__ __forceinline__ bool plain_miss(const Cull& C, const PlainTrack& p, const PlainLocal& L, float& from,
+                                           bool& near) {
   float lo = 0.f, hi = f32::BIG, e[3];
-  bool near = false;
+  near = false;
 #pragma unroll
   for (int i = 0; i < 3; i++) {
     const float d = e[i] = fmaf(C.R[6 + i], p.w, fmaf(C.R[3 + i], p.v, C.R[i] * p.u));
@@ -68,7 +70,13 @@ __device__ __forceinline__ bool plain_miss(const Cull& C, const PlainTrack& p, c
     const float c = L.q[0] * e[1] - L.q[1] * e[0], E = C.e[0] + L.margin, xy = fmaf(e[0], e[0], e[1] * e[1]);
     if (xy > 0.01f && c * c > 1.0001f * E * E * xy) hi = -f32::BIG;
   }
-  return lo > hi && !near;
+  from = lo;
+  return lo > hi;
+}
+
+// Is the point certainly outside the bounding box (its code is OUTSIDE)?
+__device__ __forceinline__ bool plain_outside(const Cull& C, const PlainLocal& L) {
+  return fabsf(L.q[0]) > C.e[0] + L.margin || fabsf(L.q[1]) > C.e[1] + L.margin || fabsf(L.q[2]) > C.e[2] + L.margin;
 }
 
 // The safety (largest constraint value) of a box or a full tube, within the margin.

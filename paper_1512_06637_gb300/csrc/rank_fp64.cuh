@@ -149,6 +149,7 @@ __device__ __forceinline__ void rank32(const Desc& S, const f32::TrackF& T, unsi
   R.code = 1;
   R.din = R.dout = R.sin = R.sout = 0.f;
   R.rank = 0u;
+  R.te = R.se = 0.f;
   if (R.flag) return;
   if (FAMILY == 0) f32::box32<false, true>(S, T, want, R);
   else if (FAMILY == 1) f32::planar32<false, true>(S, T, want, R);

@@ -57,6 +57,7 @@ struct R32 {
   float din, dout, sin, sout;
   bool flag;
   uint32_t rank;  // RANK passes: the verdict for the binary64 evaluation (Verdict)
+  float te, se;   // RANK passes: error bounds of the distance sought and of the safety
 };
 
 // The RANK instances of the passes decide, with the same certified arithmetic, which constraint
@@ -279,6 +280,8 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
     Arg m = arg_none();
     for (int i = 0; i < 3; i++) m.add(g[i].g, g[i].E, i + 1);
     R.rank = (uint32_t)R.code | ver_safety(R.code == 1 ? (uint32_t)kNone : m.sure() ? m.id : (uint32_t)kWhole, 0);
+    R.se = R.code == 1 ? 0.f : si.err();
+    R.te = 0.f;
   }
   if (!(want & (kWantDin | kWantDout))) return;
   Val tn{-BIG, 0.f}, tf{BIG, 0.f};
@@ -355,10 +358,12 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
       if ((want & kWantDout) && !(R.code == 1 && R.dout == 0.f)) {
         R.rank |= ver_dist(af.id, 0);
         R.flag |= !af.sure() || af.id == kNone;
+        R.te = af.e;
       }
     } else if ((want & kWantDin) && R.din < F_INF) {
       R.rank |= ver_dist(an.id, 0);
       R.flag |= !an.sure() || an.id == kNone;
+      R.te = an.e;
     }
   }
 }
@@ -392,6 +397,8 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
     Arg m = arg_none();
     for (int i = 0; i < 5; i++) m.add(g[i].g, g[i].E, i + 1);
     R.rank = (uint32_t)R.code | ver_safety(R.code == 1 ? (uint32_t)kNone : m.sure() ? m.id : (uint32_t)kWhole, 0);
+    R.se = R.code == 1 ? 0.f : si.err();
+    R.te = 0.f;
   }
   if (!(want & (kWantDin | kWantDout))) return;
   Val tn{-BIG, 0.f}, tf{BIG, 0.f};
@@ -489,10 +496,12 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
       if ((want & kWantDout) && !(R.code == 1 && R.dout == 0.f)) {
         R.rank |= ver_dist(af.id, 0);
         R.flag |= !af.sure() || af.id == kNone;
+        R.te = af.e;
       }
     } else if ((want & kWantDin) && R.din < F_INF) {
       R.rank |= ver_dist(an.id, 0);
       R.flag |= !an.sure() || an.id == kNone;
+      R.te = an.e;
     }
   }
 }
@@ -809,7 +818,11 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   const float s = si.s;
   R.code = decide(si, R.flag);
   if (FRAME && near_plane) R.flag = true;
-  if (RANK) R.rank = (uint32_t)R.code;
+  if (RANK) {
+    R.rank = (uint32_t)R.code;
+    R.te = 0.f;
+    R.se = R.code == 1 ? 0.f : si.err();
+  }
 
   if (want & (kWantSin | kWantSout)) {
     R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
@@ -863,7 +876,10 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
         const Val c = closed_df(k0, kind);
         R.sout = -c.v;
         if (!RANK && !certified({fabsf(c.v), c.e})) R.flag = true;
-        if (RANK) R.rank |= ver_safety(kind, k0);
+        if (RANK) {
+          R.rank |= ver_safety(kind, k0);
+          R.se = c.e;
+        }
       } else {
         // SafetyToIn = min over pieces.  Plain binary32 values with their bounds give an
         // upper bound umin on the minimum; only pieces whose lower bound is below it can
@@ -932,6 +948,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
         if (RANK) {
           R.flag |= !m.sure();
           R.rank |= ver_safety(mkind, (int)m.id);
+          R.se = best.e;
         }
       }
     }
@@ -1263,6 +1280,9 @@ __device__ inline void pcon_end(const Walk& W, R32& R) {
   if (RANK) {
     if ((W.need_out || W.need_in) && (u || (W.need_out && !W.answered && R.code == 0))) R.flag = true;
     if (W.answered) R.rank |= W.did;
+    R.te = W.answered ? W.ans.e : 0.f;
+    if (W.need_out) R.dout = W.answered ? unbig(W.ans.v) : 0.f;
+    if (W.need_in) R.din = W.answered ? W.ans.v : F_INF;
     return;
   }
   if (W.need_out) {
