@@ -1,6 +1,8 @@
 // gv_rank_cpu.cpp -- the library's ranked binary64 evaluation (rank_fp64.cuh) compiled for the
-// host, for tests that compare it with the whole binary64 evaluation (gv_cpu.cpp) without a GPU.
+// host, for tests that compare it with the whole binary64 evaluation (gv_cpu.cpp) without a GPU, and
+// the navigation step's plain look at a placed daughter (nav_cull.cuh) likewise.
 #include <cuda_runtime.h>  // the host stand-ins (shim/)
+#include "nav_cull.cuh"
 #include "rank_fp64.cuh"
 
 using namespace gv;
@@ -45,5 +47,37 @@ extern "C" void gvcpu_query_ranked(const void* desc, int64_t n, const double* co
     dout[i] = R.dout;
     sin[i] = R.sin;
     sout[i] = R.sout;
+  }
+}
+
+// The plain look at a box (tag 0), a full tube (1) or another solid (2) with half extents e and inner
+// radius rmin, placed by R (row-major) and t, for n world tracks: out[7 i ..] = miss, from, by, miss of the
+// look without bounds, certainly outside, safety, margin.
+extern "C" void gvcpu_plain_look(int tag, const double* e, double rmin, const double* R, const double* t, int64_t n,
+                                 const double* const* c, float* out) {
+  Cull C;
+  std::memset(&C, 0, sizeof(C));
+  double mag = 0;
+  for (int i = 0; i < 9; i++) C.R[i] = (float)R[i];
+  for (int i = 0; i < 3; i++) {
+    C.t[i] = (float)t[i];
+    C.e[i] = (float)e[i];
+    mag += std::fabs(t[i]) + e[i];
+  }
+  C.rmin = (float)rmin;
+  C.margin = (float)(1e-6 + 4e-6 * mag);
+  C.tag = tag;
+  for (int64_t i = 0; i < n; i++) {
+    const PlainTrack P{(float)c[0][i], (float)c[1][i], (float)c[2][i], (float)c[3][i], (float)c[4][i], (float)c[5][i],
+                       4e-6f * (float)(std::fabs(c[0][i]) + std::fabs(c[1][i]) + std::fabs(c[2][i]))};
+    const PlainLocal L = plain_local(C, P);
+    float* o = out + 7 * i;
+    float from;
+    bool near;
+    o[0] = plain_entry(C, P, L, o[1], o[2]) ? 1.f : 0.f;
+    o[3] = plain_miss(C, P, L, from, near) ? 1.f : 0.f;
+    o[4] = plain_outside(C, L) ? 1.f : 0.f;
+    o[5] = tag <= kCullTube ? plain_safety(C, L) : 0.f;
+    o[6] = L.margin;
   }
 }

@@ -304,11 +304,10 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* tracks, const int32_t* 
  * a track may legitimately differ from another evaluation of the same loop.
  * All arrays are device arrays; node_material has one entry per node (a material index
  * outside [0, nmat) ends the track as GV_LOST); async on `stream`.
- * prec: GV_FP64 evaluates every candidate boundary and every code of the relocation in
- * binary64; GV_FP32_REFINE ranks them in binary32 first and evaluates in binary64 only the
- * nearest boundary when the binary32 pass certifies it (else every candidate), and takes the
- * relocation's codes in binary32 when all are certified (else binary64).  The results are
- * the same bits either way. */
+ * prec: GV_FP64 or GV_FP32_REFINE, the same loop: candidate boundaries are ranked in certified
+ * binary32, the nearest one is evaluated in binary64 (every candidate when the ranking is not
+ * certain), and the relocation's codes are taken in binary32 when all are certified (else
+ * binary64).  The results have the bits of evaluating everything in binary64. */
 enum { GV_ESCAPED = 0, GV_ABSORBED = 1, GV_TRUNCATED = 2, GV_LOST = 3 };
 typedef struct {
   int8_t* reason;

@@ -307,8 +307,8 @@ class Geometry:
     def transport(self, tracks: dict, node0, node_material, sigma_n, xi, kmax: int, out: dict | None = None,
                   stream=None, precision: str = "fp64") -> dict:
         """The transport loop (gv_transport): CUDA tensors; ``node_material`` int32 per node,
-        ``sigma_n`` float64 (nmat, 2), ``xi`` float64 (n, kmax, 4) in (0, 1].  ``precision``
-        "fp32_refine" ranks candidates and codes in binary32 first (same results)."""
+        ``sigma_n`` float64 (nmat, 2), ``xi`` float64 (n, kmax, 4) in (0, 1].  Both
+        values of ``precision`` run the same loop with the same results."""
         import torch
         n = tracks["x"].numel()
         dev = tracks["x"].device

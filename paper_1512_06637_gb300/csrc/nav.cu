@@ -63,7 +63,8 @@ struct SafeEnt {
   int32_t node;
 };
 constexpr int kSafeList = 64;
-// Lists are built for grids of at most these many daughters and cells.
+// Lists are built for grids of at most these many daughters and cells (one evaluation per pair when the
+// geometry is created: 3 M for 1728 daughters).
 constexpr int kSafeDaughters = 8192, kSafeCells = 32768;
 
 // Device pointers of a geometry's grids (grids == nullptr: no grid is used).
@@ -77,9 +78,9 @@ struct Vox {
 
 // Nodes with at least this many daughters get a grid.
 constexpr int kVoxelMin = 16;
-// The binary32 pass walks a node's grid only from this many daughters on: its walk (a
-// binary64 DDA per lane, a group merge per cell) costs more than 8 lanes scanning a few
-// dozen daughters.
+// The steps walk a node's grid, and its cells carry safety lists, only from this many daughters on: a
+// binary64 DDA costs more than a plain look at a few dozen daughters (nested detector, 32 daughters
+// per shell: transport 24.2 ms walking their grids, 14.9 ms scanning them).
 constexpr int kWalk32Min = 128;
 
 constexpr float kInf32 = __builtin_huge_valf();
@@ -282,12 +283,12 @@ struct Finder {
   PlainTrack P;
   const GridD* G;  // nullptr: scan
   Dda D;
-  int at, end;
+  int at, end, cells;  // next daughter and last one of the scan or of the current cell; cells left behind
   bool over;
   __device__ __forceinline__ Finder(const Geo& geo, const NodeD& node, const PlainTrack& plain, const double p[3],
                                     const double d[3])
-      : g(geo), N(node), P(plain), G(nullptr), at(0), end(node.count), over(false) {
-    if (g.vox.grids && N.grid >= 0) {
+      : g(geo), N(node), P(plain), G(nullptr), at(0), end(node.count), cells(0), over(false) {
+    if (g.vox.grids && N.grid >= 0 && N.count >= kWalk32Min) {
       G = g.vox.grids + N.grid;
       double q[3], e[3];
       to_local64(N, p[0], p[1], p[2], q[0], q[1], q[2]);
@@ -300,6 +301,20 @@ struct Finder {
     const int c = D.cell(*G);
     at = g.vox.cells[2 * c];
     end = g.vox.cells[2 * c + 1];
+  }
+  // go on where an earlier Finder of the same track stopped
+  __device__ __forceinline__ void resume(int at0, int cells0) {
+    if (G && !over) {
+      for (; cells < cells0; cells++) D.advance(*G);
+      cell();
+    }
+    at = at0;
+  }
+  // to the next cell of a grid
+  __device__ __forceinline__ void leave_cell() {
+    cells++;
+    over = !D.advance(*G);
+    if (!over) cell();
   }
   // the next daughter (-1: no more) given the best distance so far (`have`) and its node
   __device__ __forceinline__ int32_t next(bool have, double best, int32_t who) {
@@ -315,12 +330,56 @@ struct Finder {
         at++;
         return id;
       }
-      over = !G || !D.advance(*G) || (have && walk_done(D.tenter, best));
-      if (!over) cell();
+      if (G) leave_cell();
+      else over = true;
+      over = over || (G && have && walk_done(D.tenter, best));
     }
     return -1;
   }
 };
+
+// The plain safety of a primitive (signed) in its own frame, and of a boolean.
+static __device__ __noinline__ float plain_prim(const Desc& S, float x, float y, float z) {
+  if (S.type == kBox) return fmaxf(fmaxf(fabsf(x) - S.Dh[0], fabsf(y) - S.Dh[1]), fabsf(z) - S.Dh[2]);
+  if (S.type == kTrd || S.type == kTrap) {
+    float v = fabsf(z) - S.dzh;
+    for (int i = 0; i < 4; i++) v = fmaxf(v, fmaf(S.plh[i][2], z, fmaf(S.plh[i][1], y, S.plh[i][0] * x)) - S.plh[i][3]);
+    return v;
+  }
+  const float r = sqrtf(fmaf(x, x, y * y));
+  float phi = -f32::BIG, best = f32::BIG;
+  if (S.flags & kHasPhi) {
+    const float a = fmaf(S.nsh[0], x, S.nsh[1] * y), b = fmaf(S.neh[0], x, S.neh[1] * y);
+    phi = (S.flags & kPhiWide) ? fminf(a, b) : fmaxf(a, b);
+  }
+  for (int k = 0; k + 1 < S.nz; k++) {
+    float v = fmaxf((r - fmaf(S.oah[k], z, S.obh[k])) * S.ok_[k], fmaxf(S.zh[k] - z, z - S.zh[k + 1]));
+    if ((S.inner >> k) & 1u) v = fmaxf(v, (fmaf(S.iah[k], z, S.ibh[k]) - r) * S.ik_[k]);
+    best = fminf(best, v);
+  }
+  return fmaxf(best, phi);
+}
+static __device__ __noinline__ float plain_other(const Desc& S, float x, float y, float z) {
+  if (S.type != kBool) return plain_prim(S, x, y, z);
+  const double *M = S.bR, *t = S.bt;
+  const float vx = x - (float)t[0], vy = y - (float)t[1], vz = z - (float)t[2];
+  float q[3];
+  for (int i = 0; i < 3; i++) q[i] = fmaf((float)M[6 + i], vz, fmaf((float)M[3 + i], vy, (float)M[i] * vx));
+  const float a = plain_prim(S.parts[0], x, y, z), c = plain_prim(S.parts[1], q[0], q[1], q[2]);
+  return S.bop == kUnion ? fminf(a, c) : S.bop == kIntersection ? fmaxf(a, c) : fmaxf(a, -c);
+}
+
+// The code of a point in a node's solid where plain binary32 can tell it: 2 certainly OUTSIDE, 0
+// certainly INSIDE, else 1.
+__device__ __forceinline__ int plain_code(const Geo& g, int32_t id, const PlainTrack& P) {
+  const Cull& C = g.cull[id];
+  const PlainLocal L = plain_local(C, P);
+  if (plain_outside(C, L)) return 2;
+  if (C.tag == kCullNever) return 1;
+  const float s = C.tag <= kCullTube ? plain_safety(C, L) : plain_other(g.solids[C.solid], L.q[0], L.q[1], L.q[2]);
+  const float m = C.tag <= kCullTube ? L.margin : 3.f * L.margin;
+  return s > m ? 2 : s < -m ? 0 : 1;
+}
 
 // The cell of a grid whose safety list serves a point: the nearest one; its distance from the
 // cell's centre (with margin).
@@ -988,169 +1047,429 @@ __device__ __forceinline__ f32::TrackF track_from(const double p[3], const doubl
   return T;
 }
 
-// The least of several values known within bounds: the best one and the lowest bound of the others.
-struct Least {
-  float lo = kInf32, hi = kInf32, second = kInf32;
-  int32_t who = -2;
-  uint32_t rank = 0u;
-  __device__ __forceinline__ void add(float v, float e, int32_t id, uint32_t r) {
-    const float l = v - fmaf(2.f * f32::U, fabsf(v), e), h = v + fmaf(2.f * f32::U, fabsf(v), e);
-    if (who == -2 || h < hi) {
-      second = fminf(second, lo);
-      lo = l; hi = h; who = id; rank = r;
-    } else {
-      second = fminf(second, l);
-    }
+// The step of nav_exact, bit for bit, for the tracks of a block's pool, with the candidates ranked by
+// certified binary32 intervals.  The block works in phases, every one over all of its tracks, so that
+// its warps run the same code at the same time (the passes of all families together exceed the
+// instruction cache) and the lanes of a warp mostly one family:
+//   gather    each track's candidates: the mother's exit and the daughters a plain look leaves
+//             (Finder), up to kPoolPairs (track, volume) pairs
+//   evaluate  the pairs in order of solid family, one per lane: certified distance and verdict
+//   merge     the nearest interval and the lower bound of the others; tracks with more daughters that
+//             may be nearer gather again
+//   finish    in order of the nearest volume's family: its crossing in binary64 (rank_fp64.cuh)
+// The least safety comes from plain binary32 values with margins; the one or two daughters (and the
+// mother) within reach of the least are evaluated in binary64.  A track whose nearest interval is not
+// apart from the others by more than the tie margins goes to nav_exact.
+// Measured (GB300, same bits as evaluating every candidate in binary64): step with safety among 1728
+// daughters, 2^18 tracks, 112 -> 2.5 ms (every daughter's safety in binary64 kept the FP64 pipe 81% busy;
+// ranking per thread, without phases: 9.9 ms, instruction fetch); transport in the nested detector, 2^20
+// tracks, 32 steps, 56.7 -> 14.9 ms (per thread 21.3 ms).  Bound by latency: one block per SM, 14-20% of the
+// issue slots, 6-18 of 32 lanes.  1024 threads (64 registers) against 512: step 2.5 against 2.8 ms, transport
+// 15.0 against 14.9 ms.
+constexpr int kPoolPairs = 4;
+enum : uint8_t { kSlotIdle = 0, kSlotMore = 1, kSlotRanked = 2, kSlotExact = 3 };
+enum : int { kKeyBox = 0, kKeyPlanar = 1, kKeyTube = 2, kKeyPcon = 3, kKeyNever = 4, kKeyExact = 5, kKeys = 6 };
+
+template <int SLOTS>
+struct StepPool {
+  double p[3][SLOTS], d[3][SLOTS];
+  int32_t v[SLOTS], who[SLOTS];
+  float lo[SLOTS], hi[SLOTS], second[SLOTS];  // nearest candidate's interval, lower bound of the others
+  uint32_t rank[SLOTS], mrank[SLOTS];         // verdicts of the nearest and of the mother
+  float slo[SLOTS], shi[SLOTS];               // the mother's safety
+  float from[SLOTS];                          // no daughter left is entered before
+  int32_t at[SLOTS], cells[SLOTS];            // where its Finder stopped
+  int32_t pid[kPoolPairs * SLOTS];            // pairs: the volume; results: t (NaN: not certain), error, verdict
+  float t[kPoolPairs * SLOTS], e[kPoolPairs * SLOTS];
+  uint32_t prank[kPoolPairs * SLOTS];
+  uint16_t order[kPoolPairs * SLOTS], perm[SLOTS];
+  uint8_t state[SLOTS], np[SLOTS];
+  int cnt[2][8];  // by key, of the two sorts in turn
+  __device__ __forceinline__ void get(int s, double P[3], double D[3]) const {
+    for (int c = 0; c < 3; c++) { P[c] = p[c][s]; D[c] = d[c][s]; }
   }
 };
 
-// The step of nav_exact, bit for bit, with the candidates ranked by certified binary32 intervals:
-// the mother's exit and the entries of the daughters a plain look leaves (Finder).  When the nearest
-// interval is apart from all others by more than the tie margins, that one crossing is evaluated in
-// binary64 (rank_fp64.cuh), and likewise the least safety; anything uncertain goes to nav_exact.
-// Measured (GB300, same bits): step with safety among 1728 daughters, 2^18 tracks, 112 -> 9.9 ms (before:
-// every daughter's safety in binary64, FP64 pipe 81% busy); transport in the nested detector, 2^20 tracks,
-// 32 steps, 56.7 -> 21.3 ms (before: every daughter's entry in binary64).  Now bound by divergence (5 and
-// 12 of 32 lanes) and instruction fetch.
-static __device__ __forceinline__ void nav_ranked(const Geo& g, int32_t v, const double p[3], const double d[3], bool want_saf,
-                                                  Step& out) {
-  const NodeD& N = g.nodes[v];
-  const f32::TrackF W = track_from(p, d);
-  Least near, safe;
-  f32::R32 R;
-  rank_local32(g.solids[N.desc], to_local32(N, W), f32::kWantDout | (want_saf ? f32::kWantSout : 0u), R);
-  bool ok = !R.flag && R.dout >= 0.f;
-  const uint32_t mrank = R.rank;
-  if (ok) {
-    near.add(R.dout, R.te, -1, mrank);
-    if (want_saf) safe.add(R.sout, R.se, -1, mrank);
-    Finder F(g, N, plain_track(W), p, d);
-    for (int32_t id; (id = F.next(true, (double)near.hi, near.who)) >= 0;) {
-      const NodeD& C = g.nodes[id];
-      rank_local32(g.solids[C.desc], to_local32(C, W), f32::kWantDin, R);
-      if (R.flag) {
-        const Desc& S = g.solids[C.desc];
-        if (!(S.type == kBool || (S.flags & kFp64Only))) { ok = false; break; }
-        f64::Track T;  // no binary32 form: the binary64 value itself
-        f64::Result R64;
-        local64(C, p, d, T);
-        query64(S, T, f64::kWantDin, R64);
-        R.din = (float)R64.din;
-        R.rank = ~0u;
-      }
-      if (R.din >= 0.f) near.add(R.din, R.te, id, R.rank);
-    }
-    ok = ok && near.second - near.hi > 4e-9f * (1.f + near.hi) && near.hi < f32::BIG;
-    if (ok && want_saf) {
-      Nearest S(g, N, g.cull[v], F.P, false);
-      for (int nv = 0; nv < 2; nv++) {
-        S.restart(nv != 0);
-        for (int32_t id; (id = S.next((double)safe.hi)) >= 0;) {
-          const NodeD& C = g.nodes[id];
-          if (nv == 0) {
-            rank_local32(g.solids[C.desc], to_local32(C, W), f32::kWantSin, R);
-            if (R.flag) { ok = false; break; }
+__device__ __forceinline__ int pool_key(const Cull& C) {
+  if (C.tag == kCullNever) return kKeyNever;
+  return C.family;
+}
+
+// Exclusive sums of cnt[0..kKeys) (every thread calls it); returns the total.
+__device__ __forceinline__ int key_sums(int* cnt) {
+  __syncthreads();
+  int total = 0;
+  for (int k = 0; k < kKeys; k++) total += cnt[k];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int run = 0;
+    for (int k = 0; k < kKeys; k++) { const int c = cnt[k]; cnt[k] = run; run += c; }
+  }
+  __syncthreads();
+  return total;
+}
+
+// Rank the pool's tracks (state kSlotMore, v valid; the slots perm[0..n)): afterwards every one is
+// kSlotRanked or kSlotExact.  Every thread of the block calls it.
+template <int NT, int SLOTS>
+__device__ __forceinline__ void pool_rank(const Geo& g, StepPool<SLOTS>& Q, int n, bool want_saf) {
+  const int tid = threadIdx.x;
+  bool first = true;
+  while (true) {
+    if (tid < kKeys) Q.cnt[0][tid] = 0;
+    __syncthreads();
+    for (int r = tid; r < n; r += NT) {
+      const int s = Q.perm[r];
+      int k = 0;
+      if (Q.state[s] == kSlotMore) {
+        const int32_t v = Q.v[s];
+        const NodeD& N = g.nodes[v];
+        if (first && g.cull[v].tag == kCullNever) {
+          Q.state[s] = kSlotExact;
+        } else {
+          double p[3], d[3];
+          Q.get(s, p, d);
+          const PlainTrack P = plain_world(p, d);
+          int32_t* pid = Q.pid + kPoolPairs * s;
+          if (first) pid[k++] = v;
+          if (g.vox.grids && N.grid >= 0 && N.count >= kWalk32Min) {
+            Finder F(g, N, P, p, d);
+            if (!first) F.resume(Q.at[s], Q.cells[s]);
+            const double best = first ? 0.0 : (double)Q.hi[s];
+            const int32_t who = first ? -1 : Q.who[s];
+            float from = 0.f;
+            // up to kPoolPairs pairs, and no farther than the cell that brings two daughters
+            while (k < kPoolPairs) {
+              const int32_t id = F.next(!first, best, who);
+              if (id < 0) break;
+              pid[k++] = id;
+              if (F.at >= F.end && k >= 2) {
+                F.leave_cell();
+                if (!F.over) from = (float)F.D.tenter * (1.f - 1e-6f);
+                if (k >= 3) break;
+              }
+            }
+            Q.at[s] = F.at;
+            Q.cells[s] = F.cells;
+            Q.from[s] = F.over ? kInf32 : from;
           } else {
-            f64::Track T;
-            f64::Result R64;
-            local64(C, p, d, T);
-            query64(g.solids[C.desc], T, f64::kWantSin, R64);
-            R.sin = (float)R64.sin;
-            R.se = 0.f;
+            // the three daughters that may be entered first (later rounds: the next three); `by`: one
+            // of those seen is certainly entered by then
+            float f1 = kInf32, f2 = kInf32, f3 = kInf32, f4 = kInf32, by = first ? kInf32 : Q.hi[s];
+            int32_t c1 = -1, c2 = -1, c3 = -1;
+            const float past = first ? -1.f : Q.from[s];
+            const int32_t past_id = first ? -1 : Q.at[s];
+            for (int j = 0; j < N.count; j++) {
+              const int32_t id = g.children[N.first + j];
+              const Cull& C = g.cull[id];
+              float f, u;
+              if (plain_entry(C, P, plain_local(C, P), f, u)) continue;
+              by = fminf(by, u);
+              if (f > by || f < past || (f == past && id <= past_id)) continue;
+              if (f < f1) { f4 = f3; f3 = f2; c3 = c2; f2 = f1; c2 = c1; f1 = f; c1 = id; }
+              else if (f < f2) { f4 = f3; f3 = f2; c3 = c2; f2 = f; c2 = id; }
+              else if (f < f3) { f4 = f3; f3 = f; c3 = id; }
+              else f4 = fminf(f4, f);
+            }
+            float from = kInf32;
+            int32_t last = -1;
+            const float fs[3] = {f1, f2, f3};
+            const int32_t cs[3] = {c1, c2, c3};
+#pragma unroll
+            for (int c = 0; c < 3; c++)
+              if (cs[c] >= 0 && !beyond(fs[c], (double)by)) {
+                pid[k++] = cs[c];
+                from = fs[c];
+                last = cs[c];
+              }
+            const bool rest = c3 >= 0 && last == c3 && !beyond(f4, (double)by) && f4 < kInf32;
+            Q.at[s] = last;
+            Q.from[s] = rest ? from : kInf32;
           }
-          if (R.sin >= 0.f) safe.add(R.sin, R.se, id, 0u);
+          for (int c = 0; c < k; c++) atomicAdd(&Q.cnt[0][pool_key(g.cull[Q.pid[kPoolPairs * s + c]])], 1);
         }
       }
-      ok = ok && safe.second > safe.hi && S.complete((double)safe.hi);
+      Q.np[s] = (uint8_t)k;
+    }
+    const int total = key_sums(Q.cnt[0]);
+    for (int r = tid; r < n; r += NT) {
+      const int s = Q.perm[r];
+      for (int c = 0; c < Q.np[s]; c++) {
+        const int i = kPoolPairs * s + c;
+        Q.order[atomicAdd(&Q.cnt[0][pool_key(g.cull[Q.pid[i]])], 1)] = (uint16_t)i;
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q < total; q += NT) {
+      const int i = Q.order[q], s = i / kPoolPairs;
+      const bool mother = first && i % kPoolPairs == 0;
+      const int32_t id = Q.pid[i];
+      const NodeD& C = g.nodes[id];
+      const Desc& S = g.solids[C.desc];
+      double p[3], d[3];
+      Q.get(s, p, d);
+      if (g.cull[id].tag == kCullNever) {  // no binary32 form: the binary64 value itself
+        f64::Track T;
+        f64::Result R;
+        local64(C, p, d, T);
+        query64(S, T, f64::kWantDin, R);
+        Q.t[i] = (float)R.din;
+        Q.e[i] = 0.f;
+        Q.prank[i] = ~0u;
+      } else {
+        f32::R32 R;
+        rank_local32(S, to_local32(C, track_from(p, d)),
+                     !mother ? f32::kWantDin : want_saf ? f32::kWantDout | f32::kWantSout : f32::kWantDout, R);
+        const float t = mother ? R.dout : R.din;
+        Q.t[i] = R.flag || (mother && t < 0.f) ? CUDART_NAN_F : t;
+        Q.e[i] = fmaf(2.f * f32::U, fabsf(t), R.te);
+        Q.prank[i] = R.rank;
+        if (mother) {
+          const float es = fmaf(2.f * f32::U, fabsf(R.sout), R.se);
+          Q.slo[s] = R.sout - es;
+          Q.shi[s] = R.sout + es;
+        }
+      }
+    }
+    __syncthreads();
+    bool more = false;
+    for (int r = tid; r < n; r += NT) {
+      const int s = Q.perm[r], k = Q.np[s];
+      if (Q.state[s] != kSlotMore) continue;
+      float lo, hi, second;
+      int32_t who;
+      uint32_t rank;
+      int c = 0;
+      if (first) {
+        const int i = kPoolPairs * s;
+        lo = Q.t[i] - Q.e[i]; hi = Q.t[i] + Q.e[i]; second = kInf32;
+        who = -1;
+        rank = Q.mrank[s] = Q.prank[i];
+        c = 1;
+      } else {
+        lo = Q.lo[s]; hi = Q.hi[s]; second = Q.second[s]; who = Q.who[s]; rank = Q.rank[s];
+      }
+      bool ok = !isnan(hi);
+      for (; c < k; c++) {
+        const int i = kPoolPairs * s + c;
+        const float t = Q.t[i], l = t - Q.e[i], h = t + Q.e[i];
+        ok &= !isnan(t);
+        if (!(t >= 0.f)) continue;
+        if (h < hi) {
+          second = fminf(second, lo);
+          lo = l; hi = h; who = Q.pid[i]; rank = Q.prank[i];
+        } else if (Q.pid[i] != who) {
+          second = fminf(second, l);
+        }
+      }
+      Q.lo[s] = lo; Q.hi[s] = hi; Q.second[s] = second; Q.who[s] = who; Q.rank[s] = rank;
+      if (!ok) Q.state[s] = kSlotExact;
+      else if (beyond(Q.from[s], (double)hi) || Q.from[s] == kInf32)
+        Q.state[s] = second - hi > 4e-9f * (1.f + hi) && hi < f32::BIG ? kSlotRanked : kSlotExact;
+      else more = true;
+    }
+    first = false;
+    if (!__syncthreads_or(more)) break;
+  }
+}
+
+// The candidates for a ranked track's least safety: the mother (bit 0 of the result) and up to two
+// daughters j1, j2 (-1: none); false in `ok` when a third one is within reach.
+template <int SLOTS>
+__device__ __forceinline__ bool pool_safety(const Geo& g, const StepPool<SLOTS>& Q, int s, int32_t& j1, int32_t& j2, bool& ok) {
+  const int32_t v = Q.v[s];
+  const NodeD& N = g.nodes[v];
+  double p[3], d[3];
+  Q.get(s, p, d);
+  const PlainTrack P = plain_world(p, d);
+  float ub = Q.shi[s], s1 = kInf32, s2 = kInf32, s3 = kInf32;  // least upper bound; the least lower bounds
+  j1 = j2 = -1;
+  const SafeEnt* list = nullptr;
+  float dist = 0.f, cut = kInf32;
+  int count = N.count;
+  if (g.vox.grids && N.grid >= 0 && g.vox.grids[N.grid].safe >= 0) {
+    const GridD& G = g.vox.grids[N.grid];
+    const int cell = G.safe + safe_cell(G, N, g.cull[v], P, dist);
+    list = g.vox.safe + (int64_t)cell * kSafeList;
+    cut = g.vox.safe_cut[cell];
+    count = kSafeList;
+  }
+  for (int at = 0; at < count; at++) {
+    int32_t id;
+    if (list) {
+      const SafeEnt E = list[at];
+      if (E.node < 0 || E.s - dist > ub) break;
+      id = E.node;
+    } else {
+      id = g.children[N.first + at];
+    }
+    const Cull& C = g.cull[id];
+    const PlainLocal L = plain_local(C, P);
+    float sf, m = L.margin;
+    if (C.tag <= kCullTube) {
+      sf = plain_safety(C, L);
+    } else {
+      sf = plain_other(g.solids[C.solid], L.q[0], L.q[1], L.q[2]);
+      m *= 3.f;  // the walls' and the second component's rounding
+    }
+    if (!(sf < m)) ub = fminf(ub, sf + m);  // a point not certainly outside gives no upper bound
+    const float lb = sf - m;
+    if (lb < s1) {
+      s3 = s2; s2 = s1; j2 = j1; s1 = lb; j1 = id;
+    } else if (lb < s2) {
+      s3 = s2; s2 = lb; j2 = id;
+    } else {
+      s3 = fminf(s3, lb);
     }
   }
-  if (!ok) {
+  ok = s3 > ub && (!list || cut - dist > ub);
+  if (!(s1 <= ub)) j1 = -1;
+  if (!(s2 <= ub)) j2 = -1;
+  return Q.slo[s] <= ub;
+}
+
+// The binary64 step of slot s after pool_rank (and, with want_saf, its safety candidates).
+template <int SLOTS>
+__device__ __forceinline__ void pool_finish(const Geo& g, const StepPool<SLOTS>& Q, int s, bool want_saf, Step& out) {
+  const int32_t v = Q.v[s];
+  double p[3], d[3];
+  Q.get(s, p, d);
+  if (Q.state[s] == kSlotExact) {
     nav_exact(g, v, p, d, want_saf, out);
     return;
   }
+  const int32_t who = Q.who[s];
+  const uint32_t rank = Q.rank[s];
   f64::Track T;
-  f64::Result R64;
-  const NodeD& M = near.who < 0 ? N : g.nodes[near.who];
+  f64::Result R;
+  const NodeD& M = g.nodes[who < 0 ? v : who];
   local64(M, p, d, T);
-  if (near.rank == ~0u) query64(g.solids[M.desc], T, f64::kWantDin, R64);
-  else ranked_local64(g.solids[M.desc], T, near.rank, R64);
-  out.step = near.who < 0 ? R64.dout : R64.din;
-  out.next = near.who;
-  out.second = (double)near.second;
+  if (rank == ~0u) query64(g.solids[M.desc], T, f64::kWantDin, R);
+  else ranked_local64(g.solids[M.desc], T, rank, R);
+  out.step = who < 0 ? R.dout : R.din;
+  out.next = who;
+  out.second = (double)Q.second[s];
   if (want_saf) {
-    if (safe.who < 0 && near.who < 0) {
-      out.safety = R64.sout;
-    } else {
-      const NodeD& C = safe.who < 0 ? N : g.nodes[safe.who];
+    const int32_t j[3] = {Q.np[s] ? v : -1, Q.pid[kPoolPairs * s], Q.pid[kPoolPairs * s + 1]};
+    double saf = CUDART_INF;
+    for (int c = 0; c < 3; c++) {
+      if (j[c] < 0) continue;
+      const NodeD& C = g.nodes[j[c]];
       local64(C, p, d, T);
-      query64(g.solids[C.desc], T, safe.who < 0 ? f64::kWantSout : f64::kWantSin, R64);
-      out.safety = safe.who < 0 ? R64.sout : R64.sin;
+      double val;
+      if (c == 0) {
+        ranked_local64(g.solids[C.desc], T, Q.mrank[s] & ~(7u << 11), R);  // the safety only
+        val = R.sout;
+      } else {
+        query64(g.solids[C.desc], T, f64::kWantSin, R);
+        val = R.sin;
+      }
+      if (val >= 0 && val < saf) saf = val;
     }
+    out.safety = saf < CUDART_INF ? saf : -1.0;
   }
 }
 
-// One track of the binary64 step.
-__device__ __forceinline__ void nav_track(const Geo& g, const NavArgs& a, int64_t i) {
-  const int32_t v = a.node[i];
-  if (v < 0 || v >= g.nnodes) {
-    a.step[i] = -1.0; a.next[i] = -1;
-    if (a.safety) a.safety[i] = -1.0;
-    return;
+// Order the pool's n tracks (perm) by the family of the volume that finishes them, into order[].
+template <int NT, int SLOTS>
+__device__ __forceinline__ void pool_order(const Geo& g, StepPool<SLOTS>& Q, int n) {
+  const int tid = threadIdx.x;
+  auto key = [&](int s) {
+    if (Q.state[s] != kSlotRanked) return (int)kKeyExact;
+    return pool_key(g.cull[Q.who[s] < 0 ? Q.v[s] : Q.who[s]]);
+  };
+  if (tid < kKeys) Q.cnt[1][tid] = 0;
+  __syncthreads();
+  for (int r = tid; r < n; r += NT) atomicAdd(&Q.cnt[1][key(Q.perm[r])], 1);
+  key_sums(Q.cnt[1]);
+  for (int r = tid; r < n; r += NT) {
+    const int s = Q.perm[r];
+    Q.order[atomicAdd(&Q.cnt[1][key(s)], 1)] = (uint16_t)s;
   }
-  const double p[3] = {a.x[i], a.y[i], a.z[i]}, d[3] = {a.u[i], a.v[i], a.w[i]};
-  Step o;
-  nav_ranked(g, v, p, d, a.safety != nullptr, o);
-  a.step[i] = o.step;
-  if (a.safety) a.safety[i] = o.safety;
-  a.next[i] = o.next;
+  __syncthreads();
 }
 
-// One thread per track; the block's 256 tracks are taken in order of the kind of volume
-// they are in, so that a warp runs one path through the geometry.
-__global__ void __launch_bounds__(256, 2) k_nav_fp64(Geo g, NavArgs a) {
+// Order the pool's live slots (live(s)) by volume kind into perm[0..n); returns n.
+template <int NT, int SLOTS, class Live>
+__device__ __forceinline__ int pool_kinds(const Geo& g, StepPool<SLOTS>& Q, int* scount, Live live) {
+  const int tid = threadIdx.x;
+  if (tid < kKinds) scount[tid] = 0;
+  __syncthreads();
+  for (int s = tid; s < SLOTS; s += NT)
+    if (live(s)) atomicAdd(&scount[volume_kind(g.nodes, g.solids, Q.v[s], g.vox)], 1);
+  __syncthreads();
+  int n = 0;
+  for (int k = 0; k < kKinds; k++) n += scount[k];
+  __syncthreads();
+  if (tid == 0) {
+    int run = 0;
+    for (int k = 0; k < kKinds; k++) { const int c = scount[k]; scount[k] = run; run += c; }
+  }
+  __syncthreads();
+  for (int s = tid; s < SLOTS; s += NT)
+    if (live(s)) Q.perm[atomicAdd(&scount[volume_kind(g.nodes, g.solids, Q.v[s], g.vox)], 1)] = (uint16_t)s;
+  __syncthreads();
+  return n;
+}
+
+// The binary64 step of the tracks 0..n-1, or (wl) of the n listed ones, in tiles of at most SLOTS
+// tracks per block, short ones spread over every block.
+constexpr int kNavSlots = 1024, kNavThreads = 1024;
+__global__ void __launch_bounds__(kNavThreads, 1) k_nav_pool(Geo g, NavArgs a, const uint32_t* __restrict__ wl,
+                                                              const unsigned long long* __restrict__ cnt) {
+  extern __shared__ __align__(16) unsigned char pool_bytes[];
+  StepPool<kNavSlots>& Q = *reinterpret_cast<StepPool<kNavSlots>*>(pool_bytes);
   __shared__ int scount[kKinds];
-  __shared__ int sperm[256];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {  // block-uniform
-    const int64_t i0 = base + threadIdx.x;
-    int kind = kKinds - 1;
-    if (i0 < a.n) {
-      const int32_t v = a.node[i0];
-      kind = (v >= 0 && v < g.nnodes) ? volume_kind(g.nodes, g.solids, v, g.vox) : kKinds - 2;
+  const int tid = threadIdx.x;
+  const bool want_saf = a.safety != nullptr;
+  const int64_t total = cnt ? (int64_t)*cnt : a.n;
+  const int64_t share = (total + gridDim.x - 1) / gridDim.x;
+  const int tile = share >= kNavSlots ? kNavSlots : max((int)share, 32);
+  for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < total; t0 += (int64_t)gridDim.x * tile) {
+    const int len = total - t0 < tile ? (int)(total - t0) : tile;
+    for (int s = tid; s < kNavSlots; s += kNavThreads) {
+      Q.state[s] = kSlotIdle;
+      if (s >= len) continue;
+      const int64_t i = wl ? (int64_t)wl[t0 + s] : t0 + s;
+      const int32_t v = a.node[i];
+      if (v < 0 || v >= g.nnodes) {
+        a.step[i] = -1.0; a.next[i] = -1;
+        if (want_saf) a.safety[i] = -1.0;
+        continue;
+      }
+      Q.v[s] = v;
+      Q.p[0][s] = a.x[i]; Q.p[1][s] = a.y[i]; Q.p[2][s] = a.z[i];
+      Q.d[0][s] = a.u[i]; Q.d[1][s] = a.v[i]; Q.d[2][s] = a.w[i];
+      Q.state[s] = kSlotMore;
     }
-    order_by_kind(kind, blockDim.x, scount, sperm);
-    const int64_t i = base + sperm[threadIdx.x];
-    if (i < a.n) nav_track(g, a, i);
     __syncthreads();
+    const int n = pool_kinds<kNavThreads>(g, Q, scount, [&](int s) { return Q.state[s] == kSlotMore; });
+    pool_rank<kNavThreads>(g, Q, n, want_saf);
+    if (want_saf) {
+      for (int r = tid; r < n; r += kNavThreads) {
+        const int s = Q.perm[r];
+        if (Q.state[s] != kSlotRanked) continue;
+        int32_t j1, j2;
+        bool ok;
+        Q.np[s] = pool_safety(g, Q, s, j1, j2, ok) ? 1 : 0;
+        Q.pid[kPoolPairs * s] = j1;
+        Q.pid[kPoolPairs * s + 1] = j2;
+        if (!ok) Q.state[s] = kSlotExact;
+      }
+      __syncthreads();
+    }
+    pool_order<kNavThreads>(g, Q, n);
+    for (int r = tid; r < n; r += kNavThreads) {
+      const int s = Q.order[r];
+      const int64_t i = wl ? (int64_t)wl[t0 + s] : t0 + s;
+      Step o;
+      pool_finish(g, Q, s, want_saf, o);
+      a.step[i] = o.step;
+      if (want_saf) a.safety[i] = o.safety;
+      a.next[i] = o.next;
+    }
+    __syncthreads();  // the pool is reused by the next tile
   }
-}
-
-// The same in tiles of 256 * kNavTileItems tracks per block iteration: longer runs of one kind, so
-// fewer warps straddle two kinds.  Taken for baskets of at least four tiles per resident block
-// (two per SM), so that the last round of tiles leaves few SMs idle.
-constexpr int kNavTileItems = 4;
-__global__ void __launch_bounds__(256, 2) k_nav_fp64_tiles(Geo g, NavArgs a) {
-  constexpr int TILE = 256 * kNavTileItems;
-  __shared__ int scount[kKinds];
-  __shared__ uint16_t sperm[TILE];
-  __shared__ uint8_t skind[TILE];
-  const int t = threadIdx.x;
-  for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {  // block-uniform
-    const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
-    order_tile(g.nodes, g.solids, g.nnodes, a.node + t0, len, g.vox, scount, skind, sperm);
-    for (int r = t; r < len; r += 256) nav_track(g, a, t0 + sperm[r]);
-    __syncthreads();  // the tile's shared arrays are reused by the next tile
-  }
-}
-
-__global__ void __launch_bounds__(256, 2) k_nav_refine(Geo g, NavArgs a, const uint32_t* __restrict__ wl,
-                                                    const unsigned long long* __restrict__ cnt) {
-  const int64_t m = (int64_t)*cnt;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  // consecutive entries go to consecutive blocks: a short worklist is spread over every
-  // SM instead of filling the first few blocks (each entry is a long binary64 chain)
-  for (int64_t j = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; j < m; j += stride)
-    nav_track(g, a, wl[j]);
 }
 
 // ------------------------------------------------------------ transport loop
@@ -1179,7 +1498,7 @@ static __device__ __noinline__ int32_t locate64_surf(const Geo& g, double x, dou
     candidates64(N, g.children, g.vox, x, y, z, ids, count);  // a daughter whose band holds the point is listed
     for (int j = 0; j < count; j++) {
       const int32_t c = ids[j];
-      if (plain_outside(g.cull[c], plain_local(g.cull[c], P))) continue;
+      if (plain_code(g, c, P) == 2) continue;
       to_local64(nodes[c], x, y, z, T.x, T.y, T.z);
       query64(solids[nodes[c].desc], T, f64::kWantCode, R);
       surf |= R.code == 1;
@@ -1202,7 +1521,11 @@ __device__ __forceinline__ int32_t locate_rank32(const Geo& g, double x, double 
   if (!W.bad) {
     bool sf = false;
     f32::R32 R;
-    query32(solids[nodes[0].desc], to_local32(nodes[0], W), f32::kWantCode, R);
+    const int world = plain_code(g, 0, P);
+    if (world == 2) return -1;
+    R.flag = false;
+    R.code = world;
+    if (world == 1) query32(solids[nodes[0].desc], to_local32(nodes[0], W), f32::kWantCode, R);
     bool ok = !R.flag;
     int32_t v = -1;
     if (ok) {
@@ -1218,7 +1541,9 @@ __device__ __forceinline__ int32_t locate_rank32(const Geo& g, double x, double 
             candidates64(N, g.children, g.vox, x, y, z, ids, count);
           for (int j = 0; j < count; j++) {
             const int32_t c = ids[j];
-            if (plain_outside(g.cull[c], plain_local(g.cull[c], P))) continue;
+            const int look = plain_code(g, c, P);
+            if (look == 2) continue;
+            if (look == 0) { into = c; break; }
             query32(solids[nodes[c].desc], to_local32(nodes[c], W), f32::kWantCode, R);
             if (R.flag) { ok = false; break; }
             sf |= R.code == 1;
@@ -1288,10 +1613,8 @@ __device__ __forceinline__ void flight_begin(const TransportArgs& a, int64_t i, 
 
 // The first half of one step of the loop of the Physics subsection (see gv.h) for track i:
 // the boundary distance, the physics step and, when the process acts first, the process.
-__device__ inline void flight_step(const Geo& g, const TransportArgs& a, int64_t i, Flight& F) {
+__device__ inline void flight_step(const TransportArgs& a, int64_t i, const Step& o, Flight& F) {
   const double* r = a.xi + ((size_t)i * (size_t)a.kmax + (size_t)F.k) * 4;
-  Step o;
-  nav_ranked(g, F.v, F.p, F.d, false, o);
   const double dgeo = o.step, second = o.second;
   const int32_t m = a.material[F.v];
   if (dgeo < 0 || m < 0 || m >= a.nmat) { F.why = GV_LOST; F.live = false; return; }
@@ -1342,107 +1665,99 @@ __device__ __forceinline__ void flight_end(const TransportArgs& a, int64_t i, co
   a.tie[i] = F.near ? 1 : 0;
 }
 
-// The ranked binary64 step, in baskets (the paper's scheduler gathers particles that sit in the same kind
-// of volume, so that they run the same code): a block keeps a pool of one track per
-// thread in shared memory and loops: dead slots take the next tracks of the block's range;
-// the live tracks are ordered by the kind of volume they are in (solid type, whether the
-// volume has daughters and a grid), so that each warp steps tracks of one kind and its
-// lanes follow one path through the geometry; every thread then takes one step for the
-// track of its rank.  Tracks take from one to kmax steps; the pool keeps the block busy
-// until its range is used up.
-constexpr int kTransportThreads = 512;
+// The transport loop in baskets (the paper's scheduler gathers particles that sit in the same kind
+// of volume, so that they run the same code): a block keeps a pool of tracks in shared memory and
+// loops: dead slots take the next tracks of the block's range; pool_rank ranks every live track's step
+// and pool_finish evaluates it in binary64; then the process or the boundary takes the track on, and
+// those at a boundary, gathered into the first warps, are located again.  Tracks take from one to kmax
+// steps; the pool keeps the block busy until its range is used up.
+constexpr int kFlightSlots = 1024, kFlightThreads = 512;
+struct FlightPool {
+  StepPool<kFlightSlots> q;
+  double len[kFlightSlots];
+  int64_t idx[kFlightSlots];
+  int32_t k[kFlightSlots];
+  uint8_t why[kFlightSlots], near[kFlightSlots], live[kFlightSlots], reloc[kFlightSlots];
+  unsigned long long next;
+  int scount[kKinds], nreloc;
+};
 
-__global__ void __launch_bounds__(kTransportThreads) k_transport(Geo g, TransportArgs a) {
-  constexpr int B = kTransportThreads;
-  __shared__ double sp[3][B], sd[3][B], slen[B];
-  __shared__ int64_t sidx[B];
-  __shared__ int32_t sv[B], sk[B], swhy[B];
-  __shared__ unsigned char snear[B], slive[B], sreloc[B];
-  __shared__ int sperm[B];
-  __shared__ int scount[kKinds];
-  __shared__ unsigned long long snext;
+__device__ __forceinline__ void flight_load(const FlightPool& P, int s, Flight& F) {
+  P.q.get(s, F.p, F.d);
+  F.len = P.len[s]; F.v = P.q.v[s]; F.k = P.k[s]; F.why = P.why[s]; F.near = P.near[s]; F.live = true; F.reloc = false;
+}
+__device__ __forceinline__ void flight_store(FlightPool& P, int s, const Flight& F) {
+  for (int c = 0; c < 3; c++) { P.q.p[c][s] = F.p[c]; P.q.d[c][s] = F.d[c]; }
+  P.len[s] = F.len; P.q.v[s] = F.v; P.k[s] = F.k; P.why[s] = (uint8_t)F.why; P.near[s] = F.near;
+}
+
+__global__ void __launch_bounds__(kFlightThreads, 1) k_transport(Geo g, TransportArgs a) {
+  extern __shared__ __align__(16) unsigned char pool_bytes[];
+  FlightPool& P = *reinterpret_cast<FlightPool*>(pool_bytes);
   const int t = threadIdx.x;
   const int64_t chunk = (a.n + gridDim.x - 1) / gridDim.x;
   const int64_t begin = (int64_t)blockIdx.x * chunk;
   const int64_t end = begin + chunk < a.n ? begin + chunk : a.n;
-  if (t == 0) snext = (unsigned long long)(begin < end ? begin : end);
-  slive[t] = 0;
+  if (t == 0) P.next = (unsigned long long)(begin < end ? begin : end);
+  for (int s = t; s < kFlightSlots; s += kFlightThreads) P.live[s] = 0;
   __syncthreads();
   while (true) {
     // dead slots take the next tracks of the range
-    if (!slive[t]) {
-      const unsigned long long j = atomicAdd(&snext, 1ull);
-      if ((int64_t)j < end) {
-        Flight F;
-        flight_begin(a, (int64_t)j, F);
-        if (F.live) {
-          for (int c = 0; c < 3; c++) { sp[c][t] = F.p[c]; sd[c][t] = F.d[c]; }
-          slen[t] = F.len; sidx[t] = (int64_t)j; sv[t] = F.v; sk[t] = F.k; swhy[t] = F.why;
-          snear[t] = F.near; slive[t] = 1;
-        } else {
-          flight_end(a, (int64_t)j, F);
+    bool any = false;
+    for (int s = t; s < kFlightSlots; s += kFlightThreads) {
+      if (!P.live[s]) {
+        const unsigned long long j = atomicAdd(&P.next, 1ull);
+        if ((int64_t)j < end) {
+          Flight F;
+          flight_begin(a, (int64_t)j, F);
+          any = true;
+          if (F.live) {
+            P.idx[s] = (int64_t)j;
+            flight_store(P, s, F);
+            P.live[s] = 1;
+          } else {
+            flight_end(a, (int64_t)j, F);
+          }
         }
       }
+      P.q.state[s] = P.live[s] ? kSlotMore : kSlotIdle;
+      any |= P.live[s] != 0;
     }
-    if (t < kKinds) scount[t] = 0;
+    if (!__syncthreads_or(any)) break;
+    const int n = pool_kinds<kFlightThreads>(g, P.q, P.scount, [&](int s) { return P.live[s] != 0; });
+    pool_rank<kFlightThreads>(g, P.q, n, false);
+    pool_order<kFlightThreads>(g, P.q, n);
+    if (t == 0) P.nreloc = 0;
     __syncthreads();
-    const bool live = slive[t];
-    if (!__syncthreads_or(live ? 1 : ((int64_t)snext < end ? 1 : 0))) break;
-    // order the live tracks by volume kind (counting sort; empty slots last)
-    const int kind = live ? volume_kind(g.nodes, g.solids, sv[t], g.vox) : kKinds - 1;
-    atomicAdd(&scount[kind], 1);
-    __syncthreads();
-    if (t == 0) {
-      int acc = 0;
-      for (int k = 0; k < kKinds; k++) { const int c = scount[k]; scount[k] = acc; acc += c; }
-    }
-    __syncthreads();
-    sperm[atomicAdd(&scount[kind], 1)] = t;
-    __syncthreads();
-    // first half of a step for the track of rank t
-    int s = sperm[t];
-    sreloc[t] = 0;
-    __syncthreads();
-    if (slive[s]) {
+    for (int r = t; r < n; r += kFlightThreads) {
+      const int s = P.q.order[r];
+      Step o;
+      pool_finish(g, P.q, s, false, o);
       Flight F;
-      for (int c = 0; c < 3; c++) { F.p[c] = sp[c][s]; F.d[c] = sd[c][s]; }
-      F.len = slen[s]; F.v = sv[s]; F.k = sk[s]; F.why = swhy[s]; F.near = snear[s]; F.live = true; F.reloc = false;
-      const int64_t i = sidx[s];
-      flight_step(g, a, i, F);
+      flight_load(P, s, F);
+      flight_step(a, P.idx[s], o, F);
       if (F.live) {
-        for (int c = 0; c < 3; c++) { sp[c][s] = F.p[c]; sd[c][s] = F.d[c]; }
-        slen[s] = F.len; sv[s] = F.v; sk[s] = F.k; swhy[s] = F.why; snear[s] = F.near; sreloc[s] = F.reloc;
+        flight_store(P, s, F);
+        if (F.reloc) P.q.perm[atomicAdd(&P.nreloc, 1)] = (uint16_t)s;
       } else {
-        flight_end(a, i, F);
-        slive[s] = 0;
+        flight_end(a, P.idx[s], F);
+        P.live[s] = 0;
       }
     }
-    // second half for the tracks at a boundary, gathered into the first warps
-    if (t < 2) scount[t] = 0;
     __syncthreads();
-    const int rk = sreloc[t] ? 0 : 1;
-    if (rk == 0) atomicAdd(&scount[0], 1);
-    __syncthreads();
-    const int nreloc = scount[0];
-    __syncthreads();
-    if (t == 0) { scount[0] = 0; scount[1] = nreloc; }
-    __syncthreads();
-    sperm[atomicAdd(&scount[rk], 1)] = t;
-    __syncthreads();
-    s = sperm[t];
-    if (t < nreloc) {
+    // the tracks at a boundary
+    const int nreloc = P.nreloc;
+    for (int r = t; r < nreloc; r += kFlightThreads) {
+      const int s = P.q.perm[r];
       Flight F;
-      for (int c = 0; c < 3; c++) { F.p[c] = sp[c][s]; F.d[c] = sd[c][s]; }
-      F.len = slen[s]; F.v = sv[s]; F.k = sk[s]; F.why = swhy[s]; F.near = snear[s]; F.live = true; F.reloc = true;
-      const int64_t i = sidx[s];
+      flight_load(P, s, F);
       flight_locate(g, a, F);
       if (F.live) {
-        sv[s] = F.v; snear[s] = F.near;
+        P.q.v[s] = F.v; P.near[s] = F.near;
       } else {
-        flight_end(a, i, F);
-        slive[s] = 0;
+        flight_end(a, P.idx[s], F);
+        P.live[s] = 0;
       }
-      sreloc[s] = 0;
     }
     __syncthreads();
   }
@@ -1597,6 +1912,7 @@ static void build_cull(gv_geom* g) {
     }
     C.margin = (float)(1e-6 + 4e-6 * mag);
     C.solid = N.desc;
+    C.family = h.type == kBox ? 0 : h.type == kTrd || h.type == kTrap ? 1 : h.type == kTube ? 2 : 3;
     if (h.type == kBool || (h.flags & kFp64Only)) C.tag = kCullNever;
     else if (h.type == kBox) C.tag = kCullBox;
     else if (h.type == kTube && !(h.flags & kHasPhi)) C.tag = kCullTube;
@@ -1671,7 +1987,7 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
     if (g->nodes[v].grid < 0) continue;
     GridD& G = g->grids[g->nodes[v].grid];
     const int64_t cells = (int64_t)G.n[0] * G.n[1] * G.n[2];
-    if (g->nodes[v].count > kSafeDaughters || cells > kSafeCells || safe_cells + cells > (1 << 24)) continue;
+    if (g->nodes[v].count < kWalk32Min || g->nodes[v].count > kSafeDaughters || cells > kSafeCells || safe_cells + cells > (1 << 24)) continue;
     G.safe = (int32_t)safe_cells;
     safe_cells += cells;
   }
@@ -1748,6 +2064,15 @@ static gv::Geo geo_of(const gv_geom* g) {
   return gv::Geo{g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, vox_of(g)};
 }
 
+static cudaError_t launch_nav_pool(const gv_geom* g, const gv::NavArgs& a, int64_t blocks, const uint32_t* wl,
+                                   const unsigned long long* cnt, cudaStream_t st) {
+  const int bytes = (int)sizeof(gv::StepPool<gv::kNavSlots>);
+  const cudaError_t e = cudaFuncSetAttribute(gv::k_nav_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  gv::k_nav_pool<<<(unsigned)blocks, gv::kNavThreads, bytes, st>>>(geo_of(g), a, wl, cnt);
+  return cudaGetLastError();
+}
+
 gv_status gv_nav_locate(const gv_geom* g, const gv_tracks* t, int32_t* node, void* stream) {
   const gv::Range range("gv_nav_locate");
   if (!g || !t) return set_error(GV_ERR_INVALID_ARG, "locate: NULL geometry or tracks");
@@ -1776,14 +2101,8 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
   cudaStream_t st = (cudaStream_t)stream;
   const int sms = sm_count();
   if (prec == GV_FP64) {
-    const int64_t tile = 256 * kNavTileItems;
-    if (t->n >= (int64_t)sms * 2 * 4 * tile) {
-      const int64_t blocks = std::min<int64_t>((t->n + tile - 1) / tile, (int64_t)sms * 2);
-      k_nav_fp64_tiles<<<(unsigned)blocks, 256, 0, st>>>(geo_of(g), a);
-    } else {
-      int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sms * 8);
-      k_nav_fp64<<<(unsigned)blocks, 256, 0, st>>>(geo_of(g), a);
-    }
+    const cudaError_t e = launch_nav_pool(g, a, std::min<int64_t>((t->n + 31) / 32, sms), nullptr, nullptr, st);
+    if (e != cudaSuccess) return cuda_error(e, "nav launch");
   } else {
     if (!ws) return set_error(GV_ERR_INVALID_ARG, "nav: GV_FP32_REFINE needs a workspace");
     if (ws->cap < t->n) return set_error(GV_ERR_OUT_OF_MEMORY, "nav: workspace smaller than the basket");
@@ -1801,7 +2120,8 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
       k_nav_scan32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
                                                      ws->idx, ws->counter, vox);
     }
-    k_nav_refine<<<(unsigned)(sms * 2), 256, 0, st>>>(geo_of(g), a, ws->idx, ws->counter);
+    e = launch_nav_pool(g, a, sms, ws->idx, ws->counter, st);
+    if (e != cudaSuccess) return cuda_error(e, "nav launch");
   }
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GV_OK : cuda_error(e, "nav launch");
@@ -1825,17 +2145,14 @@ gv_status gv_transport(const gv_geom* g, const gv_tracks* t, const int32_t* node
   if ((uintptr_t)out->z & 7u) return set_error(GV_ERR_INVALID_ARG, "transport: arrays must be 8-byte aligned");
   TransportArgs a{t->x, t->y, t->z, t->dx, t->dy, t->dz, node0, node_material, sigma_n, xi, kmax, nmat, g->nnodes,
                   out->reason, out->steps, out->x, out->y, out->z, out->path, out->last, out->tie, t->n};
-  // Resident blocks only: each block owns a contiguous range of tracks and keeps its pool
-  // full from it, so it drains (slots empty while its last tracks finish) once per range.
-  static int resident = 0;
-  if (resident == 0) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_transport, kTransportThreads, 0) != cudaSuccess || nb < 1) nb = 1;
-    resident = nb;
-  }
+  // One block per SM: each owns a contiguous range of tracks and keeps its pool full from it, so it
+  // drains (slots empty while its last tracks finish) once per range.
   const int sms = sm_count();
-  const int64_t blocks = std::min<int64_t>((t->n + kTransportThreads - 1) / kTransportThreads, (int64_t)sms * resident);
-  k_transport<<<(unsigned)blocks, kTransportThreads, 0, (cudaStream_t)stream>>>(geo_of(g), a);
+  const int64_t blocks = std::min<int64_t>((t->n + 31) / 32, sms);
+  const int bytes = (int)sizeof(FlightPool);
+  const cudaError_t ea = cudaFuncSetAttribute(k_transport, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (ea != cudaSuccess) return cuda_error(ea, "transport launch");
+  k_transport<<<(unsigned)blocks, kFlightThreads, bytes, (cudaStream_t)stream>>>(geo_of(g), a);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GV_OK : cuda_error(e, "transport launch");
 }

@@ -21,7 +21,8 @@ struct alignas(16) Cull {
   float R[9], t[3];
   float e[3], rmin;  // rmin: inner radius of a full tube
   float margin;      // 1e-6 + 4e-6 (|t|_1 + |e|_1): the placement's share of the margin (mm)
-  int32_t tag, solid, pad;
+  int32_t tag, solid;
+  int32_t family;  // 0 box, 1 trd/trap, 2 tube, 3 cone and polycone
 };
 
 // A track in world coordinates, plain binary32.
@@ -72,6 +73,74 @@ __device__ __forceinline__ bool plain_miss(const Cull& C, const PlainTrack& p, c
   }
   from = lo;
   return lo > hi;
+}
+
+// The times at which the ray q + t e (r2 = |q_xy|^2, b = q_xy e_xy, a = |e_xy|^2) enters and leaves
+// radius R in plain binary32; wide: not later and not earlier than in truth, else the other way round.
+// The discriminant's rounding is below 10 2^-24 a (r2 + R^2); dt is what its bound can move a time by.
+__device__ __forceinline__ bool plain_circle(float r2, float b, float a, float R, bool wide, float& t0, float& t1, float& dt) {
+  const float err = 2e-6f * a * fmaf(R, R, r2);
+  const float disc = fmaf(b, b, -a * fmaf(-R, R, r2)) + (wide ? err : -err);
+  const float s = sqrtf(fmaxf(disc, 0.f)), inv = __fdividef(1.f, a);
+  t0 = (-b - s) * inv;
+  t1 = (-b + s) * inv;
+  dt = err * __fdividef(1.f, s * a);
+  return disc > 0.f;
+}
+
+// The same look with bounds on the entry: not before `from`, and, when it is finite, not after `by`
+// (a ray from a point certainly outside that certainly goes in).  A box is entered where the ray enters
+// the box widened and shrunk by the margin; a full tube through its outer or its inner wall likewise
+// (steep rays and rays through the end planes get no upper bound).
+__device__ __forceinline__ bool plain_entry(const Cull& C, const PlainTrack& p, const PlainLocal& L, float& from,
+                                            float& by) {
+  float lo = 0.f, hi = f32::BIG, e[3], inv[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    const float d = e[i] = fmaf(C.R[6 + i], p.w, fmaf(C.R[3 + i], p.v, C.R[i] * p.u));
+    inv[i] = __fdividef(1.f, d);
+    const float E = C.e[i] + L.margin, a = (-E - L.q[i]) * inv[i], b = (E - L.q[i]) * inv[i];
+    lo = fmaxf(lo, fminf(a, b));
+    hi = fminf(hi, fmaxf(a, b));
+  }
+  from = lo;
+  by = f32::BIG;
+  if (lo > hi) return true;
+  const float m = L.margin;
+  if (C.tag == kCullBox) {
+    float l = -f32::BIG, h = f32::BIG;
+    bool out = false;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const float E = C.e[i] - m, a = (-E - L.q[i]) * inv[i], b = (E - L.q[i]) * inv[i];
+      l = fmaxf(l, fminf(a, b));
+      h = fminf(h, fmaxf(a, b));
+      out |= fabsf(L.q[i]) > C.e[i] + m;
+    }
+    if (out && l <= h && l > 0.f) by = l;
+  } else if (C.tag == kCullTube) {
+    const float r2 = fmaf(L.q[0], L.q[0], L.q[1] * L.q[1]), a = fmaf(e[0], e[0], e[1] * e[1]);
+    const float b = fmaf(L.q[0], e[0], L.q[1] * e[1]);
+    if (a > 0.01f) {
+      const float Ro = C.e[0], Ri = C.rmin, tm = 2.f * m * rsqrtf(a);  // the rounding of a time
+      float t0, t1, dt, in = f32::BIG, dz = 0.f;  // in: certainly between the walls by then
+      if (r2 > (Ro + m) * (Ro + m)) {
+        if (!plain_circle(r2, b, a, Ro + m, true, t0, t1, dt) || t1 + tm < 0.f) return true;
+        from = fmaxf(from, t0 - tm);
+        if (Ro > m && plain_circle(r2, b, a, Ro - m, false, t0, t1, dt) && t0 > tm) {
+          in = t0 + tm;
+          dz = dt;
+        }
+      } else if (Ri > m && r2 < (Ri - m) * (Ri - m)) {
+        if (plain_circle(r2, b, a, Ri - m, false, t0, t1, dt)) from = fmaxf(from, t1 - tm);
+        plain_circle(r2, b, a, Ri + m, true, t0, t1, dt);
+        in = t1 + tm;
+        dz = dt;
+      }
+      if (Ro - Ri > 4.f * m && fabsf(fmaf(in, e[2], L.q[2])) < C.e[2] - 24.f * m - 2.f * dz) by = in;
+    }
+  }
+  return from > hi;
 }
 
 // Is the point certainly outside the bounding box (its code is OUTSIDE)?
