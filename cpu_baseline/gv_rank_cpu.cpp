@@ -9,8 +9,9 @@ using namespace gv;
 
 template <int FAMILY>
 static bool one(const Desc& S, const uint2* const p[6], int64_t i, bool dirs, const f64::Track& T, unsigned want,
-                f64::Result& R) {
+                bool given, f64::Result& R) {
   const f32::TrackF F = f32::load_track<(FAMILY >= 2)>(p[0], p[1], p[2], p[3], p[4], p[5], i, dirs);
+  if (given) return f64::query_given<FAMILY>(S, T, F, want, R);
   f32::R32 r;
   f64::rank32<FAMILY>(S, F, want, r);
   if (r.flag) return false;
@@ -19,8 +20,8 @@ static bool one(const Desc& S, const uint2* const p[6], int64_t i, bool dirs, co
 }
 
 // The requested results of n tracks against a descriptor of gvcpu_build; ranked[i] tells whether
-// track i had a certain verdict (its results are left alone if not).
-extern "C" void gvcpu_query_ranked(const void* desc, int64_t n, const double* const* t, unsigned want, int8_t* ranked,
+// track i had a certain verdict (its results are left alone if not).  given: the code from binary64.
+extern "C" void gvcpu_query_ranked(const void* desc, int64_t n, const double* const* t, unsigned want, int given, int8_t* ranked,
                                    int8_t* inside, double* din, double* dout, double* sin, double* sout) {
   Desc S;
   std::memcpy(&S, desc, sizeof(Desc));
@@ -34,11 +35,11 @@ extern "C" void gvcpu_query_ranked(const void* desc, int64_t n, const double* co
     f64::Result R;
     bool ok = false;
     if (!(S.flags & kFp64Only)) switch (S.type) {
-      case kBox: ok = one<0>(S, p, i, dirs, T, want, R); break;
+      case kBox: ok = one<0>(S, p, i, dirs, T, want, given, R); break;
       case kTrd:
-      case kTrap: ok = one<1>(S, p, i, dirs, T, want, R); break;
-      case kTube: ok = one<2>(S, p, i, dirs, T, want, R); break;
-      default: ok = one<3>(S, p, i, dirs, T, want, R); break;
+      case kTrap: ok = one<1>(S, p, i, dirs, T, want, given, R); break;
+      case kTube: ok = one<2>(S, p, i, dirs, T, want, given, R); break;
+      default: ok = one<3>(S, p, i, dirs, T, want, given, R); break;
     }
     ranked[i] = ok;
     if (!ok) continue;

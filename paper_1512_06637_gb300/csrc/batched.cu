@@ -23,6 +23,7 @@
 #include <string>
 #include <vector>
 #include "gv_internal.h"
+#include "rank_fp64.cuh"
 #include "solid_fp32.cuh"
 #include "solid_fp64.cuh"
 #include "work_class.cuh"
@@ -122,6 +123,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_batched(const Desc* 
   }
 }
 
+// The worklist of one binary32 family: 0 box, 1 trd/trap, 2 tube, 3 polycone, 4 cone.
+template <int FAMILY>
 __global__ void __launch_bounds__(256) k_batched_refine(const Desc* __restrict__ solids, QueryArgs a,
                                                         const unsigned long long* __restrict__ worklist,
                                                         const unsigned long long* __restrict__ wl_count) {
@@ -138,10 +141,12 @@ __global__ void __launch_bounds__(256) k_batched_refine(const Desc* __restrict__
     f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
     if (want & 6u) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
     f64::Result R;
-    if (S.type == kBox) f64::box_query(S, T, want, R);
-    else if (S.type == kTrd || S.type == kTrap) f64::planar_query(S, T, want, R);
-    else if (S.type == kBool) f64::bool_query(S, T, want, R);
-    else f64::pcon_query(S, T, want, R);
+    f64::query_refined<FAMILY>(S, T,
+                               f32::load_track<(FAMILY >= 2)>(
+                                   reinterpret_cast<const uint2*>(a.x), reinterpret_cast<const uint2*>(a.y),
+                                   reinterpret_cast<const uint2*>(a.z), reinterpret_cast<const uint2*>(a.u),
+                                   reinterpret_cast<const uint2*>(a.v), reinterpret_cast<const uint2*>(a.w), i, want & 6u),
+                               want, R);
     if (a.inside) a.inside[i] = (int8_t)R.code;
     if (a.din) a.din[i] = R.din;
     if (a.dout) a.dout[i] = R.dout;
@@ -558,7 +563,12 @@ static gv_status capture(gv_batch* b, const QueryArgs& a, int prec) {
         le = launch_family(f, b->cfg.ctas_per_sm, b->d_solids, b->d_tiles + b->fam_first[f], b->fam_count[f],
                            b->d_next + 1 + f, a, wl, wl_count_ptr(b, f), fs);
       if (le == cudaSuccess && f != kFamBool) {
-        k_batched_refine<<<sm_count() * 2, 256, 0, fs>>>(b->d_solids, a, wl, wl_count_ptr(b, f));
+        const unsigned grid = (unsigned)sm_count() * 2;
+        if (f == kFamBox) k_batched_refine<0><<<grid, 256, 0, fs>>>(b->d_solids, a, wl, wl_count_ptr(b, f));
+        else if (f == kFamPlanar) k_batched_refine<1><<<grid, 256, 0, fs>>>(b->d_solids, a, wl, wl_count_ptr(b, f));
+        else if (f == kFamTube) k_batched_refine<2><<<grid, 256, 0, fs>>>(b->d_solids, a, wl, wl_count_ptr(b, f));
+        else if (f == kFamCone) k_batched_refine<4><<<grid, 256, 0, fs>>>(b->d_solids, a, wl, wl_count_ptr(b, f));
+        else k_batched_refine<3><<<grid, 256, 0, fs>>>(b->d_solids, a, wl, wl_count_ptr(b, f));
         le = cudaGetLastError();
       }
       if (le == cudaSuccess) le = cudaEventRecord(b->join_ev[f], fs);

@@ -5,11 +5,12 @@
 // memory (cp.async) while it computes the current one, splits them into binary32
 // pairs with integer operations; every certified result is written; the indices of
 // the others are appended to a worklist (one atomicAdd per warp after a ballot).
-// Pass 2 (k_refine_fp64): the same binary64 evaluation as the plain FP64 pass,
+// Pass 2 (k_refine_fp64): binary64 results, ranked with the code from binary64 (query_refined),
 // over the worklist only; its length is read on the device, so the two launches
 // need no host round trip.
 #include "gv_debug.cuh"
 #include "gv_internal.h"
+#include "rank_fp64.cuh"
 #include "solid_fp32.cuh"
 #include "solid_fp64.cuh"
 
@@ -232,9 +233,13 @@ __global__ void __launch_bounds__(256) k_refine_fp64(const Desc* __restrict__ de
     f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
     if (want & (f64::kWantDin | f64::kWantDout)) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
     f64::Result R;
-    if (FAMILY == 0) f64::box_query(S, T, want, R);
-    else if (FAMILY == 1) f64::planar_query(S, T, want, R);
-    else f64::pcon_query(S, T, want, R);
+    const bool dirs = want & (f64::kWantDin | f64::kWantDout);
+    f64::query_refined<FAMILY>(S, T,
+                               f32::load_track<(FAMILY >= 2)>(
+                                   reinterpret_cast<const uint2*>(a.x), reinterpret_cast<const uint2*>(a.y),
+                                   reinterpret_cast<const uint2*>(a.z), reinterpret_cast<const uint2*>(a.u),
+                                   reinterpret_cast<const uint2*>(a.v), reinterpret_cast<const uint2*>(a.w), i, dirs),
+                               want, R);
     if (a.inside) a.inside[i] = (int8_t)R.code;
     if (a.din) a.din[i] = R.din;
     if (a.dout) a.dout[i] = R.dout;
@@ -297,7 +302,8 @@ cudaError_t launch_query_fp32(const gv_solid* s, const QueryArgs& a, uint32_t* w
         k_query_walk<3><<<wblocks, kWalkThreads, 0, stream>>>(s->d, a, worklist, counter);
       else
         launch_pass32<3>(s, a, worklist, counter, stream, sms);
-      k_refine_fp64<2><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
+      if (s->h.nz > 2) k_refine_fp64<3><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
+      else k_refine_fp64<4><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
       break;
   }
   return cudaGetLastError();

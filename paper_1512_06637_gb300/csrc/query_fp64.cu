@@ -121,14 +121,17 @@ __global__ void __launch_bounds__(256) k_query_fp64_tiles(const Desc* __restrict
   }
 }
 
+// A track whose ranking left its code open.
 template <int FAMILY>
-static __device__ __noinline__ void query_whole(const Desc& S, const QueryArgs& a, int64_t i, unsigned want) {
+static __device__ __noinline__ void query_open(const Desc& S, const QueryArgs& a, int64_t i, unsigned want) {
   f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
-  if (want & (f64::kWantDin | f64::kWantDout)) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+  const bool dirs = want & (f64::kWantDin | f64::kWantDout);
+  if (dirs) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+  const f32::TrackF F = f32::load_track<(FAMILY >= 2)>(
+      reinterpret_cast<const uint2*>(a.x), reinterpret_cast<const uint2*>(a.y), reinterpret_cast<const uint2*>(a.z),
+      reinterpret_cast<const uint2*>(a.u), reinterpret_cast<const uint2*>(a.v), reinterpret_cast<const uint2*>(a.w), i, dirs);
   f64::Result R;
-  if (FAMILY == 0) f64::box_query(S, T, want, R);
-  else if (FAMILY == 1) f64::planar_query(S, T, want, R);
-  else f64::pcon_query(S, T, want, R);
+  f64::query_refined<FAMILY>(S, T, F, want, R);
   if (a.inside) a.inside[i] = (int8_t)R.code;
   if (a.din) a.din[i] = R.din;
   if (a.dout) a.dout[i] = R.dout;
@@ -140,27 +143,31 @@ static __device__ __noinline__ void query_whole(const Desc& S, const QueryArgs& 
 // ranks its tile's tracks in binary32 (one verdict word per track in shared memory), orders them by
 // the binary64 work their verdict asks for, and evaluates that work in this order, so that the FP64
 // pipe sees full warps.  While one resident block evaluates, others rank: the two halves use
-// different pipes.  A track without a certain verdict goes on the block's list, which is evaluated
-// whole when 256 have gathered and at the end.
-// Measured (GB300, all five queries): cone, 2^20 tracks, 500 -> 180 us; 8-plane polycone, 4 M tracks,
-// 6876 -> 1274 us; tube DistanceToOut, 50021 tracks, 44.6 -> 24.3 us (before: every candidate in
-// binary64, tiles ordered by class).  FP64 warp instructions per 32 tracks: cone 226 -> 42, polycone
-// 859 -> 45; issue 41-45% and FP64 23-46% busy: bound by latency at 24 warps per SM.  Three blocks of
-// 256 threads (80 registers) against two (128): 1274 against 1389 us (polycone).
-constexpr int kWholeFlush = 256;
-template <int FAMILY, int ITEMS>
-__global__ void __launch_bounds__(256, 3) k_query_rank64(const Desc* __restrict__ desc, QueryArgs a) {
+// different pipes.  A track without a certain verdict (its code within about 1e-11 mm of the band's
+// edges) goes on the block's list, which is evaluated when 256 have gathered and at the end: its code in
+// binary64, the rest ranked.
+// Measured (GB300, all five queries): cone, 2^20 tracks, 500 -> 179 us; 8-plane polycone, 4 M tracks,
+// 6876 -> 1274 us in this kernel alone; tube DistanceToOut, 50021 tracks, 44.6 -> 22.5 us (before: every
+// candidate in binary64, tiles ordered by class).  FP64 warp instructions per 32 tracks: cone 226 -> 42,
+// polycone 859 -> 45; issue 41% and FP64 46% busy (cone): bound by latency at 24 warps per SM.  Three
+// blocks of 256 threads (80 registers) against two (128): cone 179 against 186 us; one-row tiles (short
+// baskets) 24.0 against 22.5 us.
+constexpr int kOpenFlush = 256;
+constexpr uint32_t kOpenVerdict = 0xFFFFFFFFu;
+// STORED: the verdicts are read from `stored`, where an earlier launch left them.
+template <int FAMILY, int ITEMS, bool STORED = false>
+__global__ void __launch_bounds__(256, ITEMS == 1 ? 2 : 3) k_query_rank64(const Desc* __restrict__ desc, QueryArgs a, const uint2* stored) {
   constexpr int NT = 256, TILE = NT * ITEMS;
   constexpr uint32_t NC = f64::kRankClasses;
   __shared__ Desc S;
   __shared__ uint32_t ver[TILE];
   __shared__ uint16_t ord[TILE];
-  __shared__ int64_t whole[TILE + kWholeFlush];
-  __shared__ unsigned cnt[NC], nwhole;
+  __shared__ int64_t open[TILE + kOpenFlush];
+  __shared__ unsigned cnt[NC], nopen;
   stage_desc(S, desc);
   const int tid = threadIdx.x;
   const unsigned lane = tid & 31u;
-  if (tid == 0) nwhole = 0u;
+  if (tid == 0) nopen = 0u;
   const unsigned want = (a.inside ? f64::kWantCode : 0u) | (a.din ? f64::kWantDin : 0u) |
                         (a.dout ? f64::kWantDout : 0u) | (a.sin ? f64::kWantSin : 0u) |
                         (a.sout ? f64::kWantSout : 0u);
@@ -174,20 +181,25 @@ __global__ void __launch_bounds__(256, 3) k_query_rank64(const Desc* __restrict_
     __syncthreads();
     for (int j = tid; j < len; j += NT) {
       const int64_t i = t0 + j;
-      const f32::TrackF T = f32::load_track<(FAMILY >= 2)>(X, Y, Z, Ux, Uy, Uz, i, dirs);
-      GV_DCHECK(!dirs || dbg_unit(a.u[i], a.v[i], a.w[i]), kDbgDirection, i);
-      f32::R32 R;
-      f64::rank32<FAMILY>(S, T, want, R);
-      if (R.flag) {
-        ver[j] = 0xFFFFFFFFu;
-        whole[atomicAdd(&nwhole, 1u)] = i;
+      uint32_t V;
+      if constexpr (STORED) {
+        V = stored[i].x;
       } else {
-        ver[j] = R.rank;
-        atomicAdd(&cnt[f64::rank_class<FAMILY>(f64::Verdict{R.rank})], 1u);
+        const f32::TrackF T = f32::load_track<(FAMILY >= 2)>(X, Y, Z, Ux, Uy, Uz, i, dirs);
+        GV_DCHECK(!dirs || dbg_unit(a.u[i], a.v[i], a.w[i]), kDbgDirection, i);
+        f32::R32 R;
+        f64::rank32<FAMILY>(S, T, want, R);
+        V = R.flag ? kOpenVerdict : R.rank;
+      }
+      ver[j] = V;
+      if (V == kOpenVerdict) {
+        open[atomicAdd(&nopen, 1u)] = i;
+      } else {
+        atomicAdd(&cnt[f64::rank_class<FAMILY>(f64::Verdict{V})], 1u);
       }
     }
     __syncthreads();
-    const unsigned gathered = nwhole;
+    const unsigned gathered = nopen;
     unsigned ranked = 0;
     if (tid < 32) {  // exclusive sums of the class counts
       const unsigned c = lane < NC ? cnt[lane] : 0u;
@@ -201,7 +213,7 @@ __global__ void __launch_bounds__(256, 3) k_query_rank64(const Desc* __restrict_
     }
     __syncthreads();
     for (int j = tid; j < len; j += NT)
-      if (ver[j] != 0xFFFFFFFFu) ord[atomicAdd(&cnt[f64::rank_class<FAMILY>(f64::Verdict{ver[j]})], 1u)] = (uint16_t)j;
+      if (ver[j] != kOpenVerdict) ord[atomicAdd(&cnt[f64::rank_class<FAMILY>(f64::Verdict{ver[j]})], 1u)] = (uint16_t)j;
     __syncthreads();
     ranked = cnt[NC - 1];
     for (unsigned p = tid; p < ranked; p += NT) {
@@ -217,15 +229,111 @@ __global__ void __launch_bounds__(256, 3) k_query_rank64(const Desc* __restrict_
       if (a.sin) a.sin[i] = R.sin;
       if (a.sout) a.sout[i] = R.sout;
     }
-    if (gathered >= (unsigned)kWholeFlush) {
-      for (unsigned q = tid; q < gathered; q += NT) query_whole<FAMILY>(S, a, whole[q], want);
+    if (gathered >= (unsigned)kOpenFlush) {
+      for (unsigned q = tid; q < gathered; q += NT) query_open<FAMILY>(S, a, open[q], want);
       __syncthreads();
-      if (tid == 0) nwhole = 0u;
+      if (tid == 0) nopen = 0u;
     }
     __syncthreads();  // the tile's shared arrays are reused by the next tile
   }
   __syncthreads();
-  for (unsigned q = tid; q < nwhole; q += NT) query_whole<FAMILY>(S, a, whole[q], want);
+  for (unsigned q = tid; q < nopen; q += NT) query_open<FAMILY>(S, a, open[q], want);
+}
+
+// The ranking of multi-section polycones on its own, with lane refill as in the binary32 pass
+// (k_query_walk): a warp keeps one track per lane and refills idle lanes from its rows of 32 tracks (the
+// warps take rows in turn).  The verdict of track i is left in the low word of out[i].
+// Measured (8-plane polycone, 4 M tracks): 957 us with the evaluation, against 1274 us ranking a tile's
+// tracks in place, where a warp walks as long as its longest track (12.2 against 13.8 lanes, barriers).
+// Below 2^18 tracks the second launch and its traffic cost more than that.  Blocks of 256 x 3: 976 us,
+// 384 x 2: 962 us.
+constexpr int64_t kRankWalkMin = 1 << 18;
+constexpr int kRankWalkThreads = 320, kRankWalkBlocks = 2;
+__global__ void __launch_bounds__(kRankWalkThreads, kRankWalkBlocks) k_rank_walk(const Desc* __restrict__ desc, QueryArgs a,
+                                                                                 uint2* out) {
+  __shared__ Desc S;
+  stage_desc(S, desc);
+  __syncthreads();
+  const unsigned want = (a.inside ? f64::kWantCode : 0u) | (a.din ? f64::kWantDin : 0u) |
+                        (a.dout ? f64::kWantDout : 0u) | (a.sin ? f64::kWantSin : 0u) |
+                        (a.sout ? f64::kWantSout : 0u);
+  const uint2 *X = reinterpret_cast<const uint2*>(a.x), *Y = reinterpret_cast<const uint2*>(a.y),
+              *Z = reinterpret_cast<const uint2*>(a.z), *Ux = reinterpret_cast<const uint2*>(a.u),
+              *Uy = reinterpret_cast<const uint2*>(a.v), *Uz = reinterpret_cast<const uint2*>(a.w);
+  const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+  const int64_t W = (int64_t)gridDim.x * (kRankWalkThreads / 32);
+  const int64_t w = (int64_t)blockIdx.x * (kRankWalkThreads / 32) + (threadIdx.x >> 5);
+  int64_t next = 0;  // next position in the warp's rows (warp-uniform)
+  bool busy = false, more = w * 32 < a.n;
+  int64_t i = 0;
+  f32::TrackF T;
+  f32::R32 R;
+  f32::Walk K;
+  while (true) {
+    const unsigned idle = __ballot_sync(0xffffffffu, !busy);
+    if (more && (__popc(idle) >= 16 || idle == 0xffffffffu)) {
+      const int64_t seq = next + __popc(idle & below);
+      const int64_t j = ((seq >> 5) * W + w) * 32 + (seq & 31);
+      next += __popc(idle);
+      more = ((next >> 5) * W + w) * 32 < a.n;
+      if (!busy && j < a.n) {
+        i = j;
+        T = f32::load_track<true>(X, Y, Z, Ux, Uy, Uz, i, true);
+        GV_DCHECK(dbg_unit(a.u[i], a.v[i], a.w[i]), kDbgDirection, i);
+        R.flag = T.bad;
+        R.rank = 0u;
+        R.code = 1;
+        R.din = R.dout = R.sin = R.sout = 0.f;
+        R.te = R.se = 0.f;
+        K.need_in = K.need_out = K.answered = K.live = false;
+        if (!R.flag) busy = f32::pcon_begin<false, false, true>(S, T, want, R, K);
+        if (!busy) out[i] = make_uint2(R.flag ? kOpenVerdict : R.rank, 0u);
+      }
+    }
+    if (__ballot_sync(0xffffffffu, busy) == 0u) {
+      if (!more) break;
+      continue;
+    }
+    if (busy) {
+      f32::pcon_step<false, false, true>(S, T, K);
+      if (!K.live) {
+        f32::pcon_end<true>(K, R);
+        out[i] = make_uint2(R.flag ? kOpenVerdict : R.rank, 0u);
+        busy = false;
+      }
+    }
+  }
+}
+
+// Multi-section polycones in two launches: the walk leaves its verdicts in a distance result that the
+// second launch overwrites.  Not when that array overlaps one that is read (an in-place call): the
+// one-launch pass reads and writes each track in turn.
+static bool overlaps(const void* p, const void* q, int64_t n) {
+  const char *a = static_cast<const char*>(p), *b = static_cast<const char*>(q);
+  return a < b + 8 * n && b < a + 8 * n;
+}
+static double* verdict_array(const QueryArgs& a) {
+  double* out = a.dout ? a.dout : a.din;
+  const double* in[6] = {a.x, a.y, a.z, a.u, a.v, a.w};
+  for (const double* p : in)
+    if (overlaps(out, p, a.n)) return nullptr;
+  const double* other[4] = {a.din, a.dout, a.sin, a.sout};
+  for (const double* p : other)
+    if (p && p != out && overlaps(out, p, a.n)) return nullptr;
+  if (a.inside && overlaps(out, a.inside, a.n)) return nullptr;
+  return out;
+}
+
+template <int ITEMS>
+static void launch_rank_stored(const gv_solid* s, const QueryArgs& a, const uint2* ver, int64_t cap, cudaStream_t stream) {
+  const int64_t tiles = (a.n + 256 * ITEMS - 1) / (256 * ITEMS);
+  k_query_rank64<3, ITEMS, true><<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, stream>>>(s->d, a, ver);
+}
+static void launch_rank_walk(const gv_solid* s, const QueryArgs& a, double* out, int sms, cudaStream_t stream) {
+  const int64_t blocks = (a.n + kRankWalkThreads - 1) / kRankWalkThreads, cap = (int64_t)sms * kRankWalkBlocks;
+  uint2* ver = reinterpret_cast<uint2*>(out);
+  k_rank_walk<<<(unsigned)(blocks < cap ? blocks : cap), kRankWalkThreads, 0, stream>>>(s->d, a, ver);
+  launch_rank_stored<4>(s, a, ver, (int64_t)sms * 3, stream);
 }
 
 template <int FAMILY, int ITEMS>
@@ -240,7 +348,7 @@ static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaSt
   }();
   const int64_t tiles = (a.n + 256 * ITEMS - 1) / (256 * ITEMS);
   const int64_t cap = (int64_t)sms * occ;
-  k_query_rank64<FAMILY, ITEMS><<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, stream>>>(s->d, a);
+  k_query_rank64<FAMILY, ITEMS><<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, stream>>>(s->d, a, nullptr);
 }
 
 // Tiles of 2048 tracks when every resident block gets four of them, of 1024 when it gets one, else of
@@ -276,7 +384,12 @@ cudaError_t launch_query_fp64(const gv_solid* s, const QueryArgs& a, cudaStream_
       case kTrd:
       case kTrap: launch_rank64<1>(s, a, sms, stream); break;
       case kTube: launch_rank64<2>(s, a, sms, stream); break;
-      default: launch_rank64<3>(s, a, sms, stream); break;
+      default:
+        if (double* out = s->h.nz > 2 && (a.din || a.dout) && a.n >= kRankWalkMin ? verdict_array(a) : nullptr)
+          launch_rank_walk(s, a, out, sms, stream);
+        else if (s->h.nz > 2) launch_rank64<3>(s, a, sms, stream);
+        else launch_rank64<4>(s, a, sms, stream);
+        break;
     }
     return cudaGetLastError();
   }

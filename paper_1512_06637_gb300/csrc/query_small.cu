@@ -1,6 +1,7 @@
 // query_small.cu -- the binary32 pass for small baskets in one launch.
 #include "gv_debug.cuh"
 #include "gv_internal.h"
+#include "rank_fp64.cuh"
 #include "solid_fp32.cuh"
 #include "solid_fp64.cuh"
 
@@ -60,9 +61,8 @@ __global__ void __launch_bounds__(256) k_query_fused(const Desc* __restrict__ de
       f64::Track T64{a.x[i], a.y[i], a.z[i], 0, 0, 0};
       if (dirs) { T64.u = a.u[i]; T64.v = a.v[i]; T64.w = a.w[i]; }
       f64::Result R64;
-      if (FAMILY == 0) f64::box_query(S, T64, w64, R64);
-      else if (FAMILY == 1) f64::planar_query(S, T64, w64, R64);
-      else f64::pcon_query(S, T64, w64, R64);
+      if constexpr (FAMILY == 3) f64::query_refined<FAMILY>(S, T64, T, w64, R64);
+      else f64::query_whole<FAMILY>(S, T64, w64, R64);
       if (a.inside) a.inside[i] = (int8_t)R64.code;
       if (a.din) a.din[i] = R64.din;
       if (a.dout) a.dout[i] = R64.dout;
@@ -88,7 +88,10 @@ bool launch_query_small(const gv_solid* s, const QueryArgs& a, uint32_t* slots, 
     case kTrd:
     case kTrap: k_query_fused<1><<<blocks, 256, 0, stream>>>(s->d, a, slots); break;
     case kTube: k_query_fused<2><<<blocks, 256, 0, stream>>>(s->d, a, slots); break;
-    default: k_query_fused<3><<<blocks, 256, 0, stream>>>(s->d, a, slots); break;
+    default:
+      if (s->h.nz > 2) k_query_fused<3><<<blocks, 256, 0, stream>>>(s->d, a, slots);
+      else k_query_fused<4><<<blocks, 256, 0, stream>>>(s->d, a, slots);
+      break;
   }
   if (fused_blocks) *fused_blocks = (int)blocks;
   return true;

@@ -71,6 +71,8 @@ struct R32 {
 //   bit 19     the distance sought is DistanceToOut (else DistanceToIn)
 // Box: constraint and crossing 1-3, the axis; trd/trap: 1-4 the side plane, 5 the z slab;
 // polycone family: the names below.  A track whose verdict is not certain has R32::flag set.
+// The GIVEN instances take the code from R32::code on entry (from binary64, for tracks whose code
+// binary32 cannot certify) and decide the rest.
 enum : uint32_t { kNone = 0, kOuter = 1, kInner = 2, kZLow = 3, kZHigh = 4, kPhiS = 5, kPhiE = 6, kWhole = 7 };
 constexpr uint32_t kVerGoalOut = 1u << 19;
 __device__ __forceinline__ uint32_t ver_safety(uint32_t kind, int k) { return kind << 3 | (uint32_t)k << 6; }
@@ -234,6 +236,17 @@ __device__ __forceinline__ int decide(const SInt& S, bool& flag) {
 // Constraint value with its bound.
 struct Gv { float g, E; };
 
+// GIVEN: a surface point's constraint that is too close to the band's edge -h to tell is within the
+// band if no other one is (the largest constraint of a surface point is).
+struct Band {
+  int in = 0, edge = 0;
+  __device__ __forceinline__ void add(float g, float E) {
+    if (fabsf(g + HF) <= E) edge++;
+    else if (g >= -HF) in++;
+  }
+  __device__ __forceinline__ bool resolved() const { return in == 0 && edge == 1; }
+};
+
 // |p| - D from split values (the low part may have either sign: |p| = |ph| + sign(ph) pl)
 __device__ __forceinline__ Gv abs_minus(float ph, float pl, float Dh, float Dl, float fl) {
   const float a = fabsf(ph);
@@ -262,7 +275,7 @@ __device__ __forceinline__ Gv plane_g(const float* nh, const float* nl, float ch
 // the near face the slab is entered at -b and left at -a, otherwise entered at a
 // and left at b.  DistanceToOut = min exit, DistanceToIn = max entry when it comes
 // before the min exit.
-template <bool FRAME = false, bool RANK = false>
+template <bool FRAME = false, bool RANK = false, bool GIVEN = false>
 __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   const float ph[3] = {T.xh, T.yh, T.zh}, pl[3] = {T.xl, T.yl, T.zl}, d[3] = {T.u, T.v, T.w};
   Gv g[3];
@@ -272,7 +285,14 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
     si.add(g[i].g, g[i].E);
   }
   const float s = si.s;
-  R.code = decide(si, R.flag);
+  bool edge = false;  // GIVEN: a constraint at the band's edge is within the band
+  if (GIVEN) {
+    Band m;
+    for (int i = 0; i < 3; i++) m.add(g[i].g, g[i].E);
+    edge = R.code == 1 && m.resolved();
+  } else {
+    R.code = decide(si, R.flag);
+  }
   R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
   R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
   if (!RANK && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
@@ -310,14 +330,15 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
       }
     }
     // surface start: constraints within the band
-    if (g[i].g >= -HF) {
+    const bool at_edge = fabsf(g[i].g + HF) <= g[i].E;
+    if (g[i].g >= -HF || (GIVEN && edge && at_edge)) {
       const float gd = ph[i] < 0 ? -d[i] : d[i];
       any_out |= gd > 0;
       all_in &= gd < 0;
     }
     // along or nearly along the face plane: sliding is decided in binary64
     if (fabsf(d[i]) <= TAUF + (FRAME ? 4.f * T.dfl : 0.f) && fabsf(g[i].g) <= HF + g[i].E) R.flag = true;
-    if (R.code == 1 && fabsf(g[i].g + HF) <= g[i].E) R.flag = true;
+    if (R.code == 1 && at_edge && !(GIVEN && edge)) R.flag = true;
   }
   if (want & kWantDout) {
     if (R.code == 2) R.dout = -1.f;
@@ -373,7 +394,7 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
 // One uniform path as for the box: every side plane gives one crossing
 // t = -g / (n.d), an entry when n.d < 0 and an exit when n.d > 0; the z slab
 // gives its two crossings like a box axis.
-template <bool FRAME = false, bool RANK = false>
+template <bool FRAME = false, bool RANK = false, bool GIVEN = false>
 __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   Gv g[5];
   float gd[5], egd[5];
@@ -389,7 +410,14 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
   SInt si = sint();
   for (int i = 0; i < 5; i++) si.add(g[i].g, g[i].E);
   const float s = si.s;
-  R.code = decide(si, R.flag);
+  bool edge = false;  // GIVEN: a constraint at the band's edge is within the band
+  if (GIVEN) {
+    Band m;
+    for (int i = 0; i < 5; i++) m.add(g[i].g, g[i].E);
+    edge = R.code == 1 && m.resolved();
+  } else {
+    R.code = decide(si, R.flag);
+  }
   R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
   R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
   if (!RANK && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
@@ -448,12 +476,13 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
     }
   }
   for (int i = 0; i < 5; i++) {
-    if (g[i].g >= -HF) {
+    const bool at_edge = fabsf(g[i].g + HF) <= g[i].E;
+    if (g[i].g >= -HF || (GIVEN && edge && at_edge)) {
       any_out |= gd[i] > 0;
       all_in &= gd[i] < 0;
       if (R.code == 1 && fabsf(gd[i]) <= egd[i] + TAUF) R.flag = true;
     }
-    if (R.code == 1 && fabsf(g[i].g + HF) <= g[i].E) R.flag = true;
+    if (R.code == 1 && at_edge && !(GIVEN && edge)) R.flag = true;
   }
   if (want & kWantDout) {
     if (R.code == 2) R.dout = -1.f;
@@ -755,7 +784,7 @@ __device__ __forceinline__ uint32_t phi_ids(const Iv& a, const Iv& b) {
   return id;
 }
 
-template <bool TUBE, bool FRAME = false, bool RANK = false>
+template <bool TUBE, bool FRAME = false, bool RANK = false, bool GIVEN = false>
 __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want, R32& R, Walk& W) {
   W.live = false;
   W.need_in = W.need_out = false;
@@ -816,7 +845,25 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   si.add(gz1, Ez1);
   if (has_phi) si.add_int(gphi, phlo, phhi);
   const float s = si.s;
-  R.code = decide(si, R.flag);
+  bool edge = false;  // GIVEN: a constraint at the band's edge is within the band
+  if (GIVEN) {
+    Band m;
+    m.add(lo_.g, lo_.E);
+    if (has_in) m.add(li_.g, li_.E);
+    m.add(gz0, Ez0);
+    m.add(gz1, Ez1);
+    if (has_phi) {
+      if (wide) {
+        m.add(gphi, fmaxf(gphi - phlo, phhi - gphi));
+      } else {
+        m.add(pa.g, pa.E);
+        m.add(pb.g, pb.E);
+      }
+    }
+    edge = R.code == 1 && m.resolved();
+  } else {
+    R.code = decide(si, R.flag);
+  }
   if (FRAME && near_plane) R.flag = true;
   if (RANK) {
     R.rank = (uint32_t)R.code;
@@ -999,8 +1046,9 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   bool any_out = false, all_in = true, unsure = false;
   if (R.code == 1) {
     auto add = [&](float g, float Eg, float gd, float egd) {
-      if (fabsf(g + HF) <= Eg) { unsure = true; return; }
-      if (g >= -HF) {
+      const bool at_edge = fabsf(g + HF) <= Eg;
+      if (at_edge && !(GIVEN && edge)) { unsure = true; return; }
+      if (g >= -HF || (GIVEN && at_edge)) {
         if (fabsf(gd) <= egd) { unsure = true; return; }
         if (gd > 0) any_out = true;
         if (!(gd < 0)) all_in = false;
@@ -1297,11 +1345,11 @@ __device__ inline void pcon_end(const Walk& W, R32& R) {
   }
 }
 
-template <bool TUBE, bool FRAME = false, bool RANK = false>
+template <bool TUBE, bool FRAME = false, bool RANK = false, bool GIVEN = false>
 __device__ inline void pcon32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   Walk W;
   W.answered = false;
-  if (pcon_begin<TUBE, FRAME, RANK>(S, T, want, R, W))
+  if (pcon_begin<TUBE, FRAME, RANK, GIVEN>(S, T, want, R, W))
     while (W.live) pcon_step<TUBE, FRAME, RANK>(S, T, W);
   pcon_end<RANK>(W, R);
 }
