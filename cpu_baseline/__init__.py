@@ -27,7 +27,7 @@ DEPS = [SRC, os.path.join(HERE, "shim", "cuda_runtime.h"), os.path.join(HERE, "s
         os.path.join(CSRC, "solid_fp64.cuh"), os.path.join(CSRC, "desc_build.h"), os.path.join(CSRC, "gv_desc.h"),
         os.path.join(ROOT, "include", "gv.h")]
 RANK_DEPS = [RANK_SRC, os.path.join(CSRC, "rank_fp64.cuh"), os.path.join(CSRC, "solid_fp32.cuh"),
-             os.path.join(CSRC, "nav_cull.cuh")] + DEPS
+             os.path.join(CSRC, "nav_cull.cuh"), os.path.join(CSRC, "bool_rank.cuh")] + DEPS
 KINDS = {"box": 0, "trd": 1, "trap": 2, "tube": 3, "cone": 4, "polycone": 5}
 _lock = threading.Lock()
 _lib = None

@@ -2,6 +2,7 @@
 // host, for tests that compare it with the whole binary64 evaluation (gv_cpu.cpp) without a GPU, and
 // the navigation step's plain look at a placed daughter (nav_cull.cuh) likewise.
 #include <cuda_runtime.h>  // the host stand-ins (shim/)
+#include "bool_rank.cuh"
 #include "nav_cull.cuh"
 #include "rank_fp64.cuh"
 
@@ -80,5 +81,32 @@ extern "C" void gvcpu_plain_look(int tag, const double* e, double rmin, const do
     o[4] = plain_outside(C, L) ? 1.f : 0.f;
     o[5] = tag <= kCullTube ? plain_safety(C, L) : 0.f;
     o[6] = L.margin;
+  }
+}
+
+// A boolean op(a, c) of two descriptors, c placed by R (row-major) and t: the whole evaluation
+// (whole[]: inside, din, dout, sin, sout as doubles, 5 per track) and the ranked one (0 in ranked[i] when not
+// certain, or when the components have no ranked form).
+extern "C" void gvcpu_bool(int op, const void* a, const void* c, const double* R, const double* t, int64_t n,
+                           const double* const* tr, unsigned want, double* whole, double* got, int8_t* ranked) {
+  Desc parts[2], S;
+  std::memcpy(&parts[0], a, sizeof(Desc));
+  std::memcpy(&parts[1], c, sizeof(Desc));
+  std::memset(&S, 0, sizeof(S));
+  S.type = kBool;
+  S.bop = op;
+  for (int i = 0; i < 9; i++) S.bR[i] = R[i];
+  for (int i = 0; i < 3; i++) S.bt[i] = t[i];
+  S.parts = parts;
+  const bool dirs = want & (f64::kWantDin | f64::kWantDout), forms = f64::bool_ranks(parts[0], parts[1]);
+#pragma omp parallel for schedule(static, 1024)
+  for (int64_t i = 0; i < n; i++) {
+    f64::Track T{tr[0][i], tr[1][i], tr[2][i], 0, 0, 0};
+    if (dirs) { T.u = tr[3][i]; T.v = tr[4][i]; T.w = tr[5][i]; }
+    f64::Result r{0, 0, 0, 0, 0}, q{0, 0, 0, 0, 0};
+    f64::bool_query(S, T, want, r);
+    ranked[i] = forms && f64::bool_ranked(S, parts[0], parts[1], T, want, q);
+    const double w[5] = {(double)r.code, r.din, r.dout, r.sin, r.sout}, o[5] = {(double)q.code, q.din, q.dout, q.sin, q.sout};
+    for (int k = 0; k < 5; k++) { whole[5 * i + k] = w[k]; got[5 * i + k] = o[k]; }
   }
 }

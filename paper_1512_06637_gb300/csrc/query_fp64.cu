@@ -1,10 +1,11 @@
 // query_fp64.cu -- the plain binary64 query pass.  Primitive solids take the ranked pass
 // (k_query_rank64): binary32 decides which constraint and which crossing give the results, binary64
-// evaluates those.  What has no binary32 form is evaluated whole, one thread per track: booleans in
-// index order (k_query_fp64); solids with features finer than binary32 resolves in tiles ordered by
+// evaluates those; booleans of solids with at most two z-planes likewise (k_query_bool_rank).  What has
+// no binary32 form is evaluated whole, one thread per track: other booleans in index order (k_query_fp64); solids with features finer than binary32 resolves in tiles ordered by
 // work class when the basket gives every SM a 2048-track tile (k_query_fp64_tiles: the FP64 pipe
 // spends the same on a warp instruction whatever its active lanes, so warps of one class run fewer
 // instructions), else in index order.  Per track the bits are the same in every one of them.
+#include "bool_rank.cuh"
 #include "gv_debug.cuh"
 #include "gv_internal.h"
 #include "solid_fp64.cuh"
@@ -240,6 +241,64 @@ __global__ void __launch_bounds__(256, ITEMS == 1 ? 2 : 3) k_query_rank64(const 
   for (unsigned q = tid; q < nopen; q += NT) query_open<FAMILY>(S, a, open[q], want);
 }
 
+// Booleans whose components rank (bool_rank.cuh): one thread per track; a track without a certain
+// ranking (surface starts of a component above all) goes on the block's list, evaluated whole.
+// Measured (box minus tube segment, 2^20 tracks, all five queries): 1213 -> 365 us (before: every piece of
+// both components in binary64, 594 FP64 warp instructions per 32 tracks; now 139, the FP64 pipe 69% busy).
+// Three blocks per SM 361 us.
+__global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restrict__ desc, QueryArgs a) {
+  __shared__ Desc S, A, C;
+  __shared__ int64_t open[256 + kOpenFlush];
+  __shared__ unsigned nopen;
+  stage_desc(S, desc);
+  stage_desc(A, desc->parts);
+  stage_desc(C, desc->parts + 1);
+  if (threadIdx.x == 0) nopen = 0u;
+  __syncthreads();
+  const unsigned want = (a.inside ? f64::kWantCode : 0u) | (a.din ? f64::kWantDin : 0u) |
+                        (a.dout ? f64::kWantDout : 0u) | (a.sin ? f64::kWantSin : 0u) |
+                        (a.sout ? f64::kWantSout : 0u);
+  const bool dirs = want & (f64::kWantDin | f64::kWantDout);
+  auto load = [&](int64_t i) {
+    f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
+    if (dirs) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+    return T;
+  };
+  auto store = [&](int64_t i, const f64::Result& R) {
+    if (a.inside) a.inside[i] = (int8_t)R.code;
+    if (a.din) a.din[i] = R.din;
+    if (a.dout) a.dout[i] = R.dout;
+    if (a.sin) a.sin[i] = R.sin;
+    if (a.sout) a.sout[i] = R.sout;
+  };
+  auto flush = [&]() {
+    for (unsigned q = threadIdx.x; q < nopen; q += 256) {
+      f64::Result R;
+      f64::bool_query(S, load(open[q]), want, R);
+      store(open[q], R);
+    }
+  };
+  const int64_t stride = (int64_t)gridDim.x * 256;
+  for (int64_t base = (int64_t)blockIdx.x * 256; base < a.n; base += stride) {  // block-uniform
+    const int64_t i = base + threadIdx.x;
+    if (i < a.n) {
+      const f64::Track T = load(i);
+      GV_DCHECK(!dirs || dbg_unit(T.u, T.v, T.w), kDbgDirection, i);
+      f64::Result R;
+      if (f64::bool_ranked(S, A, C, T, want, R)) store(i, R);
+      else open[atomicAdd(&nopen, 1u)] = i;
+    }
+    __syncthreads();
+    if (nopen >= (unsigned)kOpenFlush) {
+      flush();
+      __syncthreads();
+      if (threadIdx.x == 0) nopen = 0u;
+      __syncthreads();
+    }
+  }
+  flush();
+}
+
 // The ranking of multi-section polycones on its own, with lane refill as in the binary32 pass
 // (k_query_walk): a warp keeps one track per lane and refills idle lanes from its rows of 32 tracks (the
 // warps take rows in turn).  The verdict of track i is left in the low word of out[i].
@@ -422,7 +481,14 @@ cudaError_t launch_query_fp64(const gv_solid* s, const QueryArgs& a, cudaStream_
     case kBox: k_query_fp64<0><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a); break;
     case kTrd:
     case kTrap: k_query_fp64<1><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a); break;
-    case kBool: k_query_fp64<4><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a); break;
+    case kBool:
+      if (f64::bool_ranks(s->ph[0], s->ph[1])) {
+        const int64_t resident = (int64_t)sms * 2;
+        k_query_bool_rank<<<(unsigned)(blocks < resident ? blocks : resident), 256, 0, stream>>>(s->d, a);
+      } else {
+        k_query_fp64<4><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a);
+      }
+      break;
     default: k_query_fp64<2><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a); break;
   }
   return cudaGetLastError();

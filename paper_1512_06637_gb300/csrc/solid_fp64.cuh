@@ -770,20 +770,23 @@ __device__ inline void prim_query(const Desc& S, const Track& T, unsigned want, 
   }
 }
 
+// A track in the second component's frame: p_c = R^T (p - t), d_c = R^T d.
+__device__ __forceinline__ void bool_frame(const Desc& S, const Track& T, Track& Tc) {
+  const double v0 = xsub(T.x, S.bt[0]), v1 = xsub(T.y, S.bt[1]), v2 = xsub(T.z, S.bt[2]);
+  const double* M = S.bR;
+  Tc.x = xadd(xadd(xmul(M[0], v0), xmul(M[3], v1)), xmul(M[6], v2));
+  Tc.y = xadd(xadd(xmul(M[1], v0), xmul(M[4], v1)), xmul(M[7], v2));
+  Tc.z = xadd(xadd(xmul(M[2], v0), xmul(M[5], v1)), xmul(M[8], v2));
+  Tc.u = xadd(xadd(xmul(M[0], T.u), xmul(M[3], T.v)), xmul(M[6], T.w));
+  Tc.v = xadd(xadd(xmul(M[1], T.u), xmul(M[4], T.v)), xmul(M[7], T.w));
+  Tc.w = xadd(xadd(xmul(M[2], T.u), xmul(M[5], T.v)), xmul(M[8], T.w));
+}
+
 static __device__ __noinline__ void bool_query(const Desc& S, const Track& T, unsigned want, Result& R) {
   const Desc& A = S.parts[0];
   const Desc& C = S.parts[1];
-  Track Tc;  // c's frame: p_c = R^T (p - t), d_c = R^T d
-  {
-    const double v0 = xsub(T.x, S.bt[0]), v1 = xsub(T.y, S.bt[1]), v2 = xsub(T.z, S.bt[2]);
-    const double* M = S.bR;
-    Tc.x = xadd(xadd(xmul(M[0], v0), xmul(M[3], v1)), xmul(M[6], v2));
-    Tc.y = xadd(xadd(xmul(M[1], v0), xmul(M[4], v1)), xmul(M[7], v2));
-    Tc.z = xadd(xadd(xmul(M[2], v0), xmul(M[5], v1)), xmul(M[8], v2));
-    Tc.u = xadd(xadd(xmul(M[0], T.u), xmul(M[3], T.v)), xmul(M[6], T.w));
-    Tc.v = xadd(xadd(xmul(M[1], T.u), xmul(M[4], T.v)), xmul(M[7], T.w));
-    Tc.w = xadd(xadd(xmul(M[2], T.u), xmul(M[5], T.v)), xmul(M[8], T.w));
-  }
+  Track Tc;
+  bool_frame(S, T, Tc);
   const int op = S.bop;
   const double sa = prim_s(A, T.x, T.y, T.z), sc = prim_s(C, Tc.x, Tc.y, Tc.z);
   const double s = op == kUnion ? dmin(sa, sc) : (op == kIntersection ? dmax(sa, sc) : dmax(sa, -sc));
