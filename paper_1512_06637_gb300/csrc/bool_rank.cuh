@@ -208,14 +208,6 @@ __host__ __device__ inline bool bool_ranks(const Desc& a, const Desc& c) {
   return pa && pc && !((a.flags | c.flags) & kFp64Only);
 }
 
-__device__ __forceinline__ f32::TrackF split_track(const Track& T, bool dirs) {
-  auto w = [](double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return make_uint2((unsigned)b, (unsigned)(b >> 32));
-  };
-  return f32::track_from_words<true>(w(T.x), w(T.y), w(T.z), w(T.u), w(T.v), w(T.w), dirs);
-}
-
 // A component's results by a verdict on its safety or one of its crossings.
 __device__ __forceinline__ void prim_ranked(const Desc& S, const Track& T, uint32_t rank, Result& R) {
   const Verdict V{rank};

@@ -154,11 +154,12 @@ static __device__ __noinline__ void query_open(const Desc& S, const QueryArgs& a
 // blocks of 256 threads (80 registers) against two (128): cone 179 against 186 us; one-row tiles (short
 // baskets) 24.0 against 22.5 us.
 constexpr int kOpenFlush = 256;
+constexpr int kRankThreads = 256, kRankBlocks = 3;
 constexpr uint32_t kOpenVerdict = 0xFFFFFFFFu;
 // STORED: the verdicts are read from `stored`, where an earlier launch left them.
 template <int FAMILY, int ITEMS, bool STORED = false>
-__global__ void __launch_bounds__(256, ITEMS == 1 ? 2 : 3) k_query_rank64(const Desc* __restrict__ desc, QueryArgs a, const uint2* stored) {
-  constexpr int NT = 256, TILE = NT * ITEMS;
+__global__ void __launch_bounds__(kRankThreads, ITEMS == 1 ? 512 / kRankThreads : kRankBlocks) k_query_rank64(const Desc* __restrict__ desc, QueryArgs a, const uint2* stored) {
+  constexpr int NT = kRankThreads, TILE = NT * ITEMS;
   constexpr uint32_t NC = f64::kRankClasses;
   __shared__ Desc S;
   __shared__ uint32_t ver[TILE];
@@ -299,14 +300,48 @@ __global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restri
   flush();
 }
 
+// Baskets too short to fill the GPU: one track per thread, ranked and evaluated at once.  Latency bounds
+// them, and a tile's barriers and second loads only add to it.
+constexpr int kShortThreads = 128;
+constexpr int64_t kRankWalkMin = 1 << 19;  // multi-section polycones: two launches from here on
+template <int FAMILY>
+__global__ void __launch_bounds__(kShortThreads) k_query_rank64_short(const Desc* __restrict__ desc, QueryArgs a) {
+  __shared__ Desc S;
+  const unsigned want = (a.inside ? f64::kWantCode : 0u) | (a.din ? f64::kWantDin : 0u) |
+                        (a.dout ? f64::kWantDout : 0u) | (a.sin ? f64::kWantSin : 0u) |
+                        (a.sout ? f64::kWantSout : 0u);
+  const bool dirs = want & (f64::kWantDin | f64::kWantDout);
+  const int64_t i = (int64_t)blockIdx.x * kShortThreads + threadIdx.x;
+  f64::Track T{0, 0, 0, 0, 0, 0};
+  if (i < a.n) {
+    T.x = a.x[i]; T.y = a.y[i]; T.z = a.z[i];
+    if (dirs) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+  }
+  stage_desc(S, desc);
+  __syncthreads();
+  if (i >= a.n) return;
+  GV_DCHECK(!dirs || dbg_unit(T.u, T.v, T.w), kDbgDirection, i);
+  const f32::TrackF F = f64::split_track(T, dirs);
+  f32::R32 r;
+  f64::rank32<FAMILY>(S, F, want, r);
+  f64::Result R;
+  if (!r.flag) f64::query_ranked<FAMILY>(S, T, f64::Verdict{r.rank}, R);
+  else f64::query_refined<FAMILY>(S, T, F, want, R);
+  if (a.inside) a.inside[i] = (int8_t)R.code;
+  if (a.din) a.din[i] = R.din;
+  if (a.dout) a.dout[i] = R.dout;
+  if (a.sin) a.sin[i] = R.sin;
+  if (a.sout) a.sout[i] = R.sout;
+}
+
 // The ranking of multi-section polycones on its own, with lane refill as in the binary32 pass
 // (k_query_walk): a warp keeps one track per lane and refills idle lanes from its rows of 32 tracks (the
 // warps take rows in turn).  The verdict of track i is left in the low word of out[i].
 // Measured (8-plane polycone, 4 M tracks): 957 us with the evaluation, against 1274 us ranking a tile's
 // tracks in place, where a warp walks as long as its longest track (12.2 against 13.8 lanes, barriers).
-// Below 2^18 tracks the second launch and its traffic cost more than that.  Blocks of 256 x 3: 976 us,
+// Below 2^19 tracks the second launch and its traffic cost more than that (300000: 143 against about 100 us
+// one track per thread).  Blocks of 256 x 3: 976 us,
 // 384 x 2: 962 us.
-constexpr int64_t kRankWalkMin = 1 << 18;
 constexpr int kRankWalkThreads = 320, kRankWalkBlocks = 2;
 __global__ void __launch_bounds__(kRankWalkThreads, kRankWalkBlocks) k_rank_walk(const Desc* __restrict__ desc, QueryArgs a,
                                                                                  uint2* out) {
@@ -385,8 +420,8 @@ static double* verdict_array(const QueryArgs& a) {
 
 template <int ITEMS>
 static void launch_rank_stored(const gv_solid* s, const QueryArgs& a, const uint2* ver, int64_t cap, cudaStream_t stream) {
-  const int64_t tiles = (a.n + 256 * ITEMS - 1) / (256 * ITEMS);
-  k_query_rank64<3, ITEMS, true><<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, stream>>>(s->d, a, ver);
+  const int64_t tiles = (a.n + kRankThreads * ITEMS - 1) / (kRankThreads * ITEMS);
+  k_query_rank64<3, ITEMS, true><<<(unsigned)(tiles < cap ? tiles : cap), kRankThreads, 0, stream>>>(s->d, a, ver);
 }
 static void launch_rank_walk(const gv_solid* s, const QueryArgs& a, double* out, int sms, cudaStream_t stream) {
   const int64_t blocks = (a.n + kRankWalkThreads - 1) / kRankWalkThreads, cap = (int64_t)sms * kRankWalkBlocks;
@@ -399,24 +434,39 @@ template <int FAMILY, int ITEMS>
 static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaStream_t stream) {
   static const int occ = [] {
     int o = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_query_rank64<FAMILY, ITEMS>, 256, 0) != cudaSuccess || o < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_query_rank64<FAMILY, ITEMS>, kRankThreads, 0) != cudaSuccess || o < 1) {
       cudaGetLastError();
       o = 1;
     }
     return o;
   }();
-  const int64_t tiles = (a.n + 256 * ITEMS - 1) / (256 * ITEMS);
+  const int64_t tiles = (a.n + kRankThreads * ITEMS - 1) / (kRankThreads * ITEMS);
   const int64_t cap = (int64_t)sms * occ;
-  k_query_rank64<FAMILY, ITEMS><<<(unsigned)(tiles < cap ? tiles : cap), 256, 0, stream>>>(s->d, a, nullptr);
+  k_query_rank64<FAMILY, ITEMS><<<(unsigned)(tiles < cap ? tiles : cap), kRankThreads, 0, stream>>>(s->d, a, nullptr);
 }
 
-// Tiles of 2048 tracks when every resident block gets four of them, of 1024 when it gets one, else of
-// 256: a short basket is spread over every SM.
+// Tiles of 2048 tracks when every resident block gets four of them, of 1024 when it gets one; shorter
+// baskets one track per thread, except tubes and cones from 1024 tracks per SM on, which gain from
+// ordering already (tile of 256: measured, all five queries, against one track per thread: 50021 tracks
+// tube 25.9 / 24.9, cone 22.2 / 19.5, polycone 32.4 / 27.2 us; 200000 tracks tube 52.1 / 56.2, cone 46.7 /
+// 48.1, box 16.2 / 12.4, trap 31.6 / 28.2 us).
 template <int FAMILY>
 static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaStream_t stream) {
-  if (a.n >= (int64_t)sms * 3 * 4 * 2048) launch_rank64<FAMILY, 8>(s, a, sms, stream);
-  else if (a.n >= (int64_t)sms * 3 * 1024) launch_rank64<FAMILY, 4>(s, a, sms, stream);
-  else launch_rank64<FAMILY, 1>(s, a, sms, stream);
+  constexpr bool kOrdered = FAMILY == 2 || FAMILY == 4;
+  const bool tiles = a.n >= (FAMILY == 3 ? kRankWalkMin : (int64_t)sms * 3 * 1024);
+  if (tiles && a.n >= (int64_t)sms * 3 * 4 * 2048) {
+    launch_rank64<FAMILY, 8>(s, a, sms, stream);
+  } else if (tiles) {
+    launch_rank64<FAMILY, 4>(s, a, sms, stream);
+  } else {
+    if constexpr (kOrdered) {
+      if (a.n >= (int64_t)sms * 1024) {
+        launch_rank64<FAMILY, 1>(s, a, sms, stream);
+        return;
+      }
+    }
+    k_query_rank64_short<FAMILY><<<(unsigned)((a.n + kShortThreads - 1) / kShortThreads), kShortThreads, 0, stream>>>(s->d, a);
+  }
 }
 
 template <int FAMILY, int ITEMS>

@@ -114,7 +114,15 @@ __device__ inline void pcon_ranked(const Desc& S, const Track& T, Verdict V, Res
       const double r = __dsqrt_rn(r2);
       if (sk == f32::kOuter) s = g_out(S.out[k], r, T.z);
       else if (sk == f32::kInner) s = g_in(S.in[k], r, T.z);
-      else s = s_closed(S, k, r, T.z, (S.flags & kHasPhi) ? phi_g(S, phi_eval(S, T.x, T.y)) : -GV_INF);
+      else {
+        const double gphi = (S.flags & kHasPhi) ? phi_g(S, phi_eval(S, T.x, T.y)) : -GV_INF;
+        if (k != f32::kAllPieces) {
+          s = s_closed(S, k, r, T.z, gphi);
+        } else {
+          s = s_closed(S, 0, r, T.z, gphi);
+          for (int j = 1; j + 1 < S.nz; j++) s = dmin(s, s_closed(S, j, r, T.z, gphi));
+        }
+      }
     } else if (sk == f32::kZLow) {
       s = xsub(S.z[k], T.z);
     } else if (sk == f32::kZHigh) {
@@ -140,6 +148,15 @@ __device__ inline void pcon_ranked(const Desc& S, const Track& T, Verdict V, Res
     t = num / den;
   }
   rank_results(V, s, t, R);
+}
+
+// A binary64 track split for the binary32 passes.
+__device__ __forceinline__ f32::TrackF split_track(const Track& T, bool dirs) {
+  auto w = [](double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return make_uint2((unsigned)b, (unsigned)(b >> 32));
+  };
+  return f32::track_from_words<true>(w(T.x), w(T.y), w(T.z), w(T.u), w(T.v), w(T.w), dirs);
 }
 
 // Families: 0 box, 1 trd/trap, 2 tube, 3 polycone, 4 cone (two z-planes).

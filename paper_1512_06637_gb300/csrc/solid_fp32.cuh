@@ -75,6 +75,7 @@ struct R32 {
 // binary32 cannot certify) and decide the rest.
 enum : uint32_t { kNone = 0, kOuter = 1, kInner = 2, kZLow = 3, kZHigh = 4, kPhiS = 5, kPhiE = 6, kWhole = 7 };
 constexpr uint32_t kVerGoalOut = 1u << 19;
+constexpr int kAllPieces = 31;  // with kWhole: the least of all pieces (sections are 0-30)
 __device__ __forceinline__ uint32_t ver_safety(uint32_t kind, int k) { return kind << 3 | (uint32_t)k << 6; }
 __device__ __forceinline__ uint32_t ver_dist(uint32_t kind, int k) { return kind << 11 | (uint32_t)k << 14; }
 
@@ -993,8 +994,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
         R.sin = best.v;
         if (!RANK && !certified(best)) R.flag = true;
         if (RANK) {
-          R.flag |= !m.sure();
-          R.rank |= ver_safety(mkind, (int)m.id);
+          R.rank |= m.sure() ? ver_safety(mkind, (int)m.id) : ver_safety(kWhole, kAllPieces);
           R.se = best.e;
         }
       }

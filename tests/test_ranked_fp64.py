@@ -88,7 +88,7 @@ def test_polycone_fp64_two_launches_and_in_place():
     import torch
 
     import paper_1512_06637_gb300 as gv
-    n = (1 << 18) + 77
+    n = (1 << 19) + 77
     spec = NAMED["polycone"]
     tr = W.tracks_for_solid(spec, n, seed=1100)
     want = cpu_baseline.Solid(spec).query(**tr, threads=8)
