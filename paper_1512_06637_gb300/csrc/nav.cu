@@ -43,7 +43,7 @@ struct alignas(16) NodeD {
   int32_t first;    // daughters: children[first .. first + count)
   int32_t count;
   int32_t grid;     // voxel grid over the daughters (-1: none)
-  int32_t pad;
+  int32_t never;    // some daughter has no binary32 form
 };
 
 // A uniform grid over the daughters of a node, in the node's frame: cell (i, j, k) lists
@@ -662,6 +662,20 @@ __device__ __forceinline__ void rank_local32(const Desc& S, const f32::TrackF& T
   else if (S.type == kTube) tube_rank_call(S, T, want, R);
   else pcon_rank_call(S, T, want, R);
 }
+// The ranking with the code from binary64, for a track whose code binary32 cannot certify.
+static __device__ __noinline__ void rank_given_call(const Desc& S, const f64::Track& T64, const f32::TrackF& T, unsigned want,
+                                                    f32::R32& R) {
+  R.flag = T.bad || S.type == kBool || (S.flags & kFp64Only);
+  if (R.flag) return;
+  R.code = f64::code_of(f64::prim_s(S, T64.x, T64.y, T64.z));
+  R.din = R.dout = R.sin = R.sout = 0.f;
+  R.rank = 0u;
+  R.te = R.se = 0.f;
+  if (S.type == kBox) f32::box32<true, true, true>(S, T, want, R);
+  else if (S.type == kTrd || S.type == kTrap) f32::planar32<true, true, true>(S, T, want, R);
+  else if (S.type == kTube) f32::pcon32<true, true, true, true>(S, T, want, R);
+  else f32::pcon32<false, true, true, true>(S, T, want, R);
+}
 __device__ __noinline__ void planar_ranked_call(const Desc& S, const f64::Track& T, f64::Verdict V, f64::Result& R) {
   f64::planar_ranked(S, T, V, R);
 }
@@ -763,7 +777,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__
       const int32_t* ids = nullptr;
       if (valid) {
         v = a.node[i];
-        flag = v < 0 || v >= nnodes;
+        flag = v < 0 || v >= nnodes || nodes[v].never;  // a daughter without binary32 form: binary64
       }
       if (valid && !flag) {
         const f32::TrackF W = f32::load_track(X, Y, Z, Ux, Uy, Uz, i, true);
@@ -793,15 +807,17 @@ __global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__
         for (int b = 0; b < m; b++) {
           const Cull& C = cull[ids[j0 + b]];
           const int tag = C.tag;
-          bool take = all || tag == kCullNever || (want_saf && tag == kCullOther);
+          bool take = all;
           if (!take) {
             const PlainLocal L = plain_local(C, P);
             float from;
             bool near;
             take = !plain_miss(C, P, L, from, near) || near;
             if (want_saf) {
-              const float s = plain_safety(C, L), lb = s - L.margin;
-              ub = fminf(ub, s < L.margin ? F_INF : s + L.margin);  // a point not outside gives none
+              const bool own = tag <= kCullTube;
+              const float s = own ? plain_safety(C, L) : plain_other(solids[C.solid], L.q[0], L.q[1], L.q[2]);
+              const float m = own ? L.margin : 3.f * L.margin, lb = s - m;
+              ub = fminf(ub, s < m ? F_INF : s + m);  // a point not outside gives none
               if (take) {  // evaluated anyway
               } else if (lb < s1) {
                 s3 = s2; s2 = s1; j2 = j1; s1 = lb; j1 = j0 + b;
@@ -1218,8 +1234,14 @@ __device__ __forceinline__ void pool_rank(const Geo& g, StepPool<SLOTS>& Q, int 
         Q.prank[i] = ~0u;
       } else {
         f32::R32 R;
-        rank_local32(S, to_local32(C, track_from(p, d)),
-                     !mother ? f32::kWantDin : want_saf ? f32::kWantDout | f32::kWantSout : f32::kWantDout, R);
+        const unsigned want = !mother ? f32::kWantDin : want_saf ? f32::kWantDout | f32::kWantSout : f32::kWantDout;
+        const f32::TrackF L = to_local32(C, track_from(p, d));
+        rank_local32(S, L, want, R);
+        if (R.flag) {
+          f64::Track T;
+          local64(C, p, d, T);
+          rank_given_call(S, T, L, want, R);
+        }
         const float t = mother ? R.dout : R.din;
         Q.t[i] = R.flag || (mother && t < 0.f) ? CUDART_NAN_F : t;
         Q.e[i] = fmaf(2.f * f32::U, fabsf(t), R.te);
@@ -1424,7 +1446,7 @@ __global__ void __launch_bounds__(kNavThreads, 1) k_nav_pool(Geo g, NavArgs a, c
   const bool want_saf = a.safety != nullptr;
   const int64_t total = cnt ? (int64_t)*cnt : a.n;
   const int64_t share = (total + gridDim.x - 1) / gridDim.x;
-  const int tile = share >= kNavSlots ? kNavSlots : max((int)share, 32);
+  const int tile = share >= kNavSlots ? kNavSlots : max((int)share, 8);
   for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < total; t0 += (int64_t)gridDim.x * tile) {
     const int len = total - t0 < tile ? (int)(total - t0) : tile;
     for (int s = tid; s < kNavSlots; s += kNavThreads) {
@@ -1917,6 +1939,7 @@ static void build_cull(gv_geom* g) {
     else if (h.type == kBox) C.tag = kCullBox;
     else if (h.type == kTube && !(h.flags & kHasPhi)) C.tag = kCullTube;
     else C.tag = kCullOther;
+    if (C.tag == kCullNever && N.parent >= 0) g->nodes[N.parent].never = 1;
     if (C.tag == kCullTube && (h.inner & 1u)) C.rmin = (float)h.in[0].b;  // a = 0: the radius
   }
 }
@@ -2101,7 +2124,7 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
   cudaStream_t st = (cudaStream_t)stream;
   const int sms = sm_count();
   if (prec == GV_FP64) {
-    const cudaError_t e = launch_nav_pool(g, a, std::min<int64_t>((t->n + 31) / 32, sms), nullptr, nullptr, st);
+    const cudaError_t e = launch_nav_pool(g, a, std::min<int64_t>((t->n + 7) / 8, sms), nullptr, nullptr, st);
     if (e != cudaSuccess) return cuda_error(e, "nav launch");
   } else {
     if (!ws) return set_error(GV_ERR_INVALID_ARG, "nav: GV_FP32_REFINE needs a workspace");
