@@ -1534,52 +1534,53 @@ static __device__ __noinline__ int32_t locate64_surf(const Geo& g, double x, dou
 
 // Locate as locate64_surf, with the codes taken in binary32 when every one on the way is
 // certified (a certified code is the binary64 one); otherwise locate64_surf decides.
+// Lanes go down the tree with plain codes until they need a certified one, and take that together.
 __device__ __forceinline__ int32_t locate_rank32(const Geo& g, double x, double y, double z, bool& surf) {
-  const NodeD* nodes = g.nodes;
-  const Desc* solids = g.solids;
   const double p[3] = {x, y, z}, d0[3] = {0.0, 0.0, 0.0};
   const f32::TrackF W = track_from(p, d0);
   const PlainTrack P = plain_track(W);
-  if (!W.bad) {
-    bool sf = false;
-    f32::R32 R;
-    const int world = plain_code(g, 0, P);
-    if (world == 2) return -1;
-    R.flag = false;
-    R.code = world;
-    if (world == 1) query32(solids[nodes[0].desc], to_local32(nodes[0], W), f32::kWantCode, R);
-    bool ok = !R.flag;
-    int32_t v = -1;
-    if (ok) {
-      sf |= R.code == 1;
-      if (R.code != 2) {
-        v = 0;
-        for (int depth = 0; ok && depth < 64; depth++) {
-          const NodeD& N = nodes[v];
-          int32_t into = -1;
-          const int32_t* ids;
-          int count;
-          if (!candidates32(N, g.cull[v], g.children, g.vox, P, ids, count))
-            candidates64(N, g.children, g.vox, x, y, z, ids, count);
-          for (int j = 0; j < count; j++) {
-            const int32_t c = ids[j];
-            const int look = plain_code(g, c, P);
-            if (look == 2) continue;
-            if (look == 0) { into = c; break; }
-            query32(solids[nodes[c].desc], to_local32(nodes[c], W), f32::kWantCode, R);
-            if (R.flag) { ok = false; break; }
-            sf |= R.code == 1;
-            if (R.code != 2) { into = c; break; }
-          }
-          if (!ok || into < 0) break;
-          v = into;
-        }
+  bool ok = !W.bad, done = W.bad, sf = false;
+  int32_t v = -1;                // the node reached
+  const int32_t* ids = nullptr;  // the daughters to look at (first the world), the next one
+  int at = 0, count = 1, depth = 0;
+  const unsigned lanes = __activemask();
+  while (__any_sync(lanes, !done)) {
+    int32_t need = -1, into = -1;
+    while (!done && at < count) {
+      const int32_t c = ids ? ids[at] : 0;
+      const int look = plain_code(g, c, P);
+      if (look == 2) { at++; continue; }
+      if (look == 0) into = c;
+      else need = c;
+      break;
+    }
+    __syncwarp(lanes);
+    if (need >= 0) {
+      f32::R32 R;
+      query32(g.solids[g.nodes[need].desc], to_local32(g.nodes[need], W), f32::kWantCode, R);
+      if (R.flag) {
+        ok = false;
+        done = true;
+      } else {
+        sf |= R.code == 1;
+        if (R.code != 2) into = need;
+        else at++;
       }
+    } else if (into < 0) {
+      done = true;  // in none of the daughters
     }
-    if (ok) {
-      surf |= sf;
-      return v;
+    __syncwarp(lanes);
+    if (into >= 0) {
+      v = into;
+      at = 0;
+      done = ++depth > 64;
+      if (!candidates32(g.nodes[v], g.cull[v], g.children, g.vox, P, ids, count))
+        candidates64(g.nodes[v], g.children, g.vox, x, y, z, ids, count);
     }
+  }
+  if (ok) {
+    surf |= sf;
+    return v;
   }
   return locate64_surf(g, x, y, z, surf);
 }
