@@ -1634,20 +1634,44 @@ __device__ __forceinline__ void flight_begin(const TransportArgs& a, int64_t i, 
   else if (F.v >= a.nnodes) F.why = GV_LOST;
 }
 
-// The first half of one step of the loop of the Physics subsection (see gv.h) for track i:
-// the boundary distance, the physics step and, when the process acts first, the process.
-__device__ inline void flight_step(const TransportArgs& a, int64_t i, const Step& o, Flight& F) {
+// Bounds in binary32 of the sampled step -log(xi) / sigma (sigma <= 0: none, +inf).
+__device__ __forceinline__ float free_path_from(double xi, double sigma) {
+  const float s = (float)sigma;
+  if (!(sigma > 0)) return F_INF;
+  // the argument's rounding moves the logarithm by at most 1.2e-7; the rest is relative
+  const float v = -logf((float)xi), lo = __fdividef(v - fmaf(4e-6f, fabsf(v), 4e-7f), s);
+  return v < 80.f && s > 1e-30f ? lo : 0.f;  // beyond binary32: binary64 decides
+}
+
+// One step of the loop of the Physics subsection (see gv.h), after its geometry (o), in two parts.
+// First: lost tracks, and those whose physics steps both exceed the boundary distance by more than the
+// tie margin, certainly in binary32: these go to the boundary.  True: the physics step decides.
+__device__ __forceinline__ bool flight_geometry(const TransportArgs& a, int64_t i, const Step& o, Flight& F) {
   const double* r = a.xi + ((size_t)i * (size_t)a.kmax + (size_t)F.k) * 4;
-  const double dgeo = o.step, second = o.second;
+  const double dgeo = o.step;
   const int32_t m = a.material[F.v];
-  if (dgeo < 0 || m < 0 || m >= a.nmat) { F.why = GV_LOST; F.live = false; return; }
+  if (dgeo < 0 || m < 0 || m >= a.nmat) { F.why = GV_LOST; F.live = false; return false; }
+  if (fabs(o.second - dgeo) <= 1e-9 * (1.0 + dgeo)) F.near = true;
+  const float reach = (float)dgeo * 1.00001f + 1e-6f;
+  if (!(free_path_from(r[0], a.sigma_n[2 * m]) > reach && free_path_from(r[1], a.sigma_n[2 * m + 1]) > reach)) return true;
+  F.k++;
+  for (int j = 0; j < 3; j++) F.p[j] = xadd(F.p[j], xmul(dgeo, F.d[j]));
+  F.len = xadd(F.len, dgeo);
+  F.reloc = true;  // the probe point past the boundary is located by flight_locate
+  return false;
+}
+
+// Second: the physics step in binary64 against the boundary distance and, when the process acts first,
+// the process.
+__device__ __forceinline__ void flight_physics(const TransportArgs& a, int64_t i, double dgeo, Flight& F) {
+  const double* r = a.xi + ((size_t)i * (size_t)a.kmax + (size_t)F.k) * 4;
+  const int32_t m = a.material[F.v];
   const double sig0 = a.sigma_n[2 * m], sig1 = a.sigma_n[2 * m + 1];
   const double s0 = sig0 > 0 ? -log(r[0]) / sig0 : CUDART_INF;
   const double s1 = sig1 > 0 ? -log(r[1]) / sig1 : CUDART_INF;
   const int proc = s1 < s0 ? 1 : 0;
   const double sp = proc ? s1 : s0;
-  const double scale = 1.0 + dgeo;
-  if (fabs(sp - dgeo) <= 1e-9 * scale || fabs(second - dgeo) <= 1e-9 * scale) F.near = true;
+  if (fabs(sp - dgeo) <= 1e-9 * (1.0 + dgeo)) F.near = true;
   F.k++;
   if (sp < dgeo) {  // the process acts before the boundary
     for (int j = 0; j < 3; j++) F.p[j] = xadd(F.p[j], xmul(sp, F.d[j]));
@@ -1658,7 +1682,7 @@ __device__ inline void flight_step(const TransportArgs& a, int64_t i, const Step
     double sb, cb;
     sincos(b, &sb, &cb);
     F.d[0] = xmul(sa, cb); F.d[1] = xmul(sa, sb); F.d[2] = ca;
-  } else {  // to the boundary; the probe point past it is located by flight_locate
+  } else {  // to the boundary
     for (int j = 0; j < 3; j++) F.p[j] = xadd(F.p[j], xmul(dgeo, F.d[j]));
     F.len = xadd(F.len, dgeo);
     F.reloc = true;
@@ -1702,7 +1726,8 @@ struct FlightPool {
   int32_t k[kFlightSlots];
   uint8_t why[kFlightSlots], near[kFlightSlots], live[kFlightSlots], reloc[kFlightSlots];
   unsigned long long next;
-  int scount[kKinds], nreloc;
+  int scount[kKinds], nreloc, nphys;
+  double dgeo[kFlightSlots];
 };
 
 __device__ __forceinline__ void flight_load(const FlightPool& P, int s, Flight& F) {
@@ -1750,15 +1775,10 @@ __global__ void __launch_bounds__(kFlightThreads, 1) k_transport(Geo g, Transpor
     const int n = pool_kinds<kFlightThreads>(g, P.q, P.scount, [&](int s) { return P.live[s] != 0; });
     pool_rank<kFlightThreads>(g, P.q, n, false);
     pool_order<kFlightThreads>(g, P.q, n);
-    if (t == 0) P.nreloc = 0;
+    if (t == 0) P.nreloc = P.nphys = 0;
     __syncthreads();
-    for (int r = t; r < n; r += kFlightThreads) {
-      const int s = P.q.order[r];
-      Step o;
-      pool_finish(g, P.q, s, false, o);
-      Flight F;
-      flight_load(P, s, F);
-      flight_step(a, P.idx[s], o, F);
+    // what the step came to: the track goes on (to be located when at a boundary) or ends
+    auto settle = [&](int s, const Flight& F) {
       if (F.live) {
         flight_store(P, s, F);
         if (F.reloc) P.q.perm[atomicAdd(&P.nreloc, 1)] = (uint16_t)s;
@@ -1766,6 +1786,28 @@ __global__ void __launch_bounds__(kFlightThreads, 1) k_transport(Geo g, Transpor
         flight_end(a, P.idx[s], F);
         P.live[s] = 0;
       }
+    };
+    for (int r = t; r < n; r += kFlightThreads) {
+      const int s = P.q.order[r];
+      Step o;
+      pool_finish(g, P.q, s, false, o);
+      Flight F;
+      flight_load(P, s, F);
+      if (flight_geometry(a, P.idx[s], o, F)) {  // gathered, so that the logarithms run on full warps
+        P.near[s] = F.near;
+        P.dgeo[s] = o.step;
+        P.q.pid[atomicAdd(&P.nphys, 1)] = s;
+      } else {
+        settle(s, F);
+      }
+    }
+    __syncthreads();
+    for (int r = t; r < P.nphys; r += kFlightThreads) {
+      const int s = P.q.pid[r];
+      Flight F;
+      flight_load(P, s, F);
+      flight_physics(a, P.idx[s], P.dgeo[s], F);
+      settle(s, F);
     }
     __syncthreads();
     // the tracks at a boundary
