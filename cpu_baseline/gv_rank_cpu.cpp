@@ -95,7 +95,11 @@ extern "C" void gvcpu_bool(int op, const void* a, const void* c, const double* R
   std::memset(&S, 0, sizeof(S));
   S.type = kBool;
   S.bop = op;
-  for (int i = 0; i < 9; i++) S.bR[i] = R[i];
+  S.unrotated = 1;
+  for (int i = 0; i < 9; i++) {
+    S.bR[i] = R[i];
+    if (R[i] != (i % 4 == 0 ? 1.0 : 0.0)) S.unrotated = 0;
+  }
   for (int i = 0; i < 3; i++) S.bt[i] = t[i];
   S.parts = parts;
   const bool dirs = want & (f64::kWantDin | f64::kWantDout), forms = f64::bool_ranks(parts[0], parts[1]);

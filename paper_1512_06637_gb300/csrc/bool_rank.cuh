@@ -216,12 +216,34 @@ __device__ __forceinline__ void prim_ranked(const Desc& S, const Track& T, uint3
   else pcon_ranked(S, T, V, R);
 }
 
-// The results of bool_query, bit for bit; false when the ranking is not certain.
-__device__ inline bool bool_ranked(const Desc& S, const Desc& A, const Desc& C, const Track& T, unsigned want, Result& R) {
+// A track in the second component's frame; unrotated: the same values (products with 0 and 1 are
+// exact for finite tracks), 30 FP64 operations less.
+__device__ __forceinline__ void bool_frame_finite(const Desc& S, const Track& T, Track& Tc) {
+  if (S.unrotated) Tc = Track{xsub(T.x, S.bt[0]), xsub(T.y, S.bt[1]), xsub(T.z, S.bt[2]), T.u, T.v, T.w};
+  else bool_frame(S, T, Tc);
+}
+
+// The verdict of a boolean: bit 0 the point is inside, 1 the safety takes a's, 2 c's, 3 the larger of two,
+// 4-6 and 7-9 the constraints of a's and c's safeties, 10 and 11 the point is inside a, c, 12-14 the
+// crossing that gives the distance (0: none), 15-16 its z-plane, 17 the component is left there, 18 it is
+// c's.
+struct BoolVerdict {
+  uint32_t w;
+  __device__ __forceinline__ bool in() const { return w & 1u; }
+  __device__ __forceinline__ bool bit(int b) const { return (w >> b) & 1u; }
+  __device__ __forceinline__ uint32_t dkind() const { return (w >> 12) & 7u; }
+  __device__ __forceinline__ bool needs_c() const { return bit(2) || (dkind() != 0u && bit(18)); }
+};
+
+// The verdict on a track; false when the ranking is not certain.  Called, not inlined: its registers would
+// spill the evaluation's.
+static __device__ __noinline__ bool bool_verdict(const Desc& S, const Desc& A, const Desc& C, const Track& T, unsigned want, uint32_t& out) {
   const bool dirs = want & (kWantDin | kWantDout);
+  const f32::TrackF Fa = split_track(T, dirs);
+  if (Fa.bad) return false;
   Track Tc;
-  bool_frame(S, T, Tc);
-  const f32::TrackF Fa = split_track(T, dirs), Fc = split_track(Tc, dirs);
+  bool_frame_finite(S, T, Tc);
+  const f32::TrackF Fc = split_track(Tc, dirs);
   f32::R32 ra, rc;
   f32::rank_safety(A, Fa, ra);
   f32::rank_safety(C, Fc, rc);
@@ -229,9 +251,8 @@ __device__ inline bool bool_ranked(const Desc& S, const Desc& A, const Desc& C, 
   const int op = S.bop;
   const bool ia = ra.code == 0, ic = rc.code == 0;
   const bool in = op == kUnion ? ia || ic : op == kIntersection ? ia && ic : ia && !ic;
-  R.code = in ? 0 : 2;
-  R.sin = R.sout = R.din = R.dout = -1.0;
-  uint32_t end = 0u;
+  uint32_t V = (in ? 1u : 0u) | Verdict{ra.rank}.skind() << 4 | Verdict{rc.rank}.skind() << 7 | (ia ? 1u << 10 : 0u) |
+               (ic ? 1u << 11 : 0u);
   if (dirs) {
     f32::Along La, Lc;
     bool unsure = false;
@@ -239,6 +260,7 @@ __device__ inline bool bool_ranked(const Desc& S, const Desc& A, const Desc& C, 
     f32::along(C, Fc, Lc, unsure);
     f32::Val t{0.f, 0.f};
     bool answered = false;
+    uint32_t end = 0u;
     // the start agrees with the codes
     if (f32::within(La, t, unsure) != ia || f32::within(Lc, t, unsure) != ic) unsure = true;
     for (int guard = 0; guard < 12 && !unsure; guard++) {
@@ -258,61 +280,86 @@ __device__ inline bool bool_ranked(const Desc& S, const Desc& A, const Desc& C, 
       }
     }
     if (unsure || (in && !answered)) return false;
-    if (!answered) end = 0u;
+    if (answered) {
+      const Verdict E{end};
+      V |= E.dkind() << 12 | (uint32_t)E.dpiece() << 15 | (E.out() ? 1u << 17 : 0u) | ((end & f32::kFromC) ? 1u << 18 : 0u);
+    }
   }
   if (want & (kWantSin | kWantSout)) {
-    // which component: for a union (subtraction) of an outside (inside) point the smaller safety, ...
-    // s: the component's own side, v its certified safety
+    // a union is left (entered) through the component whose own safety is larger (smaller), an
+    // intersection the other way round, a subtraction as a and not-c
     const float va = ia ? ra.sout : ra.sin, vc = ic ? rc.sout : rc.sin;
     const float ea = fmaf(2.f * f32::U, fabsf(va), ra.se), ec = fmaf(2.f * f32::U, fabsf(vc), rc.se);
-    bool use_a, use_c, largest;
+    const bool largest = op == kUnion ? in : !in;
+    bool use_a, use_c;
     if (op == kUnion) {
-      largest = in;
       use_a = in ? ia : true;
       use_c = in ? ic : true;
-    } else if (op == kIntersection) {
-      largest = !in;
-      use_a = in ? true : !ia;
-      use_c = in ? true : !ic;
     } else {
-      largest = !in;
       use_a = in ? true : !ia;
-      use_c = in ? true : ic;
+      use_c = in ? true : op == kIntersection ? !ic : ic;
     }
     if (use_a && use_c) {  // one of them certainly, else both in binary64
       const float lo_a = va - ea, hi_a = va + ea, lo_c = vc - ec, hi_c = vc + ec;
       if (largest ? lo_a > hi_c : hi_a < lo_c) use_c = false;
       else if (largest ? lo_c > hi_a : hi_c < lo_a) use_a = false;
     }
+    V |= (use_a ? 2u : 0u) | (use_c ? 4u : 0u) | (largest ? 8u : 0u);
+  }
+  out = V;
+  return true;
+}
+
+// The results of bool_query, bit for bit, by a verdict.
+__device__ inline void bool_evaluate(const Desc& S, const Desc& A, const Desc& C, const Track& T, BoolVerdict V, Result& R) {
+  const bool in = V.in(), ia = V.bit(10), ic = V.bit(11);
+  R.code = in ? 0 : 2;
+  R.sin = R.sout = R.din = R.dout = -1.0;
+  Track Tc;
+  if (V.needs_c()) bool_frame_finite(S, T, Tc);
+  Result P;
+  if (V.bit(1) || V.bit(2)) {
     double v = 0;
-    Result P;
-    if (use_a) {
-      prim_ranked(A, T, ra.rank, P);
+    if (V.bit(1)) {
+      prim_ranked(A, T, (ia ? 0u : 2u) | f32::ver_safety((V.w >> 4) & 7u, 0), P);
       v = ia ? P.sout : P.sin;
     }
-    if (use_c) {
-      prim_ranked(C, Tc, rc.rank, P);
+    if (V.bit(2)) {
+      prim_ranked(C, Tc, (ic ? 0u : 2u) | f32::ver_safety((V.w >> 7) & 7u, 0), P);
       const double x = ic ? P.sout : P.sin;
-      v = use_a ? (largest ? dmax(v, x) : dmin(v, x)) : x;
+      v = V.bit(1) ? (V.bit(3) ? dmax(v, x) : dmin(v, x)) : x;
     }
     if (in) R.sout = v;
     else R.sin = v;
   }
-  if (dirs) {
-    double t = in ? 0.0 : GV_INF;
-    if (end) {
-      const bool c = (end & f32::kFromC) != 0u;
-      const uint32_t id = end & ~f32::kFromC;
-      const Desc& P = c ? C : A;
-      const Track& Q = c ? Tc : T;
-      Result X;
-      prim_ranked(P, Q, id, X);
-      t = (id & f32::kVerGoalOut) ? X.dout : X.din;
-    }
-    if (in) R.dout = t;
-    else R.din = t;
+  double t = in ? 0.0 : GV_INF;
+  if (V.dkind() != 0u) {
+    const uint32_t id = f32::ver_dist(V.dkind(), (int)((V.w >> 15) & 3u)) | (V.bit(17) ? f32::kVerGoalOut : 0u);
+    if (V.bit(18)) prim_ranked(C, Tc, id, P);
+    else prim_ranked(A, T, id, P);
+    t = V.bit(17) ? P.dout : P.din;
   }
+  if (in) R.dout = t;
+  else R.din = t;
+}
+
+__device__ __forceinline__ bool bool_ranked(const Desc& S, const Desc& A, const Desc& C, const Track& T, unsigned want, Result& R) {
+  uint32_t V;
+  if (!bool_verdict(S, A, C, T, want, V)) return false;
+  bool_evaluate(S, A, C, T, BoolVerdict{V}, R);
   return true;
+}
+
+// Groups tracks whose binary64 work is alike: the distance (none, a plane's crossing, a wall's), whether
+// the second component's frame is needed, whether a safety needs a square root.
+constexpr uint32_t kBoolClasses = 12;
+__device__ __forceinline__ uint32_t bool_class(const Desc& A, const Desc& C, BoolVerdict V) {
+  auto wall = [](const Desc& P, uint32_t kind) {
+    return P.nz == 2 && (kind == f32::kOuter || kind == f32::kInner || kind == f32::kWhole);
+  };
+  const uint32_t d = V.dkind() == 0u ? 0u : wall(V.bit(18) ? C : A, V.dkind()) ? 2u : 1u;
+  const bool root = (V.bit(1) && wall(A, (V.w >> 4) & 7u)) || (V.bit(2) && wall(C, (V.w >> 7) & 7u));
+  return 4u * d + (V.needs_c() ? 2u : 0u) + (root ? 1u : 0u);
 }
 
 }  // namespace f64

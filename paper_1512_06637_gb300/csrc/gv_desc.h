@@ -70,7 +70,7 @@ struct alignas(16) Desc {
   // p_a = bR p_c + bt (row-major); parts points to the two component records
   // (device memory owned by the boolean's handle).
   int32_t bop;
-  int32_t bpad;
+  int32_t unrotated;  // bR is exactly the unit matrix
   double bR[9], bt[3];
   const Desc* parts;
   double ext[3];  // half-extents of an axis-aligned box around the origin holding the solid

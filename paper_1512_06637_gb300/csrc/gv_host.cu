@@ -150,6 +150,9 @@ gv_status gv_solid_boolean(int32_t op, const gv_solid* a, const gv_solid* c, con
   s->h.bop = op;
   std::memcpy(s->h.bR, R, sizeof(s->h.bR));
   std::memcpy(s->h.bt, t, sizeof(s->h.bt));
+  s->h.unrotated = 1;
+  for (int i = 0; i < 9; i++)
+    if (R[i] != (i % 4 == 0 ? 1.0 : 0.0)) s->h.unrotated = 0;
   s->h.size = std::fmax(a->h.size, c->h.size);
   for (int i = 0; i < 3; i++) {  // a's box and the box around c's placed box
     const double hc = std::fabs(R[3 * i]) * c->h.ext[0] + std::fabs(R[3 * i + 1]) * c->h.ext[1] +

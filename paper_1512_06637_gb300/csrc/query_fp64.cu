@@ -242,20 +242,26 @@ __global__ void __launch_bounds__(kRankThreads, ITEMS == 1 ? 512 / kRankThreads 
   for (unsigned q = tid; q < nopen; q += NT) query_open<FAMILY>(S, a, open[q], want);
 }
 
-// Booleans whose components rank (bool_rank.cuh): one thread per track; a track without a certain
-// ranking (surface starts of a component above all) goes on the block's list, evaluated whole.
-// Measured (box minus tube segment, 2^20 tracks, all five queries): 1213 -> 365 us (before: every piece of
-// both components in binary64, 594 FP64 warp instructions per 32 tracks; now 139, the FP64 pipe 69% busy).
-// Three blocks per SM 361 us.
+// Booleans whose components rank (bool_rank.cuh), in tiles ordered by the binary64 work of the verdicts as
+// in k_query_rank64 (ITEMS tracks per thread).  A track without a certain verdict (surface starts of a
+// component above all) goes on the block's list, evaluated whole.
+// Measured (box minus tube segment, 2^20 tracks, all five queries): 1213 -> 290 us (before: every piece of
+// both components in binary64, 594 FP64 warp instructions per 32 tracks); ranked but in index order
+// 365 us (139 FP64 warp instructions).  The ranking inlined: 296 us (spills).
+template <int ITEMS>
 __global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restrict__ desc, QueryArgs a) {
+  constexpr int TILE = 256 * ITEMS;
+  constexpr uint32_t NC = f64::kBoolClasses;
   __shared__ Desc S, A, C;
-  __shared__ int64_t open[256 + kOpenFlush];
-  __shared__ unsigned nopen;
+  __shared__ uint32_t ver[TILE];
+  __shared__ uint16_t ord[TILE];
+  __shared__ int64_t open[TILE + kOpenFlush];
+  __shared__ unsigned cnt[NC], nopen;
+  const int tid = threadIdx.x;
   stage_desc(S, desc);
   stage_desc(A, desc->parts);
   stage_desc(C, desc->parts + 1);
-  if (threadIdx.x == 0) nopen = 0u;
-  __syncthreads();
+  if (tid == 0) nopen = 0u;
   const unsigned want = (a.inside ? f64::kWantCode : 0u) | (a.din ? f64::kWantDin : 0u) |
                         (a.dout ? f64::kWantDout : 0u) | (a.sin ? f64::kWantSin : 0u) |
                         (a.sout ? f64::kWantSout : 0u);
@@ -272,32 +278,60 @@ __global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restri
     if (a.sin) a.sin[i] = R.sin;
     if (a.sout) a.sout[i] = R.sout;
   };
-  auto flush = [&]() {
-    for (unsigned q = threadIdx.x; q < nopen; q += 256) {
+  auto flush = [&](unsigned count) {
+    for (unsigned q = tid; q < count; q += 256) {
       f64::Result R;
       f64::bool_query(S, load(open[q]), want, R);
       store(open[q], R);
     }
   };
-  const int64_t stride = (int64_t)gridDim.x * 256;
-  for (int64_t base = (int64_t)blockIdx.x * 256; base < a.n; base += stride) {  // block-uniform
-    const int64_t i = base + threadIdx.x;
-    if (i < a.n) {
-      const f64::Track T = load(i);
-      GV_DCHECK(!dirs || dbg_unit(T.u, T.v, T.w), kDbgDirection, i);
-      f64::Result R;
-      if (f64::bool_ranked(S, A, C, T, want, R)) store(i, R);
-      else open[atomicAdd(&nopen, 1u)] = i;
+  for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {  // block-uniform
+    const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
+    if (tid < (int)NC) cnt[tid] = 0u;
+    __syncthreads();
+    for (int j = tid; j < len; j += 256) {
+      const f64::Track T = load(t0 + j);
+      GV_DCHECK(!dirs || dbg_unit(T.u, T.v, T.w), kDbgDirection, t0 + j);
+      uint32_t V;
+      if (f64::bool_verdict(S, A, C, T, want, V)) {
+        atomicAdd(&cnt[f64::bool_class(A, C, f64::BoolVerdict{V})], 1u);
+      } else {
+        V = kOpenVerdict;
+        open[atomicAdd(&nopen, 1u)] = t0 + j;
+      }
+      ver[j] = V;
     }
     __syncthreads();
-    if (nopen >= (unsigned)kOpenFlush) {
-      flush();
-      __syncthreads();
-      if (threadIdx.x == 0) nopen = 0u;
-      __syncthreads();
+    const unsigned gathered = nopen;
+    __syncthreads();
+    if (tid == 0) {
+      unsigned run = 0;
+      for (uint32_t q = 0; q < NC; q++) {
+        const unsigned c = cnt[q];
+        cnt[q] = run;
+        run += c;
+      }
     }
+    __syncthreads();
+    for (int j = tid; j < len; j += 256)
+      if (ver[j] != kOpenVerdict) ord[atomicAdd(&cnt[f64::bool_class(A, C, f64::BoolVerdict{ver[j]})], 1u)] = (uint16_t)j;
+    __syncthreads();
+    const int ranked = (int)cnt[NC - 1];
+    for (int p = tid; p < ranked; p += 256) {
+      const int j = ord[p];
+      f64::Result R;
+      f64::bool_evaluate(S, A, C, load(t0 + j), f64::BoolVerdict{ver[j]}, R);
+      store(t0 + j, R);
+    }
+    if (gathered >= (unsigned)kOpenFlush) {
+      flush(gathered);
+      __syncthreads();
+      if (tid == 0) nopen = 0u;
+    }
+    __syncthreads();
   }
-  flush();
+  __syncthreads();
+  flush(nopen);
 }
 
 // Baskets too short to fill the GPU: one track per thread, ranked and evaluated at once.  Latency bounds
@@ -533,8 +567,9 @@ cudaError_t launch_query_fp64(const gv_solid* s, const QueryArgs& a, cudaStream_
     case kTrap: k_query_fp64<1><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a); break;
     case kBool:
       if (f64::bool_ranks(s->ph[0], s->ph[1])) {
-        const int64_t resident = (int64_t)sms * 2;
-        k_query_bool_rank<<<(unsigned)(blocks < resident ? blocks : resident), 256, 0, stream>>>(s->d, a);
+        const int64_t resident = (int64_t)sms * 2, tiles = (a.n + 1023) / 1024;
+        if (tiles >= resident) k_query_bool_rank<4><<<(unsigned)resident, 256, 0, stream>>>(s->d, a);
+        else k_query_bool_rank<1><<<(unsigned)(blocks < resident ? blocks : resident), 256, 0, stream>>>(s->d, a);
       } else {
         k_query_fp64<4><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a);
       }
