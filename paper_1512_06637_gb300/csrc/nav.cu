@@ -919,9 +919,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__
   }
 }
 
-// WALK: the geometry has nodes whose daughters the pass finds by walking their grid (the
-// instance without it keeps the registers of the plain scan).
-template <bool WALK>
+// Geometries with nodes whose daughters the pass finds by walking their grid: kLanes lanes per track.
 __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
                                                   const Desc* __restrict__ solids, int nnodes, NavArgs a,
                                                   uint32_t* __restrict__ wl, unsigned long long* __restrict__ cnt,
@@ -949,13 +947,19 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
     const int64_t i = base + sperm[threadIdx.x / kLanes];
     const bool valid = i < a.n;
     bool flag = false;
-    Top2<WALK> top{F_INF, 0.f, F_INF, 0.f, kNone, kNone};
+    Top2<true> top{F_INF, 0.f, F_INF, 0.f, kNone, kNone};
     float saf = F_INF;
     int32_t v = -1;
     bool walked = false;  // keys are node indices (grid walk) rather than daughter order
     if (valid) {
       v = a.node[i];
-      if (v < 0 || v >= nnodes) flag = true;
+      if (v < 0 || v >= nnodes) {
+        flag = true;
+      } else {
+        const NodeD& N = nodes[v];
+        walked = vox.grids && N.grid >= 0 && N.count >= kWalk32Min;
+        flag = N.never && (want_saf || !walked);  // a daughter without binary32 form would be met: binary64
+      }
     }
     if (valid && !flag) {
       const f32::TrackF W = f32::load_track(X, Y, Z, Ux, Uy, Uz, i, true);
@@ -968,7 +972,6 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
         top.add(R.dout, half_tol(R.dout), kMother);
         if (want_saf) saf = R.sout;
       }
-      walked = WALK && vox.grids && N.grid >= 0 && N.count >= kWalk32Min;
       const unsigned want = (walked ? 0u : f32::kWantDin) | (want_saf ? f32::kWantSin : 0u);
       for (int j = sub; want != 0u && j < N.count; j += kLanes) {
         const NodeD& C = nodes[children[N.first + j]];
@@ -979,7 +982,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
         if (!walked && R.din >= 0) top.add(R.din, half_tol(R.din), j);
         if (want_saf && R.sin >= 0) saf = fminf(saf, R.sin);
       }
-      if (WALK && walked) {  // DistanceToIn of the daughters listed along the ray, cell by cell
+      if (walked) {  // DistanceToIn of the daughters listed along the ray, cell by cell
         const GridD& G = vox.grids[N.grid];
         double q[3], e[3];
         to_local64(N, a.x[i], a.y[i], a.z[i], q[0], q[1], q[2]);
@@ -2179,7 +2182,7 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
     if (vox.grids && g->walk32) {
       const int64_t per_block = 256 / kLanes;
       const int64_t blocks = std::min<int64_t>((t->n + per_block - 1) / per_block, (int64_t)sms * 8);
-      k_nav_fp32<true><<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a,
+      k_nav_fp32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a,
                                                          ws->idx, ws->counter, vox);
     } else {
       const int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sms * 2);
