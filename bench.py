@@ -655,8 +655,8 @@ def bench_box1024(gv, torch, reps=5000):
 
 def bench_fp64_form(gv, torch, solids, dev, outs, names, n, reps=2):
     """The same workload in plain binary64 (all five queries, the inputs already on the device):
-    per-solid CUDA-event times and the step's rate.  Baskets this large are evaluated in tiles
-    ordered by work class."""
+    per-solid CUDA-event times and the step's rate.  Binary32 decides which
+    crossing gives a result, binary64 evaluates it, in tiles ordered by that work."""
     per = {}
     for name in names:
         per[name] = _timed(torch, lambda: gv.query(solids[name], dev[name], precision="fp64", out=outs[name]), reps)

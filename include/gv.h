@@ -144,9 +144,12 @@ gv_status gv_workspace_refined(gv_workspace* ws, void* stream, int64_t* n_refine
  * three questions).  ws may be NULL for GV_FP64 and must hold >= tracks->n for
  * GV_FP32_REFINE.  With GV_FP32_REFINE, a basket of at most 65536 tracks of a
  * primitive solid is one launch (uncertain tracks are evaluated in binary64 at
- * once, with the same bits as the refinement pass).  With GV_FP64, a basket of a primitive solid with at least 2048
- * tracks per SM is evaluated in tiles ordered by work class (inside, outside, near
- * a surface): the results are the same bits as in index order, the pass is faster.
+ * once, with the same bits as the refinement pass).  With GV_FP64 binary32 may first
+ * decide which constraint and which crossing give a result, and tracks may be taken
+ * in another order: the results are the bits of evaluating each track whole in
+ * binary64.  A large basket of a polycone of several sections keeps those decisions
+ * in its dist_out or dist_in array until the results replace them (not when an
+ * array overlaps another one or an input).
  * Asynchronous on `stream`. */
 gv_status gv_query(const gv_solid* s, const gv_tracks* tracks, gv_precision prec,
                    const gv_results* res, gv_workspace* ws, void* stream);

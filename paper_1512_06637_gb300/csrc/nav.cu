@@ -80,7 +80,7 @@ struct Vox {
 constexpr int kVoxelMin = 16;
 // The steps walk a node's grid, and its cells carry safety lists, only from this many daughters on: a
 // binary64 DDA costs more than a plain look at a few dozen daughters (nested detector, 32 daughters
-// per shell: transport 24.2 ms walking their grids, 14.9 ms scanning them).
+// per shell: transport 24.2 ms walking their grids, then 14.9 ms scanning them).
 constexpr int kWalk32Min = 128;
 
 constexpr float kInf32 = __builtin_huge_valf();
@@ -732,7 +732,7 @@ __device__ __forceinline__ void group_merge(unsigned mask, Top2<DEDUP>& top) {
 // the least) are evaluated with certified bounds.  A lane leaves from none to a dozen daughters, so
 // the warp gathers its 32 tracks' (track, daughter) pairs in shared memory and evaluates them 32 at
 // a time, one per lane; each lane then reads its own pairs' results.
-// Measured (GB300, nested detector, 2^22 tracks with safety): 12.0 -> 2.75 ms (before: 8 lanes per
+// Measured (GB300, nested detector, 2^22 tracks with safety): 12.0 -> 2.80 ms (before: 8 lanes per
 // track, every daughter evaluated: 1214 warp instructions per track at 18 of 32 lanes; now 263 at 26).
 // Without the pairs, each lane evaluating its own daughters: 5.8 ms (12 lanes).  Three blocks per SM
 // (80 registers) 2.73, tiles of 2048 2.72 ms.
@@ -1082,9 +1082,10 @@ __device__ __forceinline__ f32::TrackF track_from(const double p[3], const doubl
 // Measured (GB300, same bits as evaluating every candidate in binary64): step with safety among 1728
 // daughters, 2^18 tracks, 112 -> 2.5 ms (every daughter's safety in binary64 kept the FP64 pipe 81% busy;
 // ranking per thread, without phases: 9.9 ms, instruction fetch); transport in the nested detector, 2^20
-// tracks, 32 steps, 56.7 -> 14.9 ms (per thread 21.3 ms).  Bound by latency: one block per SM, 14-20% of the
+// tracks, 32 steps, 56.7 -> 11.5 ms (per thread 21.3 ms; 14.9 before the
+// relocation in step and the gathered physics).  Bound by latency: one block per SM, 14-20% of the
 // issue slots, 6-18 of 32 lanes.  1024 threads (64 registers) against 512: step 2.5 against 2.8 ms, transport
-// 15.0 against 14.9 ms.
+// then 15.0 against 14.9 ms.
 constexpr int kPoolPairs = 4;
 enum : uint8_t { kSlotIdle = 0, kSlotMore = 1, kSlotRanked = 2, kSlotExact = 3 };
 enum : int { kKeyBox = 0, kKeyPlanar = 1, kKeyTube = 2, kKeyPcon = 3, kKeyNever = 4, kKeyExact = 5, kKeys = 6 };

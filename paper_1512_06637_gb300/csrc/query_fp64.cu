@@ -1,8 +1,8 @@
 // query_fp64.cu -- the plain binary64 query pass.  Primitive solids take the ranked pass
 // (k_query_rank64): binary32 decides which constraint and which crossing give the results, binary64
 // evaluates those; booleans of solids with at most two z-planes likewise (k_query_bool_rank).  What has
-// no binary32 form is evaluated whole, one thread per track: other booleans in index order (k_query_fp64); solids with features finer than binary32 resolves in tiles ordered by
-// work class when the basket gives every SM a 2048-track tile (k_query_fp64_tiles: the FP64 pipe
+// no ranked form is evaluated whole, one thread per track: other booleans in index order
+// (k_query_fp64); solids with features finer than binary32 resolves in tiles ordered by work class when the basket gives every SM a 2048-track tile (k_query_fp64_tiles: the FP64 pipe
 // spends the same on a warp instruction whatever its active lanes, so warps of one class run fewer
 // instructions), else in index order.  Per track the bits are the same in every one of them.
 #include "bool_rank.cuh"
