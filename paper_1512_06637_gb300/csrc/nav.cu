@@ -920,8 +920,13 @@ __global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__
 }
 
 // Geometries with nodes whose daughters the pass finds by walking their grid: kLanes lanes per track.
+// A listed daughter that the ray certainly misses (nav_cull.cuh) gets no certified evaluation: that is
+// most of them, and the frame change and pass of the rest bound the walk.  Measured (GB300, 1728
+// daughters, 2^18 tracks without safety, the same bits): 10.8 -> 4.2 ms; 1000 daughters, 10^5 tracks:
+// 4.8 -> 2.0 ms.  Leaving the walk at the first flag gained nothing.
 __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                                  const Desc* __restrict__ solids, int nnodes, NavArgs a,
+                                                  const Desc* __restrict__ solids, const Cull* __restrict__ cull,
+                                                  int nnodes, NavArgs a,
                                                   uint32_t* __restrict__ wl, unsigned long long* __restrict__ cnt,
                                                   Vox vox) {
   constexpr int kMother = 0x7ffffffe, kNone = 0x7fffffff;
@@ -987,6 +992,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
         double q[3], e[3];
         to_local64(N, a.x[i], a.y[i], a.z[i], q[0], q[1], q[2]);
         rot_local64(N, a.u[i], a.v[i], a.w[i], e[0], e[1], e[2]);
+        const PlainTrack P = plain_track(W);
         Dda D;
         if (D.begin(G, q, e)) {
           do {
@@ -997,6 +1003,10 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
             const int cell = D.cell(G);
             for (int j = vox.cells[2 * cell] + (int)sub; j < vox.cells[2 * cell + 1]; j += kLanes) {
               const int32_t id = vox.list[j];
+              const Cull& B = cull[id];
+              float from;
+              bool near;
+              if (B.tag != kCullNever && plain_miss(B, P, plain_local(B, P), from, near) && !near) continue;
               const NodeD& C = nodes[id];
               const f32::TrackF L = to_local32(C, W);
               f32::R32 R;
@@ -2183,7 +2193,7 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
     if (vox.grids && g->walk32) {
       const int64_t per_block = 256 / kLanes;
       const int64_t blocks = std::min<int64_t>((t->n + per_block - 1) / per_block, (int64_t)sms * 8);
-      k_nav_fp32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->nnodes, a,
+      k_nav_fp32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
                                                          ws->idx, ws->counter, vox);
     } else {
       const int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sms * 2);

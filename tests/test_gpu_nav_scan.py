@@ -68,3 +68,20 @@ def test_scan_matches_oracle(which, n, precision):
         if not safety:
             got["safety"] = want["safety"]
         check_nav(got, want, "fp64" if precision == "fp64" else "fp32", f"{which}-{precision}-{safety}")
+
+
+@pytest.mark.parametrize("n", [1, 31, 20_003])
+def test_grid_walk_matches_oracle(n):
+    """The binary32 step along a grid of 216 daughters, the ones the ray certainly misses left out."""
+    import torch
+
+    import paper_1512_06637_gb300 as gv
+    geo = lattice_geometry()
+    G, O = gv.Geometry(geo["solids"], geo["nodes"]), oracle.Geometry(geo["solids"], geo["nodes"])
+    for name, tr in (("crowded", W.crowded_tracks(geo, n, 18, surf_frac=0.2 if n > 1 else 0.0)), ("axis", axis_tracks(geo, n))):
+        node = O.locate(tr["x"], tr["y"], tr["z"])
+        want = O.nav_step(*[tr[k] for k in ("x", "y", "z", "dx", "dy", "dz")], node)
+        out = G.step(to_device(tr, torch), torch.from_numpy(node).cuda(), precision="fp32_refine",
+                     workspace=gv.Workspace(n), safety=False)
+        got = {k: v.cpu().numpy() for k, v in out.items()}
+        check_nav(dict(got, safety=want["safety"]), want, "fp32", f"{name}-{n}")
