@@ -1243,8 +1243,9 @@ __device__ __forceinline__ void pool_rank(const Geo& g, StepPool<SLOTS>& Q, int 
         f64::Result R;
         local64(C, p, d, T);
         query64(S, T, f64::kWantDin, R);
-        Q.t[i] = (float)R.din;
-        Q.e[i] = 0.f;
+        const float t = (float)R.din;
+        Q.t[i] = t;
+        Q.e[i] = t < f32::BIG ? 2.f * f32::U * fabsf(t) : 0.f;  // the cast's rounding: near ties go to nav_exact
         Q.prank[i] = ~0u;
       } else {
         f32::R32 R;
