@@ -66,6 +66,8 @@ constexpr int kSafeList = 64;
 // Lists are built for grids of at most these many daughters and cells (one evaluation per pair when the
 // geometry is created: 3 M for 1728 daughters).
 constexpr int kSafeDaughters = 8192, kSafeCells = 32768;
+// All lists of a geometry together: 135 MB.  Volumes beyond have none: their safeties scan the daughters.
+constexpr int64_t kSafeTotal = 1 << 18;
 
 // Device pointers of a geometry's grids (grids == nullptr: no grid is used).
 struct Vox {
@@ -2002,6 +2004,21 @@ static void build_cull(gv_geom* g) {
   }
 }
 
+// Device memory for the safety lists of `cells` cells.  The lists only spare a safety the scan of all
+// daughters, so a geometry that finds no memory for them (false) does without; e: any other error.
+static bool alloc_safe(gv_geom* g, int64_t cells, cudaError_t& e) {
+  e = cudaMalloc(&g->d_safe, sizeof(SafeEnt) * kSafeList * (size_t)cells);
+  if (e == cudaSuccess) e = cudaMalloc(&g->d_safe_cut, sizeof(float) * (size_t)cells);
+  if (e != cudaErrorMemoryAllocation) return e == cudaSuccess;
+  cudaGetLastError();  // leave no error behind for the launch checks
+  e = cudaSuccess;
+  if (g->d_safe) cudaFree(g->d_safe);
+  g->d_safe = nullptr;
+  g->d_safe_cut = nullptr;
+  for (GridD& G : g->grids) G.safe = -1;
+  return false;
+}
+
 }  // namespace gv
 
 extern "C" {
@@ -2068,7 +2085,7 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
     if (g->nodes[v].grid < 0) continue;
     GridD& G = g->grids[g->nodes[v].grid];
     const int64_t cells = (int64_t)G.n[0] * G.n[1] * G.n[2];
-    if (g->nodes[v].count < kWalk32Min || g->nodes[v].count > kSafeDaughters || cells > kSafeCells || safe_cells + cells > (1 << 24)) continue;
+    if (g->nodes[v].count < kWalk32Min || g->nodes[v].count > kSafeDaughters || cells > kSafeCells || safe_cells + cells > kSafeTotal) continue;
     G.safe = (int32_t)safe_cells;
     safe_cells += cells;
   }
@@ -2087,14 +2104,13 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
     e = cudaMalloc(&g->d_grids, sizeof(GridD) * g->grids.size());
     if (e == cudaSuccess) e = cudaMalloc(&g->d_cells, sizeof(int32_t) * g->cells.size());
     if (e == cudaSuccess) e = cudaMalloc(&g->d_list, sizeof(int32_t) * std::max<size_t>(g->list.size(), 1));
+    if (e == cudaSuccess && safe_cells > 0 && !alloc_safe(g, safe_cells, e)) safe_cells = 0;
     if (e == cudaSuccess) e = cudaMemcpy(g->d_grids, g->grids.data(), sizeof(GridD) * g->grids.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(g->d_cells, g->cells.data(), sizeof(int32_t) * g->cells.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !g->list.empty())
       e = cudaMemcpy(g->d_list, g->list.data(), sizeof(int32_t) * g->list.size(), cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess && safe_cells > 0) {
-    e = cudaMalloc(&g->d_safe, sizeof(SafeEnt) * kSafeList * (size_t)safe_cells);
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_safe_cut, sizeof(float) * (size_t)safe_cells);
     for (int v = 0; e == cudaSuccess && v < nnodes; v++) {
       if (g->nodes[v].grid < 0 || g->grids[g->nodes[v].grid].safe < 0) continue;
       const GridD& G = g->grids[g->nodes[v].grid];
