@@ -1845,53 +1845,51 @@ __global__ void __launch_bounds__(kFlightThreads, 1) k_transport(Geo g, Transpor
   }
 }
 
-// The safety lists of one grid (one block per cell): the daughters' SafetyToIn at the cell's centre
-// in shared memory, then kSafeList times the least of them.
-__global__ void __launch_bounds__(256) k_safe_lists(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
-                                                    const Desc* __restrict__ solids, int node, const GridD* __restrict__ grids,
-                                                    SafeEnt* __restrict__ list, float* __restrict__ cut) {
+// The safety lists of one grid (one block per cell): lower bounds of the daughters' SafetyToIn at the
+// cell's centre by the plain look, then kSafeList times the least of them.  A thread keeps the least of
+// its own daughters and looks for the next one only when that is taken.  Measured (GB300, gv_geom_create
+// of 4096 and 8000 daughters): 24.7 -> 6.4 and 77.3 -> 12.8 ms, of which 1.4 and 4.0 are these lists (before: every
+// SafetyToIn in binary64, and every value read again for every entry of a list).
+__global__ void __launch_bounds__(256) k_safe_lists(Geo g, int node, SafeEnt* __restrict__ list, float* __restrict__ cut) {
   extern __shared__ float val[];
-  __shared__ unsigned long long best[8];
-  const NodeD& N = nodes[node];
-  const GridD& G = grids[N.grid];
+  __shared__ unsigned long long best[2][8];
+  const NodeD& N = g.nodes[node];
+  const GridD& G = g.vox.grids[N.grid];
   const int cell = blockIdx.x, i = cell % G.n[0], j = cell / G.n[0] % G.n[1], k = cell / G.n[0] / G.n[1];
   const double q[3] = {G.lo[0] + (i + 0.5) * G.cell[0], G.lo[1] + (j + 0.5) * G.cell[1], G.lo[2] + (k + 0.5) * G.cell[2]};
-  double p[3];
+  double p[3], d[3] = {0.0, 0.0, 0.0};
   for (int r = 0; r < 3; r++) p[r] = N.R[3 * r] * q[0] + N.R[3 * r + 1] * q[1] + N.R[3 * r + 2] * q[2] + N.t[r];
+  const PlainTrack P = plain_world(p, d);
+  auto key = [&](int c) { return (unsigned long long)__float_as_uint(val[c]) << 32 | (unsigned)c; };
+  // values are not negative: their bit patterns order them
+  unsigned long long own = ~0ull;
   for (int c = threadIdx.x; c < N.count; c += blockDim.x) {
-    const NodeD& C = nodes[children[N.first + c]];
-    f64::Track T{0, 0, 0, 0, 0, 0};
-    f64::Result R;
-    to_local64(C, p[0], p[1], p[2], T.x, T.y, T.z);
-    query64(solids[C.desc], T, f64::kWantCode | f64::kWantSin, R);
-    // below the value by more than the rounding of any centre or frame change
-    val[c] = R.code == 2 ? fmaxf((float)R.sin * (1.f - 1e-5f) - 1e-5f, 0.f) : 0.f;
+    const Cull& C = g.cull[g.children[N.first + c]];
+    const PlainLocal L = plain_local(C, P);
+    const bool exact = C.tag <= kCullTube;
+    const float s = exact ? plain_safety(C, L) : plain_other(g.solids[C.solid], L.q[0], L.q[1], L.q[2]);
+    val[c] = fmaxf(s - (exact ? 1.f : 3.f) * L.margin, 0.f);
+    own = min(own, key(c));
   }
-  __syncthreads();
   const int64_t at = (int64_t)(G.safe + cell) * kSafeList;
   for (int e = 0; e <= kSafeList; e++) {
-    // values are not negative: their bit patterns order them
-    unsigned long long m = ~0ull;
-    for (int c = threadIdx.x; c < N.count; c += blockDim.x) {
-      const unsigned long long key = (unsigned long long)__float_as_uint(val[c]) << 32 | (unsigned)c;
-      m = key < m ? key : m;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long u = __shfl_xor_sync(0xffffffffu, m, o);
-      m = u < m ? u : m;
-    }
-    if ((threadIdx.x & 31) == 0) best[threadIdx.x >> 5] = m;
+    unsigned long long m = own;
+    for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) best[e & 1][threadIdx.x >> 5] = m;
     __syncthreads();
-    for (int w = 0; w < 8; w++) m = best[w] < m ? best[w] : m;
-    const bool none = (unsigned)(m >> 32) == 0x7f800000u || m == ~0ull;  // all taken
+    for (int w = 0; w < 8; w++) m = min(m, best[e & 1][w]);
+    const bool none = (unsigned)(m >> 32) >= 0x7f800000u;  // all taken
     const int c = (int)(m & 0xffffffffu);
     if (threadIdx.x == 0) {
       const float s = none ? F_INF : __uint_as_float((unsigned)(m >> 32));
-      if (e < kSafeList) list[at + e] = none ? SafeEnt{F_INF, -1} : SafeEnt{s, children[N.first + c]};
+      if (e < kSafeList) list[at + e] = none ? SafeEnt{F_INF, -1} : SafeEnt{s, g.children[N.first + c]};
       else cut[G.safe + cell] = s;
-      if (!none) val[c] = F_INF;
     }
-    __syncthreads();
+    if (!none && c % (int)blockDim.x == (int)threadIdx.x) {
+      val[c] = F_INF;
+      own = ~0ull;
+      for (int b = threadIdx.x; b < N.count; b += blockDim.x) own = min(own, key(b));
+    }
   }
 }
 
@@ -2021,6 +2019,15 @@ static bool alloc_safe(gv_geom* g, int64_t cells, cudaError_t& e) {
 
 }  // namespace gv
 
+static gv::Vox vox_of(const gv_geom* g) {
+  if (!g->use_vox || !g->d_grids) return gv::Vox{nullptr, nullptr, nullptr, nullptr, nullptr};
+  return gv::Vox{g->d_grids, g->d_cells, g->d_list, g->d_safe, g->d_safe_cut};
+}
+
+static gv::Geo geo_of(const gv_geom* g) {
+  return gv::Geo{g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, vox_of(g)};
+}
+
 extern "C" {
 
 gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, const int32_t* parent, const double* R,
@@ -2114,8 +2121,7 @@ gv_status gv_geom_create(int32_t nnodes, const gv_solid* const* node_solid, cons
     for (int v = 0; e == cudaSuccess && v < nnodes; v++) {
       if (g->nodes[v].grid < 0 || g->grids[g->nodes[v].grid].safe < 0) continue;
       const GridD& G = g->grids[g->nodes[v].grid];
-      k_safe_lists<<<G.n[0] * G.n[1] * G.n[2], 256, sizeof(float) * g->nodes[v].count>>>(
-          g->d_nodes, g->d_children, g->d_solids, v, g->d_grids, g->d_safe, g->d_safe_cut);
+      k_safe_lists<<<G.n[0] * G.n[1] * G.n[2], 256, sizeof(float) * g->nodes[v].count>>>(geo_of(g), v, g->d_safe, g->d_safe_cut);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
@@ -2151,15 +2157,6 @@ gv_status gv_geom_set_voxels(gv_geom* g, int32_t enable) {
 int32_t gv_geom_voxel_count(const gv_geom* g) { return g ? (int32_t)g->grids.size() : 0; }
 
 int32_t gv_geom_node_count(const gv_geom* g) { return g ? g->nnodes : 0; }
-
-static gv::Vox vox_of(const gv_geom* g) {
-  if (!g->use_vox || !g->d_grids) return gv::Vox{nullptr, nullptr, nullptr, nullptr, nullptr};
-  return gv::Vox{g->d_grids, g->d_cells, g->d_list, g->d_safe, g->d_safe_cut};
-}
-
-static gv::Geo geo_of(const gv_geom* g) {
-  return gv::Geo{g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, vox_of(g)};
-}
 
 static cudaError_t launch_nav_pool(const gv_geom* g, const gv::NavArgs& a, int64_t blocks, const uint32_t* wl,
                                    const unsigned long long* cnt, cudaStream_t st) {
