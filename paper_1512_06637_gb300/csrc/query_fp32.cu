@@ -5,7 +5,7 @@
 // memory (cp.async) while it computes the current one, splits them into binary32
 // pairs with integer operations; every certified result is written; the indices of
 // the others are appended to a worklist (one atomicAdd per warp after a ballot).
-// Pass 2 (k_refine_fp64): binary64 results, ranked with the code from binary64 (query_refined),
+// Pass 2 (k_refine_fp64): binary64 results, whole or ranked with the code from binary64 (query_refined),
 // over the worklist only; its length is read on the device, so the two launches
 // need no host round trip.
 #include "gv_debug.cuh"
@@ -39,7 +39,9 @@ template <int FAMILY> struct Shape32 { static constexpr int threads = 256, block
 template <> struct Shape32<0> { static constexpr int threads = 288, blocks = 4; };
 template <> struct Shape32<1> { static constexpr int threads = 288, blocks = 3; };
 
-template <int FAMILY>
+// DIRS false: an instance for calls that want no distance (trd/trap, 64 registers against 72: codes of 8 M
+// tracks 123 -> 111 us, safeties 130 -> 115 us).
+template <int FAMILY, bool DIRS = true>
 __global__ void __launch_bounds__(Shape32<FAMILY>::threads, Shape32<FAMILY>::blocks) k_query_fp32(const Desc* __restrict__ desc, QueryArgs a,
                                                     uint32_t* __restrict__ worklist,
                                                     unsigned long long* __restrict__ counter) {
@@ -48,8 +50,8 @@ __global__ void __launch_bounds__(Shape32<FAMILY>::threads, Shape32<FAMILY>::blo
   __shared__ uint2 stage[2][6][NT];  // this thread's current and next track, raw words
   stage_desc32(S, desc);
   __syncthreads();
-  const unsigned want = (a.inside ? f32::kWantCode : 0u) | (a.din ? f32::kWantDin : 0u) |
-                        (a.dout ? f32::kWantDout : 0u) | (a.sin ? f32::kWantSin : 0u) |
+  const unsigned want = (a.inside ? f32::kWantCode : 0u) | (DIRS && a.din ? f32::kWantDin : 0u) |
+                        (DIRS && a.dout ? f32::kWantDout : 0u) | (a.sin ? f32::kWantSin : 0u) |
                         (a.sout ? f32::kWantSout : 0u);
   const bool dirs = want & (f32::kWantDin | f32::kWantDout);
   const uint2* src[6] = {reinterpret_cast<const uint2*>(a.x), reinterpret_cast<const uint2*>(a.y),
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_query_walk(const 
   }
 }
 
-template <int FAMILY>
+template <int FAMILY, bool RANKED = true>
 __global__ void __launch_bounds__(256) k_refine_fp64(const Desc* __restrict__ desc, QueryArgs a,
                                                      const uint32_t* __restrict__ worklist,
                                                      const unsigned long long* __restrict__ counter) {
@@ -233,13 +235,16 @@ __global__ void __launch_bounds__(256) k_refine_fp64(const Desc* __restrict__ de
     f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
     if (want & (f64::kWantDin | f64::kWantDout)) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
     f64::Result R;
-    const bool dirs = want & (f64::kWantDin | f64::kWantDout);
-    f64::query_refined<FAMILY>(S, T,
-                               f32::load_track<(FAMILY >= 2)>(
-                                   reinterpret_cast<const uint2*>(a.x), reinterpret_cast<const uint2*>(a.y),
-                                   reinterpret_cast<const uint2*>(a.z), reinterpret_cast<const uint2*>(a.u),
-                                   reinterpret_cast<const uint2*>(a.v), reinterpret_cast<const uint2*>(a.w), i, dirs),
-                               want, R);
+    if constexpr (RANKED)
+      f64::query_refined<FAMILY>(S, T,
+                                 f32::load_track<(FAMILY >= 2)>(
+                                     reinterpret_cast<const uint2*>(a.x), reinterpret_cast<const uint2*>(a.y),
+                                     reinterpret_cast<const uint2*>(a.z), reinterpret_cast<const uint2*>(a.u),
+                                     reinterpret_cast<const uint2*>(a.v), reinterpret_cast<const uint2*>(a.w), i,
+                                     want & (f64::kWantDin | f64::kWantDout)),
+                                 want, R);
+    else
+      f64::query_whole<FAMILY>(S, T, want, R);
     if (a.inside) a.inside[i] = (int8_t)R.code;
     if (a.din) a.din[i] = R.din;
     if (a.dout) a.dout[i] = R.dout;
@@ -256,8 +261,16 @@ void launch_pass32(const gv_solid* s, const QueryArgs& a, uint32_t* worklist, un
   constexpr int T = Shape32<FAMILY>::threads;
   int64_t blocks = (a.n + T - 1) / T;
   if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-  k_query_fp32<FAMILY><<<(unsigned)blocks, T, 0, stream>>>(s->d, a, worklist, counter);
+  if (FAMILY == 1 && !a.din && !a.dout)
+    k_query_fp32<1, false><<<(unsigned)blocks, T, 0, stream>>>(s->d, a, worklist, counter);
+  else
+    k_query_fp32<FAMILY><<<(unsigned)blocks, T, 0, stream>>>(s->d, a, worklist, counter);
 }
+
+// Boxes: the refinement ranks first up to here, where the longest chain of one track decides its time
+// (all five queries, ranked against whole: 200003 tracks 16.5 / 18.5, 800011 28.8 / 32.8, 3 M 74.1 / 77.9 us);
+// a longer worklist fills the GPU (8 M tracks 174.4 / 172.6 us), and codes and safeties alone are as short whole.
+constexpr int64_t kRankedBoxMax = 1 << 22;
 
 cudaError_t launch_query_fp32(const gv_solid* s, const QueryArgs& a, uint32_t* worklist,
                               unsigned long long* counter, cudaStream_t stream, int* fused_blocks) {
@@ -281,7 +294,10 @@ cudaError_t launch_query_fp32(const gv_solid* s, const QueryArgs& a, uint32_t* w
   switch (s->h.type) {
     case kBox:
       launch_pass32<0>(s, a, worklist, counter, stream, sms);
-      k_refine_fp64<0><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
+      if ((a.din || a.dout) && a.n <= kRankedBoxMax)
+        k_refine_fp64<0><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
+      else
+        k_refine_fp64<0, false><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
       break;
     case kTrd:
     case kTrap:

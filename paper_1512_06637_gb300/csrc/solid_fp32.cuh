@@ -287,7 +287,7 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
   }
   const float s = si.s;
   bool edge = false;  // GIVEN: a constraint at the band's edge is within the band
-  if (GIVEN) {
+  if constexpr (GIVEN) {
     Band m;
     for (int i = 0; i < 3; i++) m.add(g[i].g, g[i].E);
     edge = R.code == 1 && m.resolved();
@@ -297,7 +297,7 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
   R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
   R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
   if (!RANK && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
-  if (RANK) {
+  if constexpr (RANK) {
     Arg m = arg_none();
     for (int i = 0; i < 3; i++) m.add(g[i].g, g[i].E, i + 1);
     R.rank = (uint32_t)R.code | ver_safety(R.code == 1 ? (uint32_t)kNone : m.sure() ? m.id : (uint32_t)kWhole, 0);
@@ -322,24 +322,30 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
         A.e = fmaf(1.01f * fabsf(a) * T.dfl, inv, A.e);
         B.e = fmaf(fmaf(1.01f * b, T.dfl, T.fl), inv, B.e);
       }
-      const Val en = toward ? Val{-B.v, B.e} : A, ex = toward ? Val{-A.v, A.e} : B;
-      tn = vmax(tn, en);
-      tf = vmin(tf, ex);
-      if (RANK) {
+      if constexpr (RANK) {
+        const Val en = toward ? Val{-B.v, B.e} : A, ex = toward ? Val{-A.v, A.e} : B;
+        tn = vmax(tn, en);
+        tf = vmin(tf, ex);
         an.add(en.v, en.e, i + 1);
         af.add(-ex.v, ex.e, i + 1);
+      } else {
+        tn = vmax(tn, toward ? Val{-B.v, B.e} : A);
+        tf = vmin(tf, toward ? Val{-A.v, A.e} : B);
       }
     }
     // surface start: constraints within the band
-    const bool at_edge = fabsf(g[i].g + HF) <= g[i].E;
-    if (g[i].g >= -HF || (GIVEN && edge && at_edge)) {
+    if (g[i].g >= -HF || (GIVEN && edge && fabsf(g[i].g + HF) <= g[i].E)) {
       const float gd = ph[i] < 0 ? -d[i] : d[i];
       any_out |= gd > 0;
       all_in &= gd < 0;
     }
     // along or nearly along the face plane: sliding is decided in binary64
     if (fabsf(d[i]) <= TAUF + (FRAME ? 4.f * T.dfl : 0.f) && fabsf(g[i].g) <= HF + g[i].E) R.flag = true;
-    if (R.code == 1 && at_edge && !(GIVEN && edge)) R.flag = true;
+    if constexpr (GIVEN) {  // apart: as one condition it cost the plain instance 5 of 77 us (codes of 8 M tracks)
+      if (R.code == 1 && fabsf(g[i].g + HF) <= g[i].E && !edge) R.flag = true;
+    } else {
+      if (R.code == 1 && fabsf(g[i].g + HF) <= g[i].E) R.flag = true;
+    }
   }
   if (want & kWantDout) {
     if (R.code == 2) R.dout = -1.f;
@@ -373,7 +379,7 @@ __device__ inline void box32(const Desc& S, const TrackF& T, unsigned want, R32&
       } else R.din = F_INF;
     }
   }
-  if (RANK) {
+  if constexpr (RANK) {
     const bool out = R.code == 0 || (R.code == 1 && all_in);
     if (out) {
       R.rank |= kVerGoalOut;
@@ -412,7 +418,7 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
   for (int i = 0; i < 5; i++) si.add(g[i].g, g[i].E);
   const float s = si.s;
   bool edge = false;  // GIVEN: a constraint at the band's edge is within the band
-  if (GIVEN) {
+  if constexpr (GIVEN) {
     Band m;
     for (int i = 0; i < 5; i++) m.add(g[i].g, g[i].E);
     edge = R.code == 1 && m.resolved();
@@ -422,7 +428,7 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
   R.sin = R.code == 0 ? -1.f : (R.code == 1 ? 0.f : s);
   R.sout = R.code == 2 ? -1.f : (R.code == 1 ? 0.f : -s);
   if (!RANK && R.code != 1 && !certified({fabsf(s), si.err()})) R.flag = true;
-  if (RANK) {
+  if constexpr (RANK) {
     Arg m = arg_none();
     for (int i = 0; i < 5; i++) m.add(g[i].g, g[i].E, i + 1);
     R.rank = (uint32_t)R.code | ver_safety(R.code == 1 ? (uint32_t)kNone : m.sure() ? m.id : (uint32_t)kWhole, 0);
@@ -447,7 +453,7 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
     const bool entry = gd[i] < 0;
     tn = vmax(tn, entry ? tv : Val{-BIG, 0.f});
     tf = vmin(tf, entry ? Val{BIG, 0.f} : tv);
-    if (RANK) {
+    if constexpr (RANK) {
       if (entry) an.add(tv.v, tv.e, i + 1);
       else af.add(-tv.v, tv.e, i + 1);
     }
@@ -467,12 +473,15 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
         A.e = fmaf(1.01f * fabsf(a) * T.dfl, iw, A.e);
         B.e = fmaf(fmaf(1.01f * b, T.dfl, T.fl), iw, B.e);
       }
-      const Val en = toward ? Val{-B.v, B.e} : A, ex = toward ? Val{-A.v, A.e} : B;
-      tn = vmax(tn, en);
-      tf = vmin(tf, ex);
-      if (RANK) {
+      if constexpr (RANK) {
+        const Val en = toward ? Val{-B.v, B.e} : A, ex = toward ? Val{-A.v, A.e} : B;
+        tn = vmax(tn, en);
+        tf = vmin(tf, ex);
         an.add(en.v, en.e, 5);
         af.add(-ex.v, ex.e, 5);
+      } else {
+        tn = vmax(tn, toward ? Val{-B.v, B.e} : A);
+        tf = vmin(tf, toward ? Val{-A.v, A.e} : B);
       }
     }
   }
@@ -519,7 +528,7 @@ __device__ inline void planar32(const Desc& S, const TrackF& T, unsigned want, R
       } else R.din = F_INF;
     }
   }
-  if (RANK) {
+  if constexpr (RANK) {
     const bool out = R.code == 0 || (R.code == 1 && all_in);
     if (out) {
       R.rank |= kVerGoalOut;
@@ -847,7 +856,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
   if (has_phi) si.add_int(gphi, phlo, phhi);
   const float s = si.s;
   bool edge = false;  // GIVEN: a constraint at the band's edge is within the band
-  if (GIVEN) {
+  if constexpr (GIVEN) {
     Band m;
     m.add(lo_.g, lo_.E);
     if (has_in) m.add(li_.g, li_.E);
@@ -866,7 +875,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
     R.code = decide(si, R.flag);
   }
   if (FRAME && near_plane) R.flag = true;
-  if (RANK) {
+  if constexpr (RANK) {
     R.rank = (uint32_t)R.code;
     R.te = 0.f;
     R.se = R.code == 1 ? 0.f : si.err();
@@ -911,7 +920,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
         c.add(gk0, Ek0);
         c.add(gk1, Ek1);
         if (has_phi) c.add_int(gphi, phlo, phhi);
-        if (RANK) {
+        if constexpr (RANK) {
           m.add(gk0, Ek0, kZLow);
           m.add(gk1, Ek1, kZHigh);
           if (has_phi) m.add(ph.g, ph.E, phk);
@@ -924,7 +933,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
         const Val c = closed_df(k0, kind);
         R.sout = -c.v;
         if (!RANK && !certified({fabsf(c.v), c.e})) R.flag = true;
-        if (RANK) {
+        if constexpr (RANK) {
           R.rank |= ver_safety(kind, k0);
           R.se = c.e;
         }
@@ -993,7 +1002,7 @@ __device__ inline bool pcon_begin(const Desc& S, const TrackF& T, unsigned want,
         }
         R.sin = best.v;
         if (!RANK && !certified(best)) R.flag = true;
-        if (RANK) {
+        if constexpr (RANK) {
           R.rank |= m.sure() ? ver_safety(mkind, (int)m.id) : ver_safety(kWhole, kAllPieces);
           R.se = best.e;
         }
@@ -1264,7 +1273,7 @@ __device__ inline void pcon_step(const Desc& S, const TrackF& T, Walk& W) {
         W.ans = t;
         W.answered = true;
         W.st = kDone;
-        if (RANK) {
+        if constexpr (RANK) {
           // an entry by the section's slab is one by the solid's first plane along the ray
           const bool first = (step > 0 && k == 0) || (step < 0 && k + 1 == last);
           const uint32_t zid = !first ? (uint32_t)kNone : ver_dist(kZLow, step > 0 ? 0 : last);
@@ -1325,7 +1334,7 @@ template <bool RANK = false>
 __device__ inline void pcon_end(const Walk& W, R32& R) {
   bool u = W.u;
   if (W.st == kStretch) u = true;  // a stretch must end at a surface
-  if (RANK) {
+  if constexpr (RANK) {
     if ((W.need_out || W.need_in) && (u || (W.need_out && !W.answered && R.code == 0))) R.flag = true;
     if (W.answered) R.rank |= W.did;
     R.te = W.answered ? W.ans.e : 0.f;
@@ -1348,7 +1357,7 @@ __device__ inline void pcon_end(const Walk& W, R32& R) {
 template <bool TUBE, bool FRAME = false, bool RANK = false, bool GIVEN = false>
 __device__ inline void pcon32(const Desc& S, const TrackF& T, unsigned want, R32& R) {
   Walk W;
-  W.answered = false;
+  if (RANK) W.answered = false;
   if (pcon_begin<TUBE, FRAME, RANK, GIVEN>(S, T, want, R, W))
     while (W.live) pcon_step<TUBE, FRAME, RANK>(S, T, W);
   pcon_end<RANK>(W, R);
