@@ -104,6 +104,7 @@ struct gv_geom {
   float* d_safe_cut = nullptr;
   bool use_vox = true;
   bool walk32 = false;  // some node with a grid has at least kWalk32Min daughters
+  bool never = false;   // some node has a daughter without a binary32 form
   std::vector<gv::NodeD> nodes;
   std::vector<gv::Cull> cull;
   std::vector<int32_t> children;
@@ -1466,6 +1467,12 @@ __device__ __forceinline__ int pool_kinds(const Geo& g, StepPool<SLOTS>& Q, int*
 // The binary64 step of the tracks 0..n-1, or (wl) of the n listed ones, in tiles of at most SLOTS
 // tracks per block, short ones spread over every block.
 constexpr int kNavSlots = 1024, kNavThreads = 1024;
+// Binary32 baskets of at most this many tracks do not fill the GPU one thread per track: 8 lanes take a
+// track (k_nav_fp32; not where volumes have daughters without a binary32 form, which go to binary64 at
+// once), and what is left goes to k_nav_exact.  Measured (GB300, with safety, against k_nav_scan32 and
+// k_nav_pool): nested detector, 300 tracks 46 -> 31 us, 8000 tracks 54 -> 36 us (20011: 70 against 53 us);
+// 512 daughters of all kinds, 300 tracks 1530 -> 697 us, 8000 tracks 1895 -> 928 us.
+constexpr int64_t kShortBasket = 8192;
 __global__ void __launch_bounds__(kNavThreads, 1) k_nav_pool(Geo g, NavArgs a, const uint32_t* __restrict__ wl,
                                                               const unsigned long long* __restrict__ cnt) {
   extern __shared__ __align__(16) unsigned char pool_bytes[];
@@ -1520,6 +1527,27 @@ __global__ void __launch_bounds__(kNavThreads, 1) k_nav_pool(Geo g, NavArgs a, c
       a.next[i] = o.next;
     }
     __syncthreads();  // the pool is reused by the next tile
+  }
+}
+
+// The listed tracks evaluated whole, one per thread, consecutive ones in consecutive blocks of one
+// warp: the refinement of baskets up to kShortBasket, whose few tracks the pool's phases would only delay.
+// Bound by the latency of one track's chain (blocks of 64 threads, one per SM: 958 against 731 us for 3000
+// tracks among 512 daughters).
+__global__ void __launch_bounds__(32) k_nav_exact(Geo g, NavArgs a, const uint32_t* __restrict__ wl,
+                                                  const unsigned long long* __restrict__ cnt) {
+  const int64_t m = (int64_t)*cnt, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; j < m; j += stride) {
+    const int64_t i = wl[j];
+    const int32_t v = a.node[i];
+    Step o{-1.0, -1.0, 0.0, -1};
+    if (v >= 0 && v < g.nnodes) {
+      const double p[3] = {a.x[i], a.y[i], a.z[i]}, d[3] = {a.u[i], a.v[i], a.w[i]};
+      nav_exact(g, v, p, d, a.safety != nullptr, o);
+    }
+    a.step[i] = o.step;
+    if (a.safety) a.safety[i] = o.safety;
+    a.next[i] = o.next;
   }
 }
 
@@ -2009,7 +2037,10 @@ static void build_cull(gv_geom* g) {
     else if (h.type == kBox) C.tag = kCullBox;
     else if (h.type == kTube && !(h.flags & kHasPhi)) C.tag = kCullTube;
     else C.tag = kCullOther;
-    if (C.tag == kCullNever && N.parent >= 0) g->nodes[N.parent].never = 1;
+    if (C.tag == kCullNever && N.parent >= 0) {
+      g->nodes[N.parent].never = 1;
+      g->never = true;
+    }
     if (C.tag == kCullTube && (h.inner & 1u)) C.rmin = (float)h.in[0].b;  // a = 0: the radius
   }
 }
@@ -2216,7 +2247,8 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
     cudaError_t e = cudaMemsetAsync(ws->counter, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return cuda_error(e, "nav: counter reset");
     const Vox vox = vox_of(g);
-    if (vox.grids && g->walk32) {
+    const bool brief = t->n <= kShortBasket;
+    if ((vox.grids && g->walk32) || (brief && !g->never)) {
       const int64_t per_block = 256 / kLanes;
       const int64_t blocks = std::min<int64_t>((t->n + per_block - 1) / per_block, (int64_t)sms * 8);
       k_nav_fp32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
@@ -2226,7 +2258,8 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
       k_nav_scan32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
                                                      ws->idx, ws->counter, vox);
     }
-    e = launch_nav_pool(g, a, sms, ws->idx, ws->counter, st);
+    if (brief) k_nav_exact<<<(unsigned)std::min<int64_t>(t->n, (int64_t)sms * 4), 32, 0, st>>>(geo_of(g), a, ws->idx, ws->counter);
+    else e = launch_nav_pool(g, a, sms, ws->idx, ws->counter, st);
     if (e != cudaSuccess) return cuda_error(e, "nav launch");
   }
   const cudaError_t e = cudaGetLastError();
