@@ -248,7 +248,10 @@ __global__ void __launch_bounds__(kRankThreads, ITEMS == 1 ? 512 / kRankThreads 
 // Measured (box minus tube segment, 2^20 tracks, all five queries): 1213 -> 290 us (before: every piece of
 // both components in binary64, 594 FP64 warp instructions per 32 tracks); ranked but in index order
 // 365 us (139 FP64 warp instructions).  The ranking inlined: 296 us (spills).
-template <int ITEMS>
+// PARTS: every block takes an equal, contiguous part of the basket instead of tiles in turn.  Up to three
+// tiles per block this evens out the last round (400000 tracks 151 -> 127 us, 700000 215 -> 187 us); beyond, or
+// without distances in short rows, tiles in turn are as even and up to 8% faster.
+template <int ITEMS, bool PARTS>
 __global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restrict__ desc, QueryArgs a) {
   constexpr int TILE = 256 * ITEMS;
   constexpr uint32_t NC = f64::kBoolClasses;
@@ -285,8 +288,11 @@ __global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restri
       store(open[q], R);
     }
   };
-  for (int64_t t0 = (int64_t)blockIdx.x * TILE; t0 < a.n; t0 += (int64_t)gridDim.x * TILE) {  // block-uniform
-    const int len = a.n - t0 < TILE ? (int)(a.n - t0) : TILE;
+  // tiles in turn, or an equal, contiguous part of the basket
+  const int64_t share = PARTS ? ((a.n + gridDim.x - 1) / gridDim.x + 31) / 32 * 32 : TILE;
+  const int64_t end = PARTS ? min((int64_t)(blockIdx.x + 1) * share, a.n) : a.n;
+  for (int64_t t0 = (int64_t)blockIdx.x * share; t0 < end; t0 += PARTS ? TILE : (int64_t)gridDim.x * TILE) {  // block-uniform
+    const int len = end - t0 < TILE ? (int)(end - t0) : TILE;
     if (tid < (int)NC) cnt[tid] = 0u;
     __syncthreads();
     for (int j = tid; j < len; j += 256) {
@@ -517,6 +523,15 @@ static int64_t tiles_grid(int64_t tiles, int sms) {
   return tiles < (int64_t)sms * occ ? tiles : (int64_t)sms * occ;
 }
 
+// Booleans rank from more than this many tracks on.  Up to one block of 256 threads per SM a whole evaluation
+// takes the time of one chain, and ranking only adds its own: five random booleans of 20000 tracks, all
+// queries, ranked / whole 39 / 35, 43 / 43, 64 / 62, 51 / 49, 37 / 33 us; 40000 tracks 39 / 60, 43 / 78, 64 / 110, 53 / 84,
+// 39 / 58 us.  Codes and safeties alone are shorter: 80000 tracks, codes 22.4 / 20.5, 22.5 / 18.5, 24.4 / 26.7 us,
+// safeties 28.8 / 30.8, 26.3 / 29.8, 34.9 / 43.1 us; 400000 tracks, codes 53 / 64, 53 / 58, 57 / 86 us.
+static int64_t bool_rank_min(const QueryArgs& a, int sms) {
+  return (int64_t)sms * (a.din || a.dout ? 256 : a.sin || a.sout ? 512 : 1024);
+}
+
 cudaError_t launch_query_fp64(const gv_solid* s, const QueryArgs& a, cudaStream_t stream) {
   if (a.n == 0) return cudaSuccess;
   const int threads = 256;
@@ -566,10 +581,13 @@ cudaError_t launch_query_fp64(const gv_solid* s, const QueryArgs& a, cudaStream_
     case kTrd:
     case kTrap: k_query_fp64<1><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a); break;
     case kBool:
-      if (f64::bool_ranks(s->ph[0], s->ph[1])) {
-        const int64_t resident = (int64_t)sms * 2, tiles = (a.n + 1023) / 1024;
-        if (tiles >= resident) k_query_bool_rank<4><<<(unsigned)resident, 256, 0, stream>>>(s->d, a);
-        else k_query_bool_rank<1><<<(unsigned)(blocks < resident ? blocks : resident), 256, 0, stream>>>(s->d, a);
+      if (a.n > bool_rank_min(a, sms) && f64::bool_ranks(s->ph[0], s->ph[1])) {
+        const int64_t resident = (int64_t)sms * 2;
+        const unsigned grid = (unsigned)resident;
+        if (a.n >= resident * 3072) k_query_bool_rank<4, false><<<grid, 256, 0, stream>>>(s->d, a);
+        else if (a.n >= resident * 1024) k_query_bool_rank<4, true><<<grid, 256, 0, stream>>>(s->d, a);
+        else if (a.din || a.dout) k_query_bool_rank<1, true><<<grid, 256, 0, stream>>>(s->d, a);
+        else k_query_bool_rank<1, false><<<grid, 256, 0, stream>>>(s->d, a);
       } else {
         k_query_fp64<4><<<(unsigned)blocks, threads, 0, stream>>>(s->d, a);
       }
