@@ -189,7 +189,8 @@ gv_status gv_pipeline_join(gv_pipeline* p, void* stream);
  * in the same kind of volume into baskets and hands them to the geometry.  A
  * batch holds many such baskets, each against its own solid, over one shared
  * structure-of-arrays track set, and evaluates all of them with persistent
- * kernels replayed from a CUDA graph: GV_FP64 one kernel over all tiles;
+ * kernels replayed from a CUDA graph: GV_FP64 one kernel over all tiles, and one of its
+ * own on a parallel branch for booleans and fine-featured solids;
  * GV_FP32_REFINE one kernel per solid family present (box; trd/trap; tube;
  * one-section cone; multi-section polycone, with lane refill; boolean, in
  * binary64) on parallel graph branches, then the binary64 worklist pass. */

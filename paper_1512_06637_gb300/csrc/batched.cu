@@ -13,7 +13,8 @@
 // one to several sections); booleans, which have no binary32 form, are evaluated
 // in binary64 directly.  Uncertain tracks of every solid go to one worklist of
 // (solid, track) pairs that a last kernel recomputes in binary64.  Binary64: one
-// persistent kernel over all tiles.  An autotuner picks the tile length and the
+// persistent kernel over the tiles of all solids that rank, and on a parallel branch the
+// boolean family's.  An autotuner picks the tile length and the
 // resident CTAs per SM (and, in binary64, the block size) by timing graph replays.
 #include <algorithm>
 #include <cstdio>
@@ -26,6 +27,7 @@
 #include "rank_fp64.cuh"
 #include "solid_fp32.cuh"
 #include "solid_fp64.cuh"
+#include "work_class.cuh"
 
 namespace gv {
 
@@ -44,8 +46,8 @@ __device__ __forceinline__ void stage_any(Desc& dst, const Desc* __restrict__ sr
 // The binary64 pass: a CTA takes a tile, stages the tile's solid when it changes, ranks the tile's tracks
 // in binary32 (rank_fp64.cuh), orders them by the binary64 work their verdicts ask for and evaluates that,
 // as the single-solid pass does; the bits are those of the whole evaluation in any order.  Tracks
-// without a certain verdict, booleans and solids binary32 does not resolve gather on the CTA's list as
-// (solid, track) pairs and are evaluated whole, one per thread, when it is full and at the end.
+// without a certain verdict gather on the CTA's list as (solid, track) pairs and are evaluated whole, one
+// per thread, when it is full and at the end.  (Booleans and solids binary32 does not resolve: k_bbool64.)
 // Measured (GB300, 4096 baskets over 64 solids, 2.9 M tracks, all five queries): 2508 -> 712 us; 64 baskets
 // 315 -> 54 us (before: every candidate in binary64, tiles ordered by class).
 constexpr int kBatchItems = 4;     // tracks per thread ranked at once (a longer tile goes in parts)
@@ -105,21 +107,17 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_batched(const Desc* 
       __syncthreads();
       const int type = S.type;
       const bool planar = type == kBox || type == kTrd || type == kTrap;
-      const bool ranks = type != kBool && !(S.flags & kFp64Only);
       auto cls = [&](uint32_t V) {
         return planar ? f64::rank_class<0>(f64::Verdict{V}) : f64::rank_class<3>(f64::Verdict{V});
       };
       for (int j = tid; j < len; j += THREADS) {
         const int64_t i = first + j;
         f32::R32 R;
-        R.flag = !ranks;
-        if (ranks) {
-          const f32::TrackF T = f32::load_track<true>(X, Y, Z, Ux, Uy, Uz, i, dirs);
-          if (type == kBox) f64::rank32<0>(S, T, want, R);
-          else if (planar) batch_rank<1>(S, T, want, R);
-          else if (type == kTube) batch_rank<2>(S, T, want, R);
-          else batch_rank<3>(S, T, want, R);
-        }
+        const f32::TrackF T = f32::load_track<true>(X, Y, Z, Ux, Uy, Uz, i, dirs);
+        if (type == kBox) f64::rank32<0>(S, T, want, R);
+        else if (planar) batch_rank<1>(S, T, want, R);
+        else if (type == kTube) batch_rank<2>(S, T, want, R);
+        else batch_rank<3>(S, T, want, R);
         ver[j] = R.flag ? kBatchOpen : R.rank;
         if (R.flag) open[atomicAdd(&nopen, 1u)] = ((unsigned long long)(unsigned)tl.solid << 40) | (unsigned long long)i;
         else atomicAdd(&cnt[cls(R.rank)], 1u);
@@ -383,34 +381,79 @@ __global__ void __launch_bounds__(BShape<kFamWalk>::threads, BShape<kFamWalk>::b
   }
 }
 
-// Booleans and solids with features finer than binary32 resolves: binary64 directly, one
-// track per thread.
+// Booleans and solids with features finer than binary32 resolves, in both precisions: binary64 throughout,
+// one track per thread.  Booleans against the tile's staged record and in order of work class (warps of
+// tracks that miss the bounding box are short): 16, 512 and 4096 baskets in binary64 571, 1322, 6929 -> 304,
+// 1165, 6329 us (GB300; before on the ranked kernel's list, records in global memory).  The others in index
+// order (4096 baskets of thin tubes 2397 us; in order of class 2459 us, staged in index order 3220 us).
 __global__ void __launch_bounds__(BShape<kFamBool>::threads, BShape<kFamBool>::blocks)
     k_bbool64(const Desc* __restrict__ solids, const Tile* __restrict__ tiles, int ntiles, unsigned* __restrict__ next,
               QueryArgs a) {
-  constexpr int THREADS = BShape<kFamBool>::threads;
+  constexpr int THREADS = BShape<kFamBool>::threads, PART = 2048;
+  constexpr uint32_t NC = f32::kClasses;
+  __shared__ Desc S;
   __shared__ int s_tile;
+  __shared__ uint16_t ord[PART];
+  __shared__ uint8_t cls[PART];
+  __shared__ unsigned cnt[NC];
+  const int tid = threadIdx.x;
   const unsigned want = want_of(a);
+  const bool dirs = want & 6u;
+  auto hi = [](const double* p, int64_t i) {
+    bool bad = false;  // a value outside the binary32 range only lands in some class
+    return f32::trunc_hi(__ldg(reinterpret_cast<const uint2*>(p) + i), bad);
+  };
+  int loaded = -1;
   for (;;) {
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(next, 1u);
+    if (tid == 0) s_tile = (int)atomicAdd(next, 1u);
     __syncthreads();
     const int t = s_tile;
     if (t >= ntiles) break;
     const Tile tl = tiles[t];
-    const Desc& S = solids[tl.solid];
-    for (int j = threadIdx.x; j < tl.len; j += THREADS) {
-      const int64_t i = tl.start + j;
-      f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
-      if (want & 6u) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
-      f64::Result R;
-      f64::query(S, T, want, R);
-      if (a.inside) a.inside[i] = (int8_t)R.code;
-      if (a.din) a.din[i] = R.din;
-      if (a.dout) a.dout[i] = R.dout;
-      if (a.sin) a.sin[i] = R.sin;
-      if (a.sout) a.sout[i] = R.sout;
+    if (tl.solid != loaded) {
+      stage_any(S, solids + tl.solid);
+      loaded = tl.solid;
     }
-    __syncthreads();
+    for (int part = 0; part < tl.len; part += PART) {
+      const int len = min(tl.len - part, PART);
+      const int64_t first = tl.start + part;
+      if (tid < (int)NC) cnt[tid] = 0u;
+      __syncthreads();
+      const bool order = S.type == kBool;  // block-uniform
+      for (int j = tid; order && j < len; j += THREADS) {
+        const int64_t i = first + j;
+        const uint32_t c = f32::track_class(S, hi(a.x, i), hi(a.y, i), hi(a.z, i), dirs ? hi(a.u, i) : 0.f,
+                                            dirs ? hi(a.v, i) : 0.f, dirs ? hi(a.w, i) : 0.f, dirs);
+        cls[j] = (uint8_t)c;
+        atomicAdd(&cnt[c], 1u);
+      }
+      __syncthreads();
+      if (tid == 0) {
+        unsigned run = 0;
+        for (uint32_t q = 0; q < NC; q++) {
+          const unsigned c = cnt[q];
+          cnt[q] = run;
+          run += c;
+        }
+      }
+      __syncthreads();
+      for (int j = tid; order && j < len; j += THREADS) ord[atomicAdd(&cnt[cls[j]], 1u)] = (uint16_t)j;
+      __syncthreads();
+      for (int p = tid; p < len; p += THREADS) {
+        const int64_t i = first + (order ? (int)ord[p] : p);
+        f64::Track T{a.x[i], a.y[i], a.z[i], 0, 0, 0};
+        if (dirs) { T.u = a.u[i]; T.v = a.v[i]; T.w = a.w[i]; }
+        f64::Result R;
+        if (order) f64::bool_query(S, T, want, R);
+        else f64::prim_query(solids[tl.solid], T, want, R);
+        if (a.inside) a.inside[i] = (int8_t)R.code;
+        if (a.din) a.din[i] = R.din;
+        if (a.dout) a.dout[i] = R.dout;
+        if (a.sin) a.sin[i] = R.sin;
+        if (a.sout) a.sout[i] = R.sout;
+      }
+      __syncthreads();  // the part's shared arrays, the tile number and the record are replaced
+    }
   }
 }
 
@@ -547,9 +590,10 @@ static gv_status build_tiles(gv_batch* b) {
     }
     b->fam_count[f] = (int)t.size() - b->fam_first[f];
   }
-  // then the binary64 kernel's tiles: every basket in order, tiles of the configured length
+  // then the ranked binary64 kernel's tiles: every other basket in order, tiles of the configured length
   b->first64 = (int)t.size();
-  for (const gv_basket& k : b->baskets)
+  for (const gv_basket& k : b->baskets) {
+    if (b->solid_fam[k.solid] == kFamBool) continue;
     for (int64_t off = 0; off < k.n; off += tile) {
       Tile x;
       x.start = k.offset + off;
@@ -557,6 +601,7 @@ static gv_status build_tiles(gv_batch* b) {
       x.solid = k.solid;
       t.push_back(x);
     }
+  }
   b->ntiles64 = (int)t.size() - b->first64;
   if ((int64_t)t.size() > b->tile_cap) return set_error(GV_ERR_INVALID_ARG, "batch: too many tiles");
   b->ntiles = (int)t.size();
@@ -592,8 +637,22 @@ static gv_status capture(gv_batch* b, const QueryArgs& a, int prec) {
   if (le == cudaSuccess && fp64) {
     const int occ = occupancy(b->cfg.threads);
     const int per_sm = b->cfg.ctas_per_sm > 0 ? std::min(b->cfg.ctas_per_sm, occ) : occ;
-    le = launch_batched(b->cfg.threads, std::max(1, per_sm * sm_count()), b->d_solids, b->d_tiles + b->first64, b->ntiles64,
-                        b->d_next, a, b->cap_stream);
+    const bool whole = b->fam_count[kFamBool] > 0;  // on a branch of their own
+    if (whole) {
+      cudaStream_t fs = b->fam_stream[kFamBool];
+      le = cudaEventRecord(b->fork_ev, b->cap_stream);
+      if (le == cudaSuccess) le = cudaStreamWaitEvent(fs, b->fork_ev, 0);
+      if (le == cudaSuccess)
+        le = launch_family(kFamBool, b->cfg.ctas_per_sm, b->d_solids, b->d_tiles + b->fam_first[kFamBool], b->fam_count[kFamBool],
+                           b->d_next + 1 + kFamBool, a, nullptr, nullptr, fs);
+    }
+    if (le == cudaSuccess && b->ntiles64 > 0)
+      le = launch_batched(b->cfg.threads, std::max(1, per_sm * sm_count()), b->d_solids, b->d_tiles + b->first64, b->ntiles64,
+                          b->d_next, a, b->cap_stream);
+    if (le == cudaSuccess && whole) {
+      le = cudaEventRecord(b->join_ev[kFamBool], b->fam_stream[kFamBool]);
+      if (le == cudaSuccess) le = cudaStreamWaitEvent(b->cap_stream, b->join_ev[kFamBool], 0);
+    }
   }
   if (le == cudaSuccess && !fp64) {
     // the families on parallel branches, each followed by the binary64 pass over its own
