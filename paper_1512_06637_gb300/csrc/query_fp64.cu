@@ -486,10 +486,11 @@ static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaSt
 }
 
 // Tiles of 2048 tracks when every resident block gets four of them, of 1024 when it gets one; shorter
-// baskets one track per thread, except tubes and cones from 1024 tracks per SM on, which gain from
-// ordering already (tile of 256: measured, all five queries, against one track per thread: 50021 tracks
-// tube 25.9 / 24.9, cone 22.2 / 19.5, polycone 32.4 / 27.2 us; 200000 tracks tube 52.1 / 56.2, cone 46.7 /
-// 48.1, box 16.2 / 12.4, trap 31.6 / 28.2 us).
+// baskets one track per thread, except the distances of tubes and cones from 1024 tracks per SM on, which
+// gain from ordering already (tile of 256: measured, all five queries, against one track per thread: 50021
+// tracks tube 25.9 / 24.9, cone 22.2 / 19.5, polycone 32.4 / 27.2 us; 200000 tracks tube 52.1 / 56.2, cone
+// 46.7 / 48.1, box 16.2 / 12.4, trap 31.6 / 28.2 us; without distances 200003 tracks of the cone, codes
+// 12.3 / 8.2, safeties 19.7 / 18.1 us).
 template <int FAMILY>
 static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaStream_t stream) {
   constexpr bool kOrdered = FAMILY == 2 || FAMILY == 4;
@@ -500,7 +501,7 @@ static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaSt
     launch_rank64<FAMILY, 4>(s, a, sms, stream);
   } else {
     if constexpr (kOrdered) {
-      if (a.n >= (int64_t)sms * 1024) {
+      if ((a.din || a.dout) && a.n >= (int64_t)sms * 1024) {
         launch_rank64<FAMILY, 1>(s, a, sms, stream);
         return;
       }
