@@ -934,6 +934,8 @@ __global__ void __launch_bounds__(256, 2) k_nav_scan32(const NodeD* __restrict__
 // most of them, and the frame change and pass of the rest bound the walk.  Measured (GB300, 1728
 // daughters, 2^18 tracks without safety, the same bits): 10.8 -> 4.2 ms; 1000 daughters, 10^5 tracks:
 // 4.8 -> 2.0 ms.  Leaving the walk at the first flag gained nothing.
+// WALK false: every node is scanned (short baskets; one instance for both cost 300 tracks 2 of 29 us).
+template <bool WALK>
 __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ nodes, const int32_t* __restrict__ children,
                                                   const Desc* __restrict__ solids, const Cull* __restrict__ cull,
                                                   int nnodes, NavArgs a,
@@ -962,7 +964,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
     const int64_t i = base + sperm[threadIdx.x / kLanes];
     const bool valid = i < a.n;
     bool flag = false;
-    Top2<true> top{F_INF, 0.f, F_INF, 0.f, kNone, kNone};
+    Top2<WALK> top{F_INF, 0.f, F_INF, 0.f, kNone, kNone};
     float saf = F_INF;
     int32_t v = -1;
     bool walked = false;  // keys are node indices (grid walk) rather than daughter order
@@ -972,7 +974,7 @@ __global__ void __launch_bounds__(256, 2) k_nav_fp32(const NodeD* __restrict__ n
         flag = true;
       } else {
         const NodeD& N = nodes[v];
-        walked = vox.grids && N.grid >= 0 && N.count >= kWalk32Min;
+        walked = WALK && vox.grids && N.grid >= 0 && N.count >= kWalk32Min;
         flag = N.never && (want_saf || !walked);  // a daughter without binary32 form would be met: binary64
       }
     }
@@ -1468,9 +1470,9 @@ __device__ __forceinline__ int pool_kinds(const Geo& g, StepPool<SLOTS>& Q, int*
 // tracks per block, short ones spread over every block.
 constexpr int kNavSlots = 1024, kNavThreads = 1024;
 // Binary32 baskets of at most this many tracks do not fill the GPU one thread per track: 8 lanes take a
-// track (k_nav_fp32; not where volumes have daughters without a binary32 form, which go to binary64 at
-// once), and what is left goes to k_nav_exact.  Measured (GB300, with safety, against k_nav_scan32 and
-// k_nav_pool): nested detector, 300 tracks 46 -> 31 us, 8000 tracks 54 -> 36 us (20011: 70 against 53 us);
+// track (k_nav_fp32; not where volumes have 128 daughters and more to scan, or daughters without a binary32
+// form, which go to binary64 at once), and what is left goes to k_nav_exact.  Measured (GB300, with safety, against k_nav_scan32 and
+// k_nav_pool): nested detector, 300 tracks 46 -> 30 us, 8000 tracks 54 -> 35 us (16000: 54.1 against 53.1 us);
 // 512 daughters of all kinds, 300 tracks 1530 -> 697 us, 8000 tracks 1895 -> 928 us.
 constexpr int64_t kShortBasket = 8192;
 __global__ void __launch_bounds__(kNavThreads, 1) k_nav_pool(Geo g, NavArgs a, const uint32_t* __restrict__ wl,
@@ -2248,11 +2250,12 @@ gv_status gv_nav_step(const gv_geom* g, const gv_tracks* t, const int32_t* node,
     if (e != cudaSuccess) return cuda_error(e, "nav: counter reset");
     const Vox vox = vox_of(g);
     const bool brief = t->n <= kShortBasket;
-    if ((vox.grids && g->walk32) || (brief && !g->never)) {
+    const bool walk = vox.grids && g->walk32;
+    if (walk || (brief && !g->never && !g->walk32)) {
       const int64_t per_block = 256 / kLanes;
       const int64_t blocks = std::min<int64_t>((t->n + per_block - 1) / per_block, (int64_t)sms * 8);
-      k_nav_fp32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
-                                                         ws->idx, ws->counter, vox);
+      (walk ? k_nav_fp32<true> : k_nav_fp32<false>)<<<(unsigned)blocks, 256, 0, st>>>(
+          g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a, ws->idx, ws->counter, vox);
     } else {
       const int64_t blocks = std::min<int64_t>((t->n + 255) / 256, (int64_t)sms * 2);
       k_nav_scan32<<<(unsigned)blocks, 256, 0, st>>>(g->d_nodes, g->d_children, g->d_solids, g->d_cull, g->nnodes, a,
