@@ -268,9 +268,9 @@ void launch_pass32(const gv_solid* s, const QueryArgs& a, uint32_t* worklist, un
 }
 
 // Boxes: the refinement ranks first up to here, where the longest chain of one track decides its time
-// (all five queries, ranked against whole: 200003 tracks 16.5 / 18.5, 800011 28.8 / 32.8, 3 M 74.1 / 77.9 us);
-// a longer worklist fills the GPU (8 M tracks 174.4 / 172.6 us), and codes and safeties alone are as short whole.
-constexpr int64_t kRankedBoxMax = 1 << 22;
+// (all five queries, ranked against whole: 200003 tracks 16.5 / 18.5, 800011 28.8 / 32.8, 1.6 M 47.2 / 49.3 us);
+// a longer worklist fills the GPU (8 M tracks 174.4 / 172.6 us; without DistanceToOut 3.6 M tracks 87 / 84 us), and codes and safeties alone are as short whole.
+constexpr int64_t kRankedBoxMax = 1 << 21;
 
 cudaError_t launch_query_fp32(const gv_solid* s, const QueryArgs& a, uint32_t* worklist,
                               unsigned long long* counter, cudaStream_t stream, int* fused_blocks) {
@@ -318,7 +318,8 @@ cudaError_t launch_query_fp32(const gv_solid* s, const QueryArgs& a, uint32_t* w
         k_query_walk<3><<<wblocks, kWalkThreads, 0, stream>>>(s->d, a, worklist, counter);
       else
         launch_pass32<3>(s, a, worklist, counter, stream, sms);
-      if (s->h.nz > 2) k_refine_fp64<3><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
+      if (s->h.nz > 2 && !a.din && !a.dout) k_refine_fp64<3, false><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
+      else if (s->h.nz > 2) k_refine_fp64<3><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
       else k_refine_fp64<4><<<rblocks, threads, 0, stream>>>(s->d, a, worklist, counter);
       break;
   }
