@@ -61,7 +61,7 @@ FP64_CAPTURE = {
     "fp64_warp_inst_per_track": {'tube': 10.47, 'cone': 7.29},
     "profile": "profiles/query_fp64_tube_cone_1M_pipe.md",
 }
-FP64_KERNEL_SOURCES = ("solid_fp64.cuh", "query_fp64.cu", "gv_desc.h", "work_class.cuh")
+FP64_KERNEL_SOURCES = ("solid_fp64.cuh", "rank_fp64.cuh", "solid_fp32.cuh", "query_fp64.cu", "gv_desc.h")
 E2E_CHUNK = 1 << 22  # tracks per host-streaming chunk (2^19-2^22 measured: larger is faster)
 E2E_SLOTS = 3
 

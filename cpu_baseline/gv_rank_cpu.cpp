@@ -109,7 +109,9 @@ extern "C" void gvcpu_bool(int op, const void* a, const void* c, const double* R
     if (dirs) { T.u = tr[3][i]; T.v = tr[4][i]; T.w = tr[5][i]; }
     f64::Result r{0, 0, 0, 0, 0}, q{0, 0, 0, 0, 0};
     f64::bool_query(S, T, want, r);
-    ranked[i] = forms && f64::bool_ranked(S, parts[0], parts[1], T, want, q);
+    uint32_t V;
+    ranked[i] = forms && f64::bool_verdict(S, parts[0], parts[1], T, want, V);
+    if (ranked[i]) f64::bool_evaluate(S, parts[0], parts[1], T, f64::BoolVerdict{V}, q);
     const double w[5] = {(double)r.code, r.din, r.dout, r.sin, r.sout}, o[5] = {(double)q.code, q.din, q.dout, q.sin, q.sout};
     for (int k = 0; k < 5; k++) { whole[5 * i + k] = w[k]; got[5 * i + k] = o[k]; }
   }

@@ -257,14 +257,17 @@ int32_t gv_geom_node_count(const gv_geom* g);
  * and a navigation step in such a node walks the cells along the ray in order of
  * entry (3-D DDA), evaluating DistanceToIn of the listed daughters and stopping once
  * the best distance so far lies more than 4e-9 (1 + best) mm before the next cell.
- * SafetyToIn is still taken over every daughter (the step's safety is a minimum over
- * all of them; pass safety = NULL to leave it out).  Binary64 results (locate, step,
- * safety, next, transport) are bit-identical with grids on or off: the walk sees every
- * daughter that could give the minimum or tie with it, and ties are broken by the
- * same rule.  GV_FP32_REFINE steps in a node with at least 128 daughters walk the
- * grid in binary32 with certified bounds (below that, 8 lanes per track scan them all):
- * next is the same with grids on or off, step and safety within that precision's
- * tolerance (a track certain on the walk may be refined without it, or the reverse).
+ * The step's safety is a minimum over all daughters: where a volume has 128 daughters and
+ * more, GV_FP64 steps take the candidates for it from lists of the nearest daughters kept with
+ * the grid's cells (up to 8192 daughters and 135 MB per geometry; a geometry that finds no
+ * memory for them, and larger volumes, scan the daughters); pass safety = NULL to leave it
+ * out.  Binary64 results (locate, step, safety, next, transport) are bit-identical with grids
+ * on or off: the walk sees every daughter that could give the minimum or tie with it, and
+ * ties are broken by the same rule.  Steps and transport walk the grid of a node with at
+ * least 128 daughters and scan the daughters below that.  GV_FP32_REFINE walks it in
+ * binary32 with certified bounds: next is the same with grids on or off, step and safety
+ * within that precision's tolerance (a track certain on the walk may be refined without
+ * it, or the reverse).
  * enable != 0 turns the grids on (the default), 0 off;
  * takes effect for launches made after the call.  gv_geom_voxel_count returns the
  * number of nodes that have a grid. */

@@ -343,13 +343,6 @@ __device__ inline void bool_evaluate(const Desc& S, const Desc& A, const Desc& C
   else R.din = t;
 }
 
-__device__ __forceinline__ bool bool_ranked(const Desc& S, const Desc& A, const Desc& C, const Track& T, unsigned want, Result& R) {
-  uint32_t V;
-  if (!bool_verdict(S, A, C, T, want, V)) return false;
-  bool_evaluate(S, A, C, T, BoolVerdict{V}, R);
-  return true;
-}
-
 // Groups tracks whose binary64 work is alike: the distance (none, a plane's crossing, a wall's), whether
 // the second component's frame is needed, whether a safety needs a square root.
 constexpr uint32_t kBoolClasses = 12;

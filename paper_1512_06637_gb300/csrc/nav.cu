@@ -13,10 +13,11 @@
 // Locate descends from the world into the first daughter (in index order) that
 // does not classify the point as outside.
 //
-// Kernels: binary64, one thread per track, with the candidates ranked in certified binary32 and
-// only the deciding one evaluated in binary64 (the same bits); binary32, one thread per track
-// over scanned daughters (k_nav_scan32) or kLanes lanes per track along a grid (k_nav_fp32), whose
-// tracks with an ambiguous minimum or an uncertain daughter are recomputed by the binary64 step from
+// Kernels: binary64, a block-wide pool of tracks in phases (k_nav_pool), the candidates ranked in
+// certified binary32 and only the deciding one evaluated in binary64 (the same bits); binary32, one thread
+// per track over scanned daughters (k_nav_scan32) or kLanes lanes per track along a grid or in short baskets
+// (k_nav_fp32), whose tracks with an ambiguous minimum or an uncertain daughter are recomputed by the
+// binary64 step (k_nav_pool, short baskets k_nav_exact) from
 // a worklist.  World-to-node
 // transforms are composed on the host (binary64, no fused multiply-add) and
 // applied on the device with round-to-nearest operations in a fixed order, so the
@@ -203,11 +204,6 @@ struct NavArgs {
   int64_t n;
 };
 
-// DistanceToIn of the daughters of N (which has a grid) for the ray p + t d (world):
-// the cells the ray crosses are visited in t order and the walk stops once the best
-// candidate so far is before the next cell by more than 4e-9 (1 + best) mm.  Candidates
-// are ranked by (t, node index), the mother (who = -1) after every daughter; runner is the
-// next smaller candidate among those seen (daughters not seen are farther than the margin).
 // A 3-D DDA over the cells of a grid that a ray (node frame) crosses, in order of entry.
 struct Dda {
   int c[3], step[3];
@@ -1644,7 +1640,7 @@ __device__ __forceinline__ int32_t locate_rank32(const Geo& g, double x, double 
   return locate64_surf(g, x, y, z, surf);
 }
 
-// Locate with the codes ranked in binary32 first (the same nodes as k_locate).
+// gv_nav_locate: one thread per track, the codes in binary32 where they are certain.
 __global__ void __launch_bounds__(256, 2) k_locate32(Geo g, const double* __restrict__ x, const double* __restrict__ y,
                                                   const double* __restrict__ z, int32_t* __restrict__ out, int64_t n) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;

@@ -11,8 +11,9 @@
 
 namespace gv {
 
-// kCullBox, kCullTube: the plain safety is the solid's own; kCullOther: the bounding box only;
-// kCullNever: always evaluated (no binary32 form).
+// kCullBox, kCullTube: the plain safety is the solid's own, and the entry has an upper bound too;
+// kCullOther: the bounding box tells misses, plain_other (nav.cu) the safety within a wider margin;
+// kCullNever: the same, but what is left has no certified binary32 evaluation, only a binary64 one.
 enum : int32_t { kCullBox = 0, kCullTube = 1, kCullOther = 2, kCullNever = 3 };
 
 // Per node: the world frame's rotation and translation, half extents of the bounding box around the

@@ -1,8 +1,9 @@
 // query_fp64.cu -- the plain binary64 query pass.  Primitive solids take the ranked pass
-// (k_query_rank64): binary32 decides which constraint and which crossing give the results, binary64
-// evaluates those; booleans of solids with at most two z-planes likewise (k_query_bool_rank).  What has
-// no ranked form is evaluated whole, one thread per track: other booleans in index order
-// (k_query_fp64); solids with features finer than binary32 resolves in tiles ordered by work class when the basket gives every SM a 2048-track tile (k_query_fp64_tiles: the FP64 pipe
+// (k_query_rank64, k_query_rank64_short, k_rank_walk): binary32 decides which constraint and which
+// crossing give the results, binary64 evaluates those; larger baskets of booleans of solids with at most
+// two z-planes likewise (k_query_bool_rank).  The rest is evaluated whole, one thread per track: other and
+// short booleans in index order (k_query_fp64); solids with features finer than binary32 resolves in tiles
+// ordered by work class when the basket gives every SM a 2048-track tile (k_query_fp64_tiles: the FP64 pipe
 // spends the same on a warp instruction whatever its active lanes, so warps of one class run fewer
 // instructions), else in index order.  Per track the bits are the same in every one of them.
 #include "bool_rank.cuh"
@@ -148,17 +149,17 @@ static __device__ __noinline__ void query_open(const Desc& S, const QueryArgs& a
 // edges) goes on the block's list, which is evaluated when 256 have gathered and at the end: its code in
 // binary64, the rest ranked.
 // Measured (GB300, all five queries): cone, 2^20 tracks, 500 -> 179 us; 8-plane polycone, 4 M tracks,
-// 6876 -> 1274 us in this kernel alone; tube DistanceToOut, 50021 tracks, 44.6 -> 22.5 us (before: every
-// candidate in binary64, tiles ordered by class).  FP64 warp instructions per 32 tracks: cone 226 -> 42,
-// polycone 859 -> 45; issue 41% and FP64 46% busy (cone): bound by latency at 24 warps per SM.  Three
-// blocks of 256 threads (80 registers) against two (128): cone 179 against 186 us; one-row tiles (short
-// baskets) 24.0 against 22.5 us.
+// 6876 -> 1274 us in this kernel alone (before: every candidate in binary64, tiles ordered by class).
+// FP64 warp instructions per 32 tracks: cone 226 -> 42, polycone 859 -> 45; issue 41% and FP64 46% busy
+// (cone): bound by latency at 24 warps per SM.  Three blocks of 256 threads (80 registers) against two
+// (128): cone 179 against 186 us; rows of 256 the other way round.
 constexpr int kOpenFlush = 256;
 constexpr int kRankThreads = 256, kRankBlocks = 3;
 constexpr uint32_t kOpenVerdict = 0xFFFFFFFFu;
 // STORED: the verdicts are read from `stored`, where an earlier launch left them.
 template <int FAMILY, int ITEMS, bool STORED = false>
-__global__ void __launch_bounds__(kRankThreads, ITEMS == 1 ? 512 / kRankThreads : kRankBlocks) k_query_rank64(const Desc* __restrict__ desc, QueryArgs a, const uint2* stored) {
+__global__ void __launch_bounds__(kRankThreads, ITEMS == 1 ? 512 / kRankThreads : kRankBlocks)
+    k_query_rank64(const Desc* __restrict__ desc, QueryArgs a, const uint2* stored) {
   constexpr int NT = kRankThreads, TILE = NT * ITEMS;
   constexpr uint32_t NC = f64::kRankClasses;
   __shared__ Desc S;
@@ -341,7 +342,8 @@ __global__ void __launch_bounds__(256, 2) k_query_bool_rank(const Desc* __restri
 }
 
 // Baskets too short to fill the GPU: one track per thread, ranked and evaluated at once.  Latency bounds
-// them, and a tile's barriers and second loads only add to it.
+// them, and a tile's barriers and second loads only add to it.  Measured (tube DistanceToOut, 50021 tracks):
+// 44.6 us evaluating every candidate in binary64, 22.6 us here.
 constexpr int kShortThreads = 128;
 constexpr int64_t kRankWalkMin = 1 << 19;  // multi-section polycones: two launches from here on
 template <int FAMILY>
@@ -474,7 +476,8 @@ template <int FAMILY, int ITEMS>
 static void launch_rank64(const gv_solid* s, const QueryArgs& a, int sms, cudaStream_t stream) {
   static const int occ = [] {
     int o = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_query_rank64<FAMILY, ITEMS>, kRankThreads, 0) != cudaSuccess || o < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_query_rank64<FAMILY, ITEMS>, kRankThreads, 0) != cudaSuccess ||
+        o < 1) {
       cudaGetLastError();
       o = 1;
     }

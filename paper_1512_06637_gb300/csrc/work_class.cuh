@@ -1,5 +1,5 @@
 // work_class.cuh -- the work class of a track against a primitive solid, from the high parts
-// of its binary64 words: the key by which the binary64 pass orders a basket (k_sort_classes).
+// of its binary64 words: the key by which tiles evaluated whole in binary64 are ordered.
 #pragma once
 #include "solid_fp32.cuh"
 
