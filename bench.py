@@ -40,16 +40,16 @@ BYTES_PER_TRACK = 6 * 8 + 1 + 4 * 8  # SoA point + direction in, code + 4 double
 # launch are not counted, at most 129 MB); valid only while the kernel sources hash to the value
 # recorded with them, else the bench reports traffic = null.
 DRAM_CAPTURE = {
-    "sources_sha256": "76e9d0d63b2268d4487bf17bc51db7e11e496f00247adc8c5ffbb5284f2e4c3a",
-    "bytes_per_track": {'box': 71.89, 'trd': 72.45, 'tube': 73.43, 'cone': 73.60, 'polycone': 72.30},
+    "sources_sha256": "283f43c42b9f4170bfbef6b3926ecd8c3b5b55a817c7573f13819afaf5195ea5",
+    "bytes_per_track": {'box': 71.80, 'trd': 72.07, 'tube': 73.37, 'cone': 73.61, 'polycone': 72.39},
     "profile": "profiles/query_fp32_passes_4M_counters.md",
 }
 # Warp instructions per track of each binary32 pass (smsp__inst_executed.sum of one launch ÷
 # its tracks, from the same captures; the counts do not depend on the basket size), valid while
 # the kernel sources hash to the recorded value.
 ISSUE_CAPTURE = {
-    "sources_sha256": "76e9d0d63b2268d4487bf17bc51db7e11e496f00247adc8c5ffbb5284f2e4c3a",
-    "warp_inst_per_track": {'box': 18.61, 'trd': 34.34, 'tube': 62.04, 'cone': 57.16, 'polycone': 116.11},
+    "sources_sha256": "283f43c42b9f4170bfbef6b3926ecd8c3b5b55a817c7573f13819afaf5195ea5",
+    "warp_inst_per_track": {'box': 18.61, 'trd': 34.21, 'tube': 61.52, 'cone': 57.29, 'polycone': 116.29},
     "profile": "profiles/query_fp32_passes_4M_counters.md",
 }
 KERNEL_SOURCES = ("solid_fp32.cuh", "query_fp32.cu", "gv_desc.h")
@@ -57,9 +57,9 @@ KERNEL_SOURCES = ("solid_fp32.cuh", "query_fp32.cu", "gv_desc.h")
 # (sm__inst_executed_pipe_fp64.sum of one launch / its tracks), valid while the binary64 sources
 # hash to the recorded value.
 FP64_CAPTURE = {
-    "sources_sha256": "a07399a0b4f95abb2a949a3ac5e9237dcdb23b0aab450eaf2b66597fbf4d00c7",
-    "fp64_warp_inst_per_track": {'tube': 10.47, 'cone': 7.29},
-    "profile": "profiles/query_fp64_tube_cone_1M_pipe.md",
+    "sources_sha256": "f5e0a24a23e3ebde67886460e2fb342d7472e9a3c01a76c6c1034108b77ec989",
+    "fp64_warp_inst_per_track": {'tube': 1.274, 'cone': 1.301},
+    "profile": "profiles/ranked_binary64_tube_cone_1M_pipe.md",
 }
 FP64_KERNEL_SOURCES = ("solid_fp64.cuh", "rank_fp64.cuh", "solid_fp32.cuh", "query_fp64.cu", "gv_desc.h")
 E2E_CHUNK = 1 << 22  # tracks per host-streaming chunk (2^19-2^22 measured: larger is faster)
